@@ -556,6 +556,7 @@ int sketch_order_arena(skis_sketch* s, cudaStream_t st, std::string* err) {
             const unsigned long long cur = E0 + E1;
             CV_CUDA(cudaMemcpyAsync(&s->ctr->arena, &cur, sizeof(cur), cudaMemcpyHostToDevice, st));
         }
+        s->arena_used = E0 + E1;
         CV_CUDA(cudaStreamSynchronize(st));
         return SKIS_OK;
     };

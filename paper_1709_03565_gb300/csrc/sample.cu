@@ -34,8 +34,10 @@ constexpr int kQCap = 256;         // warp-tier member capacity
 constexpr int kHCap = 512;         // warp-tier hash slots (load <= 1/2 + one insert round)
 constexpr int kHashBits = 9;
 constexpr int kIdBatch = 16;       // sample ids taken per work-cursor atomic
-constexpr uint32_t kArenaChunk = 2048;        // entries reserved per arena atomic (warp tier)
-constexpr uint32_t kLaneArenaChunk = 512;     // entries reserved per arena atomic (lane tiers)
+// entries reserved per arena atomic; once a warp's reservation did not fit it
+// asks for no more than it needs, so that the arena cursor ends at the demand
+constexpr uint32_t kArenaChunk = 2048;        // warp tier
+constexpr uint32_t kLaneArenaChunk = 512;     // lane tiers
 constexpr int kCtaGroupLog2 = 2;
 constexpr int kCtaGroup = 1 << kCtaGroupLog2;  // edge quads of a long row a CTA-tier lane draws per step
 constexpr int kCtaLongRow = 64;            // quads that make a row long
@@ -479,6 +481,7 @@ __global__ void __launch_bounds__(kLaneBlock, 4) k_iis_lane(SampleArgs a) {
     uint2 prec = make_uint2(0, 0);
     uint64_t sig = 0;  // the sample's members, one hashed bit each (member_bit)
     uint64_t chunk_pos = 0, chunk_end = 0;
+    uint32_t chunk = kLaneArenaChunk;
 
     for (;;) {
         // ---- batched maintenance: write out finished samples, refill
@@ -497,12 +500,13 @@ __global__ void __launch_bounds__(kLaneBlock, 4) k_iis_lane(SampleArgs a) {
                 const uint32_t total = __shfl_sync(kFull, incl, 31);
                 bool fits = true;
                 if (chunk_end - chunk_pos < total) {
-                    const uint64_t size = max((uint64_t)kLaneArenaChunk, (uint64_t)total);
+                    const uint64_t size = max((uint64_t)chunk, (uint64_t)total);
                     unsigned long long base = 0;
                     if (lane == 0) base = atomicAdd(a.arena_cursor, (unsigned long long)size);
                     base = __shfl_sync(kFull, base, 0);
                     if (base + size > a.arena_cap) {
                         fits = false;
+                        chunk = 0;
                         chunk_pos = chunk_end = 0;
                     } else {
                         chunk_pos = base;
@@ -753,6 +757,7 @@ __global__ void __launch_bounds__(kWarpThreads) k_iis_warp(SampleArgs a) {
     uint32_t* hash = s_hash[wib];
     int32_t* queue = s_queue[wib];
     uint64_t chunk_pos = 0, chunk_end = 0;  // this warp's arena reservation
+    uint32_t chunk = kArenaChunk;
 
     const uint64_t count = input_count(a);
     for (;;) {
@@ -815,11 +820,12 @@ __global__ void __launch_bounds__(kWarpThreads) k_iis_warp(SampleArgs a) {
             // arena append from this warp's chunk
             const uint32_t len = ins.qlen;
             if (chunk_end - chunk_pos < len) {
-                const uint64_t size = max((uint64_t)kArenaChunk, (uint64_t)len);
+                const uint64_t size = max((uint64_t)chunk, (uint64_t)len);
                 unsigned long long base = 0;
                 if (lane == 0) base = atomicAdd(a.arena_cursor, (unsigned long long)size);
                 base = __shfl_sync(kFull, base, 0);
                 if (base + size > a.arena_cap) {
+                    chunk = 0;
                     chunk_pos = chunk_end = 0;
                     if (lane == 0) arena_overflow(a, j);
                     continue;
@@ -1256,6 +1262,7 @@ __global__ void __launch_bounds__(kLtBlock) k_lt_walk(SampleArgs a) {
     uint32_t v = 0, len = 0, t = 0;
     int32_t x = 0;
     uint64_t chunk_pos = 0, chunk_end = 0;
+    uint32_t chunk = kLaneArenaChunk;
 
     for (;;) {
         const unsigned idle = __ballot_sync(kFull, !busy);
@@ -1318,12 +1325,13 @@ __global__ void __launch_bounds__(kLtBlock) k_lt_walk(SampleArgs a) {
             const uint32_t total = __shfl_sync(kFull, incl, 31);
             bool fits = true;
             if (chunk_end - chunk_pos < total) {
-                const uint64_t size = max((uint64_t)kLaneArenaChunk, (uint64_t)total);
+                const uint64_t size = max((uint64_t)chunk, (uint64_t)total);
                 unsigned long long base = 0;
                 if (lane == 0) base = atomicAdd(a.arena_cursor, (unsigned long long)size);
                 base = __shfl_sync(kFull, base, 0);
                 if (base + size > a.arena_cap) {
                     fits = false;
+                    chunk = 0;
                     chunk_pos = chunk_end = 0;
                 } else {
                     chunk_pos = base;
@@ -1522,7 +1530,8 @@ static cudaError_t grow_copy(T** p, uint64_t old_n, uint64_t new_n, cudaStream_t
     return cudaSuccess;
 }
 
-static int ensure_sample_buffers(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* err) {
+// slack: arena entries that the tiers' warps may leave unused at the ends of their chunks
+static int ensure_sample_buffers(skis_sketch* s, uint64_t count, uint64_t slack, cudaStream_t st, std::string* err) {
     const skis_graph* g = s->g;
     if (!s->ctr) {
         SK_CUDA(dev_alloc_t(&s->ctr, 1, st));
@@ -1561,9 +1570,25 @@ static int ensure_sample_buffers(skis_sketch* s, uint64_t count, cudaStream_t st
         s->list_cap = count;
     }
     if (!s->arena) {
-        uint64_t cap = s->arena_hint ? s->arena_hint : std::max<uint64_t>(count * 8, 1u << 20);
+        // the default: room for samples of 128 members within 2 GiB, at least 8 a sample, and the
+        // ends of the warps' chunks. Sizes run from 4 members a sample (trivalency) to 60-75
+        // (weighted cascade, LT 18), and a pass that overflows draws what did not fit again
+        uint64_t cap = s->arena_hint;
+        if (!cap) cap = std::max<uint64_t>({count * 8, std::min<uint64_t>(count * 128, 1u << 29), 1u << 20}) + slack;
         SK_CUDA(dev_alloc_t(&s->arena, (size_t)cap, st));
         s->arena_cap = cap;
+    } else if (s->T > 0) {
+        // more samples like the ones so far: the arena grows before the pass
+        // when they would not fit (or, without the memory now, as it overflows)
+        const uint64_t used = std::min(s->arena_used, s->arena_cap);
+        const double mean = (double)used / (double)s->T;
+        const uint64_t want = used + (uint64_t)((double)count * mean * 1.125) + slack;
+        if (want > s->arena_cap) {
+            const cudaError_t e = grow_copy(&s->arena, used, std::max(want, s->arena_cap * 2), st);
+            if (e == cudaSuccess) s->arena_cap = std::max(want, s->arena_cap * 2);
+            else if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+            else SK_CUDA(e);
+        }
     }
     if (g->lt && !s->lt_hash) {  // medium LT walks: one table, list and slot record per lane
         s->lt_mid_lanes = (uint64_t)sm_count() * kLtMidBlock * 2;  // two blocks per SM
@@ -1630,15 +1655,24 @@ int sketch_sample(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* 
         return SKIS_EINVAL;
     }
     if (count == 0) return SKIS_OK;
-    int rc = ensure_sample_buffers(s, count, st, err);
-    if (rc != SKIS_OK) return rc;
     const bool thread_tier = s->thread_max_deg > 0;
-    int warp_blocks = 0, lane_blocks = 0;
-    rc = occupancy_grid((const void*)k_iis_lane, kLaneBlock, s->thread_blocks,
+    int warp_blocks = 0, lane_blocks = 0, lt_blocks = 0;
+    int rc = occupancy_grid((const void*)k_iis_lane, kLaneBlock, s->thread_blocks,
                         (count + kLaneBlock - 1) / kLaneBlock, err, &lane_blocks);
     if (rc != SKIS_OK) return rc;
     rc = occupancy_grid((const void*)k_iis_warp, kWarpThreads, s->warp_blocks,
                         thread_tier ? UINT64_MAX : (count + kIdBatch - 1) / kIdBatch, err, &warp_blocks);
+    if (rc != SKIS_OK) return rc;
+    if (g->lt) {
+        rc = occupancy_grid((const void*)k_lt_walk, kLtBlock, s->thread_blocks, (count + kLtBlock - 1) / kLtBlock,
+                            err, &lt_blocks);
+        if (rc != SKIS_OK) return rc;
+    }
+    // every warp's open chunk (a warp without a sample opens none)
+    const uint64_t slack =
+        (uint64_t)kLaneArenaChunk * std::min<uint64_t>(count, (uint64_t)(g->lt ? lt_blocks : lane_blocks) * (kLaneBlock / 32)) +
+        (g->lt ? 0 : (uint64_t)kArenaChunk * std::min<uint64_t>(count, (uint64_t)warp_blocks * (kWarpThreads / 32)));
+    rc = ensure_sample_buffers(s, count, slack, st, err);
     if (rc != SKIS_OK) return rc;
 
     SampleArgs base;
@@ -1701,13 +1735,6 @@ int sketch_sample(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* 
         if (rc != SKIS_OK) return rc;
         base.chain = g->chain;
     }
-    int lt_blocks = 0;
-    if (g->lt) {
-        rc = occupancy_grid((const void*)k_lt_walk, kLtBlock, s->thread_blocks, (count + kLtBlock - 1) / kLtBlock,
-                            err, &lt_blocks);
-        if (rc != SKIS_OK) return rc;
-    }
-
     DevStatus hst;
     SampleCounters hc;
     int pass = 0;
@@ -1824,11 +1851,11 @@ int sketch_sample(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* 
         if (hc.novf == 0) break;
         // some reservations did not fit: grow the arena (keeping every
         // completed sample, all of which lie below the old capacity) and
-        // rerun exactly the samples that failed
+        // rerun exactly the samples that failed. The cursor counted every
+        // reservation, placed or not, so what the rerun needs is known up to
+        // the ends of chunks that a next sample does not fit in
         const uint64_t old_cap = s->arena_cap;
-        const uint64_t new_cap = old_cap * 2 + (uint64_t)kLaneArenaChunk * lane_blocks * (kLaneBlock / 32) +
-                                 (uint64_t)kLaneArenaChunk * lt_blocks * (kLtBlock / 32) +
-                                 (uint64_t)kArenaChunk * warp_blocks * (kWarpThreads / 32);
+        const uint64_t new_cap = std::max<uint64_t>(old_cap * 2, hc.arena + hc.arena / 8) + slack;
         rc = [&]() -> int {
             SK_CUDA(grow_copy(&s->arena, old_cap, new_cap, st));
             return SKIS_OK;
@@ -1848,6 +1875,7 @@ int sketch_sample(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* 
         ++pass;
     }
     s->T += count;
+    s->arena_used = hc.arena;
     if (counting) {
         s->vcount_ok = true;
         s->vcount_T = s->T;

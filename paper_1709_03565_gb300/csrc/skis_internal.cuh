@@ -299,6 +299,7 @@ struct skis_sketch {
     int32_t* arena = nullptr;            // members, sample after sample (with gaps)
     uint64_t arena_cap = 0;
     uint64_t arena_hint = 0;
+    uint64_t arena_used = 0;             // the arena cursor after the last call
     skis::SampleCounters* ctr = nullptr;
     skis::DevStatus* status = nullptr;
     uint64_t* to_warp_ids = nullptr;     // thread tier -> warp tier
