@@ -116,12 +116,13 @@ typedef struct skis_stats {
  * (up to 32 members, in-rows up to THREAD_MAX_DEG edges, up to
  * THREAD_MAX_STEPS edge quads, up to THREAD_MAX_RETRIES rejected rounds;
  * the "thread" names below refer to this tier), one warp per sample (up to
- * 256 members, up to WARP_MAX_COINS in-edges), one CTA per sample (any size). Options tune the split; they
+ * 1536 members, the first 256 in shared memory; up to WARP_MAX_COINS
+ * in-edges), one CTA per sample (any size). Options tune the split; they
  * never change the samples. */
 typedef enum skis_option {
     SKIS_OPT_RETRY_CAP = 0,      /* cap on rejected first-step rounds (default 2^24) */
     SKIS_OPT_CTA_SLOTS = 1,      /* CTAs of the CTA tier (default: 1024 threads of them per SM) */
-    SKIS_OPT_WARP_BLOCKS = 2,    /* CTAs of the warp tier (default: full occupancy) */
+    SKIS_OPT_WARP_BLOCKS = 2,    /* CTAs of the warp tier (default, and at most, full occupancy) */
     SKIS_OPT_THREAD_MAX_DEG = 3, /* longest in-row the thread tier expands (default 192; 0 = tier off) */
     SKIS_OPT_THREAD_BLOCKS = 4,  /* CTAs of the thread tier (default: full occupancy) */
     SKIS_OPT_QUERY_INDEX = 5,    /* skis_estimate: 0 = walk the inverted index (vertex -> samples) when

@@ -560,6 +560,8 @@ void skis::sketch_release(skis_sketch* s) {
     dev_free(s->srcpick, st);
     dev_free(s->ovf_ids[0], st);
     dev_free(s->ovf_ids[1], st);
+    dev_free(s->spill_hash, st);
+    dev_free(s->spill_queue, st);
     dev_free(s->bitmaps, st);
     dev_free(s->queues, st);
     dev_free(s->big_queues, st);

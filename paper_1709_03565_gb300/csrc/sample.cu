@@ -11,9 +11,11 @@
 // by id to the warp tier.
 //
 // Warp tier: one warp per sample. The member list (256 entries) and an
-// open-addressing hash set (the visited set R_j) live in shared memory. Edges
-// of up to 32 queued vertices are spread over the lanes one edge quad at a
-// time. A sample that outgrows it is handed, by id, to the CTA tier.
+// open-addressing hash set (the visited set R_j) live in shared memory; a
+// larger sample moves to the warp's slot in global memory (up to 1536
+// members). Edges of up to 32 queued vertices are spread over the lanes one
+// edge quad at a time. A sample that outgrows it is handed, by id, to the CTA
+// tier.
 //
 // CTA tier: one block per sample with a global n-bit visited bitmap and an
 // n-entry global queue per block slot.
@@ -30,10 +32,15 @@
 namespace skis {
 
 constexpr int kWarpThreads = 256;  // 8 warps per block
-constexpr int kQCap = 256;         // warp-tier member capacity
-constexpr int kHCap = 512;         // warp-tier hash slots (load <= 1/2 + one insert round)
+constexpr int kQCap = 256;         // warp-tier members held in shared memory
 constexpr int kHashBits = 9;
-constexpr int kIdBatch = 16;       // sample ids taken per work-cursor atomic
+constexpr int kHCap = 1 << kHashBits;  // their hash slots (load <= 1/2 + one insert round)
+constexpr int kIdBatch = 16;       // most sample ids a warp takes per work-cursor atomic
+constexpr int kSpillCap = 1536;    // warp-tier members in all: past kQCap in the warp's global spill slot
+constexpr int kSpillHashBits = 12;
+constexpr int kSpillHash = 1 << kSpillHashBits;  // its hash slots (load under 2/5)
+constexpr int kRing = 64;          // queued members whose in-rows wait in shared memory
+constexpr int kPend = 32 + 128;    // live edges waiting for an insert round: under 32, plus one quad a lane
 // entries reserved per arena atomic; once a warp's reservation did not fit it
 // asks for no more than it needs, so that the arena cursor ends at the demand
 constexpr uint32_t kArenaChunk = 2048;        // warp tier
@@ -92,6 +99,9 @@ struct SampleArgs {
     const uint4* up_rec;
     const uint2* up_pick;
     uint64_t up_first, up_count;
+    // warp tier: a spill slot a warp, kSpillHash table words and kSpillCap members
+    uint32_t* spill_hash;
+    int32_t* spill_queue;
 };
 
 
@@ -182,34 +192,85 @@ __device__ __forceinline__ uint32_t source_of(const SampleArgs& a, uint64_t j, R
 }
 
 // ----------------------------------------------------------- inserters
-// Warp tier: shared-memory hash set + shared-memory member queue.
+// Warp tier: the members of the warp's sample (which are also its BFS queue)
+// and their hash set. Up to kQCap members live in shared memory; a larger
+// sample moves both to the warp's spill slot in global memory (L2) and goes
+// on there, up to kSpillCap members. A candidate's in-row is loaded while its
+// hash slot is probed, and kept in a shared ring if it joins within kRing
+// places of the queue's head, so that a pop finds the row without going
+// through the queue and the row table (a chain of two memory latencies per
+// BFS level).
 struct WarpInserter {
     uint32_t* hash;
     int32_t* queue;
-    uint32_t qlen;
+    uint4* ring;      // (offset, degree, threshold, queue position) of queued members
+    uint32_t* ghash;  // the spill slot
+    int32_t* gqueue;
+    const RowInfo* rows;
+    uint32_t qlen, head;
+    bool big;         // the sample lives in the spill slot
     bool overflow;
+
+    // u joins table h (mask + 1 slots); false if it is there already
+    static __device__ __forceinline__ bool put(uint32_t* table, uint32_t h, uint32_t mask, uint32_t u) {
+        for (;;) {
+            const uint32_t old = atomicCAS(&table[h], kEmpty, u);
+            if (old == kEmpty) return true;
+            if (old == u) return false;
+            h = (h + 1) & mask;
+        }
+    }
+
+    __device__ __forceinline__ bool put_shared(uint32_t u) {
+        return put(hash, (u * 2654435761u) >> (32 - kHashBits), kHCap - 1, u);
+    }
+    __device__ __forceinline__ bool put_spill(uint32_t u) {
+        return put(ghash, (u * 2654435761u) >> (32 - kSpillHashBits), kSpillHash - 1, u);
+    }
+
+    // The sample outgrew shared memory: its members (qlen of them, and the
+    // lanes' fresh ones) go to the spill slot, whose table is cleared first.
+    __device__ __forceinline__ void spill(int32_t u, bool fresh) {
+        const int lane = threadIdx.x & 31;
+        for (int i = lane; i < kSpillHash / 4; i += 32)
+            reinterpret_cast<uint4*>(ghash)[i] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+        __syncwarp();
+        for (uint32_t i = lane; i < qlen; i += 32) {
+            const int32_t w = queue[i];
+            gqueue[i] = w;
+            put_spill((uint32_t)w);
+        }
+        if (fresh) put_spill((uint32_t)u);
+        big = true;
+        __syncwarp();
+    }
 
     __device__ __forceinline__ void insert(int32_t u) {
         if (overflow) return;  // warp-uniform
         bool fresh = false;
+        uint4 rw = make_uint4(0, 0, 0, 0);  // the row record's words: offset (low, high), degree, threshold
         if (u >= 0) {
-            uint32_t h = ((uint32_t)u * 2654435761u) >> (32 - kHashBits);
-            for (;;) {
-                const uint32_t old = atomicCAS(&hash[h], kEmpty, (uint32_t)u);
-                if (old == kEmpty) { fresh = true; break; }
-                if (old == (uint32_t)u) break;
-                h = (h + 1) & (kHCap - 1);
-            }
+            rw = __ldg(reinterpret_cast<const uint4*>(rows) + u);  // in flight while the table is probed
+            fresh = big ? put_spill((uint32_t)u) : put_shared((uint32_t)u);
         }
         const unsigned m = __ballot_sync(kFull, fresh);
         if (m) {
             const uint32_t pos = qlen + __popc(m & lanemask_lt());
-            if (fresh && pos < (uint32_t)kQCap) queue[pos] = u;
-            qlen += __popc(m);
-            if (qlen > (uint32_t)kQCap) overflow = true;
+            const uint32_t len = qlen + __popc(m);
+            if (len > (uint32_t)kQCap && !big) spill(u, fresh);
+            if (len > (uint32_t)kSpillCap) {
+                overflow = true;
+            } else if (fresh) {
+                if (big) gqueue[pos] = u;
+                else queue[pos] = u;
+                if (pos - head < (uint32_t)kRing) ring[pos & (kRing - 1)] = make_uint4(rw.x, rw.z, rw.w, pos);
+            }
+            qlen = len;
         }
         __syncwarp();
     }
+
+    __device__ __forceinline__ int32_t member(uint32_t i) const { return big ? gqueue[i] : queue[i]; }
 };
 
 // CTA tier, one lane alone (divergent code): test-and-set in the global
@@ -750,43 +811,165 @@ __global__ void __launch_bounds__(kLaneBlock, 4) k_iis_lane(SampleArgs a) {
 }
 
 // ------------------------------------------------------------- warp tier
-__global__ void __launch_bounds__(kWarpThreads) k_iis_warp(SampleArgs a) {
+// One warp per sample. Up to 32 queued rows are taken at a time and their
+// edge quads laid end to end over the lanes, two a lane and step: the row of
+// quad g is the number of rows that start at or before it, a popcount of the
+// step's row starts (one OR-reduction of the rows' start bits). Live edges
+// are only listed (their positions, in shared memory) and joined 32 at a time,
+// one a lane, so that the source gather, the probe and the row load of 32
+// candidates overlap and an insert round has every lane busy.
+// Two thirds of a weighted-cascade sketch's members lie in samples of more
+// than 256 members, so the tier goes on past shared memory: the spill slots
+// of 1536 members keep all but 1 in 130 samples of Chung-Lu 1M / 17.5M off
+// the CTA tier, which pays block barriers on every narrow level (100 us and
+// more a sample). On 1M samples of that graph this tier and the CTA tier
+// took 29 ms when samples left here at 256 members and 13.5 ms now.
+__global__ void __launch_bounds__(kWarpThreads, 4) k_iis_warp(SampleArgs a) {
     __shared__ __align__(16) uint32_t s_hash[kWarpThreads / 32][kHCap];
     __shared__ __align__(16) int32_t s_queue[kWarpThreads / 32][kQCap];
+    __shared__ uint4 s_ring[kWarpThreads / 32][kRing];
+    __shared__ uint4 s_row[kWarpThreads / 32][32];  // the batch's rows: quads before it, first and end edge, threshold
+    __shared__ uint32_t s_pend[kWarpThreads / 32][kPend];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    uint32_t* hash = s_hash[wib];
-    int32_t* queue = s_queue[wib];
+    const uint64_t wid = (uint64_t)blockIdx.x * (kWarpThreads / 32) + wib;
+    uint32_t* const hash = s_hash[wib];
+    uint4* const row = s_row[wib];
+    uint32_t* const pend = s_pend[wib];
+    const uint4* __restrict__ tau4 = reinterpret_cast<const uint4*>(a.tau);
     uint64_t chunk_pos = 0, chunk_end = 0;  // this warp's arena reservation
     uint32_t chunk = kArenaChunk;
 
     const uint64_t count = input_count(a);
+    // ids per cursor atomic: one where samples are few, so that every warp has
+    // some (their costs differ a thousandfold), up to kIdBatch where they are many
+    const uint64_t nwarps = (uint64_t)gridDim.x * (kWarpThreads / 32);
+    const uint64_t batch = max((uint64_t)1, min((uint64_t)kIdBatch, count / (8 * nwarps)));
     for (;;) {
         unsigned long long t0 = 0;
-        if (lane == 0) t0 = atomicAdd(a.work, (unsigned long long)kIdBatch);
+        if (lane == 0) t0 = atomicAdd(a.work, (unsigned long long)batch);
         t0 = __shfl_sync(kFull, t0, 0);
         if (t0 >= count) break;
-        const uint64_t t1 = min((uint64_t)t0 + kIdBatch, count);
+        const uint64_t t1 = min((uint64_t)t0 + batch, count);
         for (uint64_t t = t0; t < t1; ++t) {
             const uint64_t j = input_id(a, t);
-            // clear the visited set
+            // clear the visited set and the ring
 #pragma unroll
             for (int i = lane; i < kHCap / 4; i += 32)
                 reinterpret_cast<uint4*>(hash)[i] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+#pragma unroll
+            for (int i = lane; i < kRing; i += 32) s_ring[wib][i].w = kEmpty;
             __syncwarp();
 
-            // Alg. 1: the source
+            // Alg. 1: the source, alone in the sample
             RowInfo rv;
             int64_t pe;
             int32_t pu;
             const uint32_t v = source_of(a, j, &rv, &pe, &pu);
-            WarpInserter ins{hash, queue, 0u, false};
-            ins.insert(lane == 0 ? (int32_t)v : -1);
+            WarpInserter ins{hash, s_queue[wib], s_ring[wib], a.spill_hash + wid * kSpillHash,
+                             a.spill_queue + wid * kSpillCap, a.rows, 1u, 1u, false, false};
+            if (lane == 0) {
+                ins.put_shared(v);
+                s_queue[wib][0] = (int32_t)v;
+            }
+            __syncwarp();
 
-            // the conditioned first step by rejection: all in-edge coins of v, round r
+            uint32_t npend = 0;
+            // the sources of the last cnt listed edges join the sample, one a lane
+            auto join = [&](uint32_t cnt) {
+                __syncwarp();
+                npend -= cnt;
+                const int32_t u = (uint32_t)lane < cnt ? __ldg(a.src + pend[npend + lane]) : -1;
+                ins.insert(u);
+            };
+            // the live edges (bit k: edge 4 q + k) of every lane join the list
+            auto list = [&](uint32_t q, unsigned live) {
+                if (!__any_sync(kFull, live != 0u)) return;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const unsigned m = __ballot_sync(kFull, (live >> k) & 1u);
+                    if ((live >> k) & 1u) pend[npend + __popc(m & lanemask_lt())] = 4u * q + (uint32_t)k;
+                    npend += __popc(m);
+                }
+#pragma unroll 1
+                while (npend >= 32u) join(32u);
+            };
+            // live mask of quad q (block x, thresholds t) within its row's edges [lo, hi)
+            auto coins4 = [](uint32_t q, const uint4& x, const uint4& t, uint32_t lo, uint32_t hi) -> unsigned {
+                const uint32_t e0 = q << 2;
+                const unsigned live = (coin_live(x.x, t.x) ? 1u : 0u) | (coin_live(x.y, t.y) ? 2u : 0u) |
+                                      (coin_live(x.z, t.z) ? 4u : 0u) | (coin_live(x.w, t.w) ? 8u : 0u);
+                const uint32_t before = e0 < lo ? lo - e0 : 0u, after = e0 + 4 > hi ? e0 + 4 - hi : 0u;
+                return live & (15u << before) & (15u >> after);
+            };
+            // the FIRST coins of round r on the source's in-edges [lo, hi); whether one is live
+            auto first_row = [&](uint32_t lo, uint32_t hi, uint32_t r) -> bool {
+                if (hi <= lo) return false;
+                const uint32_t qe = ((hi - 1) >> 2) + 1;
+                bool any = false;
+#pragma unroll 1
+                for (uint32_t qb = lo >> 2; qb < qe && !ins.overflow; qb += 32) {
+                    const uint32_t q = qb + lane;
+                    unsigned live = 0;
+                    if (q < qe) {
+                        const uint4 x = coin_block(a.rk, q, r, kDomFirst, j);
+                        const uint4 t4 = tau4 ? __ldg(tau4 + q) : make_uint4(rv.tau, rv.tau, rv.tau, rv.tau);
+                        live = coins4(q, x, t4, lo, hi);
+                    }
+                    any |= live != 0u;
+                    list(q, live);
+                }
+                return __any_sync(kFull, any);
+            };
+
+            // the conditioned first step (first_step_warp's cases): the bucket
+            // form's pick and the coins after it, RIS's one round, or the
+            // accepted round r of the rejection form
+            const uint32_t s_lo = (uint32_t)rv.off, s_hi = s_lo + rv.deg;
+            uint32_t r = 0, from = s_lo;
             bool failed = false;
-            const uint32_t r = first_step_warp(a, j, rv, ins, &failed, pe, pu);
+            if (a.chain) {
+                uint32_t e = 0;
+                if (lane == 0) {
+                    e = pe >= 0 ? (uint32_t)pe : (uint32_t)bucket_pick(a, j, rv.off, rv.deg);
+                    pend[0] = e;
+                }
+                npend = 1;
+                from = __shfl_sync(kFull, e, 0) + 1;
+            } else if (!a.ris) {
+                const uint32_t nq = ((s_hi - 1) >> 2) - (s_lo >> 2) + 1;
+                if (nq <= 16) {
+                    // a short row, 32 / nq rounds a pass: lane g draws quad g % nq of round
+                    // r + g / nq; the first lane with a live coin is in the accepted round
+                    const uint32_t rounds = 32u / nq, ri = (uint32_t)lane / nq;
+                    const uint32_t q = (s_lo >> 2) + (uint32_t)lane % nq;
+                    const uint4 t4 = tau4 ? __ldg(tau4 + q) : make_uint4(rv.tau, rv.tau, rv.tau, rv.tau);
+                    for (;; r += rounds) {
+                        if (r >= a.retry_cap) {
+                            failed = true;
+                            r = a.retry_cap;
+                            break;
+                        }
+                        unsigned live = 0;
+                        if (ri < rounds && r + ri < a.retry_cap)
+                            live = coins4(q, coin_block(a.rk, q, r + ri, kDomFirst, j), t4, s_lo, s_hi);
+                        const unsigned bal = __ballot_sync(kFull, live != 0u);
+                        if (bal) {
+                            r += (uint32_t)(__ffs(bal) - 1) / nq;
+                            break;
+                        }
+                    }
+                }
+            }
+            if (!failed)
+                while (!first_row(from, s_hi, r) && !a.chain && !a.ris) {  // at once for a short row's accepted round
+                    if (++r >= a.retry_cap) {
+                        failed = true;
+                        break;
+                    }
+                }
             if (failed) {
                 if (lane == 0) record_retry_failure(a, j, v, r, rv.deg);
+                __syncwarp();
                 continue;
             }
 
@@ -794,25 +977,82 @@ __global__ void __launch_bounds__(kWarpThreads) k_iis_warp(SampleArgs a) {
             uint64_t coins = lane == 0 ? (uint64_t)rv.deg * (r + 1) : 0;
             uint64_t drawn = 0;  // in-edges of the rows taken so far (warp-uniform)
             bool heavy = false;
-            uint32_t head = 1;
-            while (head < ins.qlen && !ins.overflow) {
-                const uint32_t cnt = min(ins.qlen - head, 32u);
-                RowInfo rw;
-                rw.off = 0; rw.deg = 0; rw.tau = 0;
-                if ((uint32_t)lane < cnt) rw = a.rows[queue[head + lane]];
+            const SampleBlock blk(a.rk, j, kDomBfs);
+            for (;;) {
+                if (ins.head >= ins.qlen && npend) join(npend);  // the level's last live edges (under 32)
+                if (ins.head >= ins.qlen || ins.overflow) break;
+                const uint32_t cnt = min(ins.qlen - ins.head, 32u);
+                uint32_t lo = 0, deg = 0, tau_row = 0;
+                if ((uint32_t)lane < cnt) {
+                    const uint32_t pos = ins.head + lane;
+                    const uint4 c = s_ring[wib][pos & (kRing - 1)];
+                    if (c.w == pos) {
+                        lo = c.x;
+                        deg = c.y;
+                        tau_row = c.z;
+                    } else {  // it joined too far from the head for the ring
+                        const RowInfo rw = a.rows[ins.member(pos)];
+                        lo = (uint32_t)rw.off;
+                        deg = rw.deg;
+                        tau_row = rw.tau;
+                    }
+                }
+                ins.head += cnt;
                 // a sample that reaches huge in-rows goes to the CTA tier,
                 // where every warp of a block shares its rows
-                drawn += __reduce_add_sync(kFull, min(rw.deg, 1u << 26));
+                drawn += __reduce_add_sync(kFull, min(deg, 1u << 26));
                 if (drawn > a.warp_max_coins) {
                     heavy = true;
                     break;
                 }
-                coins += rw.deg;
-                expand_rows(a, j, kDomBfs, 0, rw.off, rw.deg, rw.tau, ins);
-                head += cnt;
+                coins += deg;
+                const uint32_t hi = lo + deg;
+                const uint32_t nq = deg ? ((hi - 1) >> 2) - (lo >> 2) + 1 : 0u;
+                uint32_t incl = nq;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint32_t y = __shfl_up_sync(kFull, incl, d);
+                    if (lane >= d) incl += y;
+                }
+                const uint32_t total = __shfl_sync(kFull, incl, 31), excl = incl - nq;
+                const unsigned rowm = __ballot_sync(kFull, nq > 0);
+                if (nq) row[__popc(rowm & lanemask_lt())] = make_uint4(excl, lo, hi, tau_row);
+                __syncwarp();
+                uint32_t started = 0;  // rows that start before this step's quads
+#pragma unroll 1
+                for (uint32_t base = 0; base < total && !ins.overflow; base += 64) {
+                    const uint32_t g0 = base + lane, g1 = g0 + 32;
+                    const uint32_t d0 = excl - base, d1 = d0 - 32;
+                    const unsigned m0 = __reduce_or_sync(kFull, nq && d0 < 32u ? 1u << d0 : 0u);
+                    const unsigned m1 = __reduce_or_sync(kFull, nq && d1 < 32u ? 1u << d1 : 0u);
+                    const unsigned le = lanemask_lt() | (1u << lane);
+                    const uint32_t i0 = started + __popc(m0 & le) - 1;
+                    started += __popc(m0);
+                    const uint32_t i1 = started + __popc(m1 & le) - 1;
+                    started += __popc(m1);
+                    // lanes past the batch's end take its last quad (i0 and i1
+                    // then name the last row) and drop its coins
+                    const uint4 r0 = row[i0], r1 = row[i1];
+                    const uint32_t q0 = (r0.y >> 2) + (min(g0, total - 1) - r0.x);
+                    const uint32_t q1 = (r1.y >> 2) + (min(g1, total - 1) - r1.x);
+                    const bool two = base + 32 < total;  // warp-uniform
+                    const uint4 t0v = tau4 ? __ldg(tau4 + q0) : make_uint4(r0.w, r0.w, r0.w, r0.w);
+                    unsigned l0 = 0, l1 = 0;
+                    if (two) {  // two independent blocks
+                        const uint4 t1v = tau4 ? __ldg(tau4 + q1) : make_uint4(r1.w, r1.w, r1.w, r1.w);
+                        const uint4 x0 = blk(q0, a.rk), x1 = blk(q1, a.rk);
+                        l0 = coins4(q0, x0, t0v, r0.y, r0.z);
+                        if (g1 < total) l1 = coins4(q1, x1, t1v, r1.y, r1.z);
+                    } else if (g0 < total) {
+                        l0 = coins4(q0, blk(q0, a.rk), t0v, r0.y, r0.z);
+                    }
+#pragma unroll 1
+                    for (int h = 0; h < (two ? 2 : 1); ++h) list(h ? q1 : q0, h ? l1 : l0);
+                }
             }
-            if (ins.overflow || heavy) {  // too large for shared memory or too many coins: CTA tier
+            if (ins.overflow || heavy) {  // more members or coins than the tier takes: CTA tier
                 if (lane == 0) hand_on(a, j);
+                __syncwarp();
                 continue;
             }
             coins = warp_sum_u64(coins);
@@ -834,8 +1074,9 @@ __global__ void __launch_bounds__(kWarpThreads) k_iis_warp(SampleArgs a) {
                 chunk_end = base + size;
             }
             for (uint32_t i = lane; i < len; i += 32) {
-                a.arena[chunk_pos + i] = queue[i];
-                count_member(a, queue[i]);
+                const int32_t u = ins.member(i);
+                a.arena[chunk_pos + i] = u;
+                count_member(a, u);
             }
             if (lane == 0) {
                 a.h_off[j - a.id_base] = chunk_pos;
@@ -1530,8 +1771,10 @@ static cudaError_t grow_copy(T** p, uint64_t old_n, uint64_t new_n, cudaStream_t
     return cudaSuccess;
 }
 
-// slack: arena entries that the tiers' warps may leave unused at the ends of their chunks
-static int ensure_sample_buffers(skis_sketch* s, uint64_t count, uint64_t slack, cudaStream_t st, std::string* err) {
+// slack: arena entries that the tiers' warps may leave unused at the ends of their chunks;
+// warps: the warp tier's warps (0: no such tier)
+static int ensure_sample_buffers(skis_sketch* s, uint64_t count, uint64_t slack, uint64_t warps, cudaStream_t st,
+                                 std::string* err) {
     const skis_graph* g = s->g;
     if (!s->ctr) {
         SK_CUDA(dev_alloc_t(&s->ctr, 1, st));
@@ -1597,6 +1840,16 @@ static int ensure_sample_buffers(skis_sketch* s, uint64_t count, uint64_t slack,
         SK_CUDA(dev_alloc_t(&s->lt_list, (size_t)(s->lt_mid_lanes * kLtMidCap), st));
         SK_CUDA(dev_alloc_t(&s->lt_slot, (size_t)(s->lt_mid_lanes * kLtMidCap), st));
     }
+    if (warps > s->spill_warps) {  // warp tier: a spill slot a warp
+        dev_free(s->spill_hash, st);
+        dev_free(s->spill_queue, st);
+        s->spill_hash = nullptr;
+        s->spill_queue = nullptr;
+        s->spill_warps = 0;
+        SK_CUDA(dev_alloc_t(&s->spill_hash, (size_t)(warps * kSpillHash), st));
+        SK_CUDA(dev_alloc_t(&s->spill_queue, (size_t)(warps * kSpillCap), st));
+        s->spill_warps = warps;
+    }
     // CTA-tier slots: an n-bit visited bitmap and a queue of min(n, cta_queue_cap)
     // entries each (a sample with more members moves to a pass over slots with
     // n-entry queues), 1024 threads of blocks per SM within ~8 GB
@@ -1660,19 +1913,23 @@ int sketch_sample(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* 
     int rc = occupancy_grid((const void*)k_iis_lane, kLaneBlock, s->thread_blocks,
                         (count + kLaneBlock - 1) / kLaneBlock, err, &lane_blocks);
     if (rc != SKIS_OK) return rc;
-    rc = occupancy_grid((const void*)k_iis_warp, kWarpThreads, s->warp_blocks,
-                        thread_tier ? UINT64_MAX : (count + kIdBatch - 1) / kIdBatch, err, &warp_blocks);
+    // no more blocks than can be resident (every warp holds a spill slot) and
+    // no more warps than samples
+    rc = occupancy_grid((const void*)k_iis_warp, kWarpThreads, 0,
+                        (count + kWarpThreads / 32 - 1) / (kWarpThreads / 32), err, &warp_blocks);
     if (rc != SKIS_OK) return rc;
+    if (s->warp_blocks > 0) warp_blocks = std::min(warp_blocks, s->warp_blocks);
     if (g->lt) {
         rc = occupancy_grid((const void*)k_lt_walk, kLtBlock, s->thread_blocks, (count + kLtBlock - 1) / kLtBlock,
                             err, &lt_blocks);
         if (rc != SKIS_OK) return rc;
     }
     // every warp's open chunk (a warp without a sample opens none)
-    const uint64_t slack =
-        (uint64_t)kLaneArenaChunk * std::min<uint64_t>(count, (uint64_t)(g->lt ? lt_blocks : lane_blocks) * (kLaneBlock / 32)) +
-        (g->lt ? 0 : (uint64_t)kArenaChunk * std::min<uint64_t>(count, (uint64_t)warp_blocks * (kWarpThreads / 32)));
-    rc = ensure_sample_buffers(s, count, slack, st, err);
+    const uint64_t lane_warps = (uint64_t)(g->lt ? lt_blocks : lane_blocks) * (kLaneBlock / 32);
+    const uint64_t warps = g->lt ? 0 : (uint64_t)warp_blocks * (kWarpThreads / 32);
+    static_assert(kLaneBlock == kLtBlock, "one block size for both lane tiers");
+    const uint64_t slack = kLaneArenaChunk * std::min(count, lane_warps) + kArenaChunk * std::min(count, warps);
+    rc = ensure_sample_buffers(s, count, slack, warps, st, err);
     if (rc != SKIS_OK) return rc;
 
     SampleArgs base;
@@ -1717,6 +1974,8 @@ int sketch_sample(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* 
     base.up_first = 0;
     base.up_count = 0;
     base.lt_cum = g->lt_cum;
+    base.spill_hash = s->spill_hash;
+    base.spill_queue = s->spill_queue;
     // per-vertex member counts, kept while they describe exactly samples
     // [0, T): invalid until this call succeeds
     const bool counting = s->vcount_ok && s->vcount_T == s->T;

@@ -308,6 +308,9 @@ struct skis_sketch {
     uint4* srcrec = nullptr;             // lane tier: prepared source records
     uint2* srcpick = nullptr;            // lane tier, bucket form: prepared first-step picks
     uint64_t list_cap = 0;
+    uint32_t* spill_hash = nullptr;      // warp tier: visited table and members of each warp's
+    int32_t* spill_queue = nullptr;      // samples past the shared-memory ones
+    uint64_t spill_warps = 0;
     uint32_t* bitmaps = nullptr;         // CTA tier: one n-bit visited bitmap per slot
     int32_t* queues = nullptr;           // CTA tier: one queue_cap-entry queue per slot
     uint32_t queue_cap = 0;              // entries of each slot's queue: min(n, cta_queue_cap)

@@ -1,0 +1,64 @@
+"""Samples whose sizes and shapes sit at the edges of the deeper sampling tiers: every edge is live, so a sample is its
+source's ancestor set and its size is known. The warp tier keeps 256 members in shared memory and 1536 in all, batches
+32 rows and joins 32 live edges at a time; the CTA tier holds 512 rows of a level in shared memory. All against the
+oracle, sample by sample (integers and sets: equal)."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_1709_03565_gb300 as skis
+from test_gpu_parity import assert_samples_equal
+
+pytestmark = pytest.mark.gpu
+
+
+def _star(n):  # one row of n - 1 in-edges
+    return np.arange(1, n), np.zeros(n - 1)
+
+
+def _path(n):  # n - 1 levels of one row each; sources at every depth, so samples of every size up to n
+    return np.arange(1, n), np.arange(n - 1)
+
+
+def _tree(n):  # levels of 1, 2, 4, ... rows of two edges
+    i = np.arange(1, n)
+    return i, (i - 1) // 2
+
+
+def _broom(n):  # a level of (n - 1) / 2 rows of one edge each
+    h = (n - 1) // 2
+    mid = np.arange(1, h + 1)
+    return np.concatenate([mid, mid + h]), np.concatenate([np.zeros(h), mid])
+
+
+SHAPES = {"star": _star, "path": _path, "tree": _tree, "broom": _broom}
+TIERS = {"default": {}, "warp": {skis.SKIS_OPT_THREAD_MAX_DEG: 0},
+         "cta": {skis.SKIS_OPT_THREAD_MAX_DEG: 0, skis.SKIS_OPT_WARP_MAX_COINS: 1},
+         "cta-hub": {skis.SKIS_OPT_THREAD_MAX_DEG: 0, skis.SKIS_OPT_WARP_MAX_COINS: 1, skis.SKIS_OPT_CTA_HUB_QUADS: 2,
+                     skis.SKIS_OPT_CTA_THREADS: 512}}
+
+
+@pytest.mark.parametrize("tier", sorted(TIERS))
+@pytest.mark.parametrize("shape,n", [("star", 33), ("star", 257), ("star", 258), ("star", 1536), ("star", 1537),
+                                     ("path", 300), ("path", 1600), ("tree", 256), ("tree", 1537), ("broom", 1027),
+                                     ("broom", 2501)])
+@pytest.mark.parametrize("bucket", [False, True])
+def test_sizes_at_the_tiers_edges(shape, n, tier, bucket):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    src, dst = (np.ascontiguousarray(x, dtype=np.int32) for x in SHAPES[shape](n))
+    tau = np.full(len(src), 0xFFFFFFFF, np.uint32)
+    g = skis.skis_load_graph(n, src, dst, tau, skis.SKIS_W_EXPLICIT_TAU)
+    o = oracle.OracleGraph(n, src, dst, weights=tau, model=oracle.W_TAU)
+    T, seed = 2000, 0xED6E + n
+    s = skis.skis_sketch_create(g, seed)
+    skis.skis_sketch_set_option(s, skis.SKIS_OPT_FIRST_STEP, 1 if bucket else 0)
+    for k, v in TIERS[tier].items():
+        skis.skis_sketch_set_option(s, k, v)
+    skis.skis_sample(s, T)
+    ora = o.sample_ids(seed, np.arange(T, dtype=np.uint64), bucket=bucket)
+    assert shape not in ("star", "path") or ora["len"].max() >= n - 4  # a sample of (nearly) all vertices is among them
+    assert_samples_equal(skis.skis_sketch_export(s, 0, T), ora)
+    s.close()
+    g.close()
