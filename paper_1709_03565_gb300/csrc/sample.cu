@@ -45,9 +45,6 @@ constexpr int kPend = 32 + 128;    // live edges waiting for an insert round: un
 // asks for no more than it needs, so that the arena cursor ends at the demand
 constexpr uint32_t kArenaChunk = 2048;        // warp tier
 constexpr uint32_t kLaneArenaChunk = 512;     // lane tiers
-constexpr int kCtaGroupLog2 = 2;
-constexpr int kCtaGroup = 1 << kCtaGroupLog2;  // edge quads of a long row a CTA-tier lane draws per step
-constexpr int kCtaLongRow = 64;            // quads that make a row long
 constexpr uint32_t kEmpty = 0xFFFFFFFFu;
 
 struct SampleArgs {
@@ -273,190 +270,126 @@ struct WarpInserter {
     __device__ __forceinline__ int32_t member(uint32_t i) const { return big ? gqueue[i] : queue[i]; }
 };
 
-// CTA tier, one lane alone (divergent code): test-and-set in the global
-// bitmap, append to the global queue through the shared counter. A vertex
-// past the queue's capacity gets its bit back, so that the bitmap always
-// holds exactly the queued vertices (the counter still counts it: the sample
-// is then known to have outgrown the slot).
-__device__ __forceinline__ void cta_insert_one(uint32_t* bitmap, int32_t* queue, uint32_t* qlen, uint32_t cap,
-                                               int32_t u) {
-    const uint32_t bit = 1u << (u & 31);
-    if ((atomicOr(&bitmap[u >> 5], bit) & bit) == 0) {
-        const uint32_t pos = atomicAdd(qlen, 1u);
-        if (pos < cap) queue[pos] = u;
-        else atomicAnd(&bitmap[u >> 5], ~bit);
-    }
+__device__ __forceinline__ uint32_t min4(const uint4& x) { return min(min(x.x, x.y), min(x.z, x.w)); }
+
+__device__ __forceinline__ uint32_t min8(const uint4& x, const uint4& y) {
+    return __vimin3_u32(__vimin3_u32(x.x, x.y, x.z), __vimin3_u32(x.w, y.x, y.y), min(y.z, y.w));
 }
 
-// CTA tier: global bitmap (test-and-set) + global queue with a shared counter.
-struct CtaInserter {
-    uint32_t* bitmap;
-    int32_t* queue;
-    uint32_t* qlen;  // shared
-    uint32_t cap;    // queue capacity (see cta_insert_one)
-    bool overflow;   // never set: the CTA tier checks the count between levels
+// Live mask of edge quad q (block x, thresholds t; bit k: edge 4 q + k) within
+// its row's edges [lo, hi).
+__device__ __forceinline__ unsigned quad_live(uint32_t q, const uint4& x, const uint4& t, uint32_t lo, uint32_t hi) {
+    const uint32_t e0 = q << 2;
+    const unsigned live = (coin_live(x.x, t.x) ? 1u : 0u) | (coin_live(x.y, t.y) ? 2u : 0u) |
+                          (coin_live(x.z, t.z) ? 4u : 0u) | (coin_live(x.w, t.w) ? 8u : 0u);
+    const uint32_t before = e0 < lo ? lo - e0 : 0u, after = e0 + 4 > hi ? e0 + 4 - hi : 0u;
+    return live & (15u << before) & (15u >> after);
+}
 
-    __device__ __forceinline__ void insert(int32_t u) {
-        bool fresh = false;
-        if (u >= 0) {
-            const uint32_t bit = 1u << (u & 31);
-            fresh = (atomicOr(&bitmap[u >> 5], bit) & bit) == 0;
+__device__ __forceinline__ uint32_t row_quads(uint32_t lo, uint32_t hi) {
+    return hi > lo ? ((hi - 1) >> 2) - (lo >> 2) + 1 : 0u;
+}
+
+// The rejection form's accepted round for a source row of 1 to 16 edge quads,
+// by one warp: rounds are independent given (j, r), so 32 / nq of them are
+// drawn a pass, lane g taking quad g % nq of round r + g / nq, and the first
+// lane with a live coin is in the accepted round, as in sequential order.
+// Returns the cap when no round below it is accepted.
+__device__ __forceinline__ uint32_t accepted_round(const SampleArgs& a, uint64_t j, uint32_t lo, uint32_t hi,
+                                                   uint32_t tau) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t nq = row_quads(lo, hi), rounds = 32u / nq, ri = (uint32_t)lane / nq;
+    const uint32_t q = (lo >> 2) + (uint32_t)lane % nq;
+    const uint4 t4 = a.tau ? __ldg(reinterpret_cast<const uint4*>(a.tau) + q) : make_uint4(tau, tau, tau, tau);
+    for (uint32_t r = 0; r < a.retry_cap; r += rounds) {
+        unsigned live = 0;
+        if (ri < rounds && r + ri < a.retry_cap)
+            live = quad_live(q, coin_block(a.rk, q, r + ri, kDomFirst, j), t4, lo, hi);
+        const unsigned bal = __ballot_sync(kFull, live != 0u);
+        if (bal) return r + (uint32_t)(__ffs(bal) - 1) / nq;
+    }
+    return a.retry_cap;
+}
+constexpr uint32_t kShortRow = 16;  // longest source row (edge quads) whose rounds are searched by accepted_round
+
+// The edge quads of up to 32 rows laid end to end, two a lane and step: the
+// rows with edges are packed into shared memory (first quad, first and end
+// edge, threshold), and the row of quad g is the number of rows that start at
+// or before it, a popcount of the step's row starts (one OR-reduction of the
+// rows' start bits).
+struct RowBatch {
+    uint4* row;       // the warp's 32 packed rows
+    uint32_t nq, excl, total;
+
+    // lane's row: edges [lo, hi), threshold tau; nq edge quads of it are drawn (0: none)
+    __device__ __forceinline__ RowBatch(uint4* rows, uint32_t lo, uint32_t hi, uint32_t tau, uint32_t nq_)
+        : row(rows), nq(nq_) {
+        const int lane = threadIdx.x & 31;
+        uint32_t incl = nq;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(kFull, incl, d);
+            if (lane >= d) incl += y;
         }
-        const unsigned m = __ballot_sync(kFull, fresh);
-        if (m) {
-            uint32_t base = 0;
-            if ((threadIdx.x & 31) == 0) base = atomicAdd(qlen, (uint32_t)__popc(m));
-            base = __shfl_sync(kFull, base, 0);
-            if (fresh) {
-                const uint32_t pos = base + __popc(m & lanemask_lt());
-                if (pos < cap) queue[pos] = u;
-                else atomicAnd(&bitmap[u >> 5], ~(1u << (u & 31)));
-            }
+        total = __shfl_sync(kFull, incl, 31);
+        excl = incl - nq;
+        const unsigned m = __ballot_sync(kFull, nq > 0);
+        if (nq) row[__popc(m & lanemask_lt())] = make_uint4(excl, lo, hi, tau);
+        __syncwarp();
+    }
+
+    // rows that start before quad `base`
+    __device__ __forceinline__ uint32_t started(uint32_t base) const {
+        return (uint32_t)__popc(__ballot_sync(kFull, nq && excl < base));
+    }
+
+    // the packed row of quad base + lane, *st rows starting before base (advanced past the 32 quads);
+    // past the batch's end the last row
+    __device__ __forceinline__ uint4 find(uint32_t base, uint32_t* st) const {
+        const uint32_t d = excl - base;
+        const unsigned m = __reduce_or_sync(kFull, nq && d < 32u ? 1u << d : 0u);
+        const uint32_t i = *st + __popc(m & (lanemask_lt() | (1u << (threadIdx.x & 31)))) - 1;
+        *st += __popc(m);
+        return row[i];
+    }
+
+    // Draws the BFS coins of quads [base, base + 64) of sample blk and hands
+    // each lane's live masks to list(quad, mask) (called warp-uniformly, with no lanes missing).
+    template <class List>
+    __device__ __forceinline__ void step(const SampleArgs& a, const SampleBlock& blk, uint32_t base, uint32_t* st,
+                                         List&& list) const {
+        const uint4* __restrict__ tau4 = reinterpret_cast<const uint4*>(a.tau);
+        const uint32_t g0 = base + (threadIdx.x & 31), g1 = g0 + 32;
+        const uint4 r0 = find(base, st), r1 = find(base + 32, st);
+        // lanes past the batch's end take its last quad and drop its coins
+        const uint32_t q0 = (r0.y >> 2) + (min(g0, total - 1) - r0.x);
+        const uint32_t q1 = (r1.y >> 2) + (min(g1, total - 1) - r1.x);
+        const bool two = base + 32 < total;  // warp-uniform
+        const uint4 t0 = tau4 ? __ldg(tau4 + q0) : make_uint4(r0.w, r0.w, r0.w, r0.w);
+        unsigned l0 = 0, l1 = 0;
+        if (two) {  // two independent blocks
+            const uint4 t1 = tau4 ? __ldg(tau4 + q1) : make_uint4(r1.w, r1.w, r1.w, r1.w);
+            const uint4 x0 = blk(q0, a.rk), x1 = blk(q1, a.rk);
+            l0 = quad_live(q0, x0, t0, r0.y, r0.z);
+            if (g1 < total) l1 = quad_live(q1, x1, t1, r1.y, r1.z);
+        } else if (g0 < total) {
+            l0 = quad_live(q0, blk(q0, a.rk), t0, r0.y, r0.z);
         }
+#pragma unroll 1
+        for (int h = 0; h < (two ? 2 : 1); ++h) list(h ? q1 : q0, h ? l1 : l0);
     }
 };
 
-// Expand the in-rows held by the lanes (lane i: row off/deg/tau_row, deg = 0
-// for none): every in-edge e gets its coin (domain dom, round retry, sample
-// j); live edges offer their source to the inserter. Returns, warp-uniform,
-// whether any edge was live.
-template <class Ins>
-__device__ __forceinline__ bool expand_rows(const SampleArgs& a, uint64_t j, uint32_t dom, uint32_t retry,
-                                            uint64_t off, uint32_t deg, uint32_t tau_row, Ins& ins) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t nq = deg ? (uint32_t)(((off + deg - 1) >> 2) - (off >> 2) + 1) : 0u;
-    uint32_t incl = nq;
+// The live edges (mask of edge quad q) of every lane join the warp's list of
+// edge positions; returns the list's new length (at most 128 more).
+__device__ __forceinline__ uint32_t list_live(uint32_t* pend, uint32_t npend, uint32_t q, unsigned live) {
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t y = __shfl_up_sync(kFull, incl, d);
-        if (lane >= d) incl += y;
+    for (int k = 0; k < 4; ++k) {
+        const unsigned m = __ballot_sync(kFull, (live >> k) & 1u);
+        if ((live >> k) & 1u) pend[npend + __popc(m & lanemask_lt())] = 4u * q + (uint32_t)k;
+        npend += __popc(m);
     }
-    const uint32_t total = __shfl_sync(kFull, incl, 31);
-    const uint32_t excl = incl - nq;
-    bool any = false;
-    for (uint32_t base = 0; base < total; base += 32) {
-        const uint32_t g = base + lane;
-        int owner = 0;
-#pragma unroll
-        for (int step = 16; step >= 1; step >>= 1) {
-            const uint32_t v = __shfl_sync(kFull, incl, owner + step - 1);
-            if (v <= g) owner += step;
-        }
-        const uint64_t o_off = __shfl_sync(kFull, off, owner);
-        const uint32_t o_deg = __shfl_sync(kFull, deg, owner);
-        const uint32_t o_tau = __shfl_sync(kFull, tau_row, owner);
-        const uint32_t o_excl = __shfl_sync(kFull, excl, owner);
-        int32_t c0 = -1, c1 = -1, c2 = -1, c3 = -1;
-        if (g < total) {
-            const uint64_t q = (o_off >> 2) + (g - o_excl);
-            const uint4 x = coin_block(a.rk, q, retry, dom, j);
-            const uint4 t4 = a.tau ? __ldg(reinterpret_cast<const uint4*>(a.tau) + q)
-                                   : make_uint4(o_tau, o_tau, o_tau, o_tau);
-            const uint64_t e0 = q << 2, lo = o_off, hi = o_off + o_deg;
-            unsigned live = 0;
-            live |= (e0 + 0 >= lo && e0 + 0 < hi && coin_live(x.x, t4.x)) ? 1u : 0u;
-            live |= (e0 + 1 >= lo && e0 + 1 < hi && coin_live(x.y, t4.y)) ? 2u : 0u;
-            live |= (e0 + 2 >= lo && e0 + 2 < hi && coin_live(x.z, t4.z)) ? 4u : 0u;
-            live |= (e0 + 3 >= lo && e0 + 3 < hi && coin_live(x.w, t4.w)) ? 8u : 0u;
-            if (live) {
-                const int4 s4 = __ldg(reinterpret_cast<const int4*>(a.src) + q);
-                any = true;
-                if (live & 1u) c0 = s4.x;
-                if (live & 2u) c1 = s4.y;
-                if (live & 4u) c2 = s4.z;
-                if (live & 8u) c3 = s4.w;
-            }
-        }
-        if (__any_sync(kFull, (c0 >= 0) | (c1 >= 0) | (c2 >= 0) | (c3 >= 0))) {
-            if (__any_sync(kFull, c0 >= 0)) ins.insert(c0);
-            if (__any_sync(kFull, c1 >= 0)) ins.insert(c1);
-            if (__any_sync(kFull, c2 >= 0)) ins.insert(c2);
-            if (__any_sync(kFull, c3 >= 0)) ins.insert(c3);
-            if (ins.overflow) break;
-        }
-    }
-    return __any_sync(kFull, any);
-}
-
-// Alg. 1's conditioned first step for one warp: the rejection rounds r = 0, 1, ... of the
-// source row, until one round has a live coin; the live in-neighbours of that
-// round are inserted. Rounds are independent given (j, r), so a short row
-// (nq <= 16 edge quads) is searched 32 / nq rounds per pass: lane g takes
-// round r0 + g / nq and quad g % nq, and the lowest round with a live coin
-// (the first set lane of the ballot, as lanes are ordered by round) is the
-// accepted one, exactly as in sequential order. Longer rows take one round
-// per pass, spread over the lanes. Returns the accepted round, or the cap
-// with *failed set.
-template <class Ins>
-__device__ __forceinline__ uint32_t first_step_warp(const SampleArgs& a, uint64_t j, const RowInfo& rv, Ins& ins,
-                                                    bool* failed, int64_t pick_e = -1, int32_t pick_u = -1) {
-    const int lane = threadIdx.x & 31;
-    *failed = false;
-    if (a.chain) {  // bucket form: the picked in-edge, then round-0 coins after it
-        int32_t u = -1;
-        uint64_t e = 0;
-        if (lane == 0) {
-            if (pick_e >= 0) {  // drawn by the prepass
-                e = (uint64_t)pick_e;
-                u = pick_u;
-            } else {
-                e = bucket_pick(a, j, rv.off, rv.deg);
-                u = a.src[e];
-            }
-        }
-        e = __shfl_sync(kFull, e, 0);
-        ins.insert(u);
-        const uint64_t rest = rv.off + rv.deg - (e + 1);
-        expand_rows(a, j, kDomFirst, 0, e + 1, lane == 0 ? (uint32_t)rest : 0u, rv.tau, ins);
-        return 0;
-    }
-    if (a.ris) {  // RIS: round 0, accepted whatever its coins
-        expand_rows(a, j, kDomFirst, 0, rv.off, lane == 0 ? rv.deg : 0u, rv.tau, ins);
-        return 0;
-    }
-    const uint64_t q_first = rv.off >> 2;
-    const uint32_t nq = (uint32_t)(((rv.off + rv.deg - 1) >> 2) - q_first + 1);
-    if (nq > 16) {
-        for (uint32_t r = 0;; ++r) {
-            if (r >= a.retry_cap) { *failed = true; return r; }
-            if (expand_rows(a, j, kDomFirst, r, rv.off, lane == 0 ? rv.deg : 0u, rv.tau, ins)) return r;
-        }
-    }
-    const uint32_t rounds = 32u / nq;
-    const uint32_t ri = (uint32_t)lane / nq, qi = (uint32_t)lane % nq;
-    const uint64_t q = q_first + qi;
-    const uint64_t e0 = q << 2, lo = rv.off, hi = rv.off + rv.deg;
-    const uint4 t4 = a.tau ? __ldg(reinterpret_cast<const uint4*>(a.tau) + q) : make_uint4(rv.tau, rv.tau, rv.tau, rv.tau);
-    for (uint32_t r0 = 0; r0 < a.retry_cap; r0 += rounds) {
-        const uint32_t r = r0 + ri;
-        unsigned live = 0;
-        if (ri < rounds && r < a.retry_cap) {
-            const uint4 x = coin_block(a.rk, q, r, kDomFirst, j);
-            live |= (e0 + 0 >= lo && e0 + 0 < hi && coin_live(x.x, t4.x)) ? 1u : 0u;
-            live |= (e0 + 1 >= lo && e0 + 1 < hi && coin_live(x.y, t4.y)) ? 2u : 0u;
-            live |= (e0 + 2 >= lo && e0 + 2 < hi && coin_live(x.z, t4.z)) ? 4u : 0u;
-            live |= (e0 + 3 >= lo && e0 + 3 < hi && coin_live(x.w, t4.w)) ? 8u : 0u;
-        }
-        const unsigned bal = __ballot_sync(kFull, live != 0);
-        if (bal) {
-            const uint32_t acc = (uint32_t)(__ffs(bal) - 1) / nq;  // accepted round = r0 + acc
-            int32_t c0 = -1, c1 = -1, c2 = -1, c3 = -1;
-            if (ri == acc && live) {
-                const int4 s4 = __ldg(reinterpret_cast<const int4*>(a.src) + q);
-                if (live & 1u) c0 = s4.x;
-                if (live & 2u) c1 = s4.y;
-                if (live & 4u) c2 = s4.z;
-                if (live & 8u) c3 = s4.w;
-            }
-            if (__any_sync(kFull, c0 >= 0)) ins.insert(c0);
-            if (__any_sync(kFull, c1 >= 0)) ins.insert(c1);
-            if (__any_sync(kFull, c2 >= 0)) ins.insert(c2);
-            if (__any_sync(kFull, c3 >= 0)) ins.insert(c3);
-            return r0 + acc;
-        }
-    }
-    *failed = true;
-    return a.retry_cap;
+    return npend;
 }
 
 __device__ __forceinline__ uint64_t warp_sum_u64(uint64_t v) {
@@ -811,13 +744,11 @@ __global__ void __launch_bounds__(kLaneBlock, 4) k_iis_lane(SampleArgs a) {
 }
 
 // ------------------------------------------------------------- warp tier
-// One warp per sample. Up to 32 queued rows are taken at a time and their
-// edge quads laid end to end over the lanes, two a lane and step: the row of
-// quad g is the number of rows that start at or before it, a popcount of the
-// step's row starts (one OR-reduction of the rows' start bits). Live edges
-// are only listed (their positions, in shared memory) and joined 32 at a time,
-// one a lane, so that the source gather, the probe and the row load of 32
-// candidates overlap and an insert round has every lane busy.
+// One warp per sample. Up to 32 queued rows are taken at a time and their edge
+// quads dealt to the lanes (RowBatch). Live edges are only listed (their
+// positions, in shared memory) and joined 32 at a time, one a lane, so that
+// the source gather, the probe and the row load of 32 candidates overlap and
+// an insert round has every lane busy.
 // Two thirds of a weighted-cascade sketch's members lie in samples of more
 // than 256 members, so the tier goes on past shared memory: the spill slots
 // of 1536 members keep all but 1 in 130 samples of Chung-Lu 1M / 17.5M off
@@ -828,14 +759,12 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_iis_warp(SampleArgs a) {
     __shared__ __align__(16) uint32_t s_hash[kWarpThreads / 32][kHCap];
     __shared__ __align__(16) int32_t s_queue[kWarpThreads / 32][kQCap];
     __shared__ uint4 s_ring[kWarpThreads / 32][kRing];
-    __shared__ uint4 s_row[kWarpThreads / 32][32];  // the batch's rows: quads before it, first and end edge, threshold
+    __shared__ uint4 s_row[kWarpThreads / 32][32];
     __shared__ uint32_t s_pend[kWarpThreads / 32][kPend];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const uint64_t wid = (uint64_t)blockIdx.x * (kWarpThreads / 32) + wib;
     uint32_t* const hash = s_hash[wib];
-    uint4* const row = s_row[wib];
     uint32_t* const pend = s_pend[wib];
-    const uint4* __restrict__ tau4 = reinterpret_cast<const uint4*>(a.tau);
     uint64_t chunk_pos = 0, chunk_end = 0;  // this warp's arena reservation
     uint32_t chunk = kArenaChunk;
 
@@ -881,39 +810,24 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_iis_warp(SampleArgs a) {
                 const int32_t u = (uint32_t)lane < cnt ? __ldg(a.src + pend[npend + lane]) : -1;
                 ins.insert(u);
             };
-            // the live edges (bit k: edge 4 q + k) of every lane join the list
             auto list = [&](uint32_t q, unsigned live) {
                 if (!__any_sync(kFull, live != 0u)) return;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const unsigned m = __ballot_sync(kFull, (live >> k) & 1u);
-                    if ((live >> k) & 1u) pend[npend + __popc(m & lanemask_lt())] = 4u * q + (uint32_t)k;
-                    npend += __popc(m);
-                }
+                npend = list_live(pend, npend, q, live);
 #pragma unroll 1
                 while (npend >= 32u) join(32u);
             };
-            // live mask of quad q (block x, thresholds t) within its row's edges [lo, hi)
-            auto coins4 = [](uint32_t q, const uint4& x, const uint4& t, uint32_t lo, uint32_t hi) -> unsigned {
-                const uint32_t e0 = q << 2;
-                const unsigned live = (coin_live(x.x, t.x) ? 1u : 0u) | (coin_live(x.y, t.y) ? 2u : 0u) |
-                                      (coin_live(x.z, t.z) ? 4u : 0u) | (coin_live(x.w, t.w) ? 8u : 0u);
-                const uint32_t before = e0 < lo ? lo - e0 : 0u, after = e0 + 4 > hi ? e0 + 4 - hi : 0u;
-                return live & (15u << before) & (15u >> after);
-            };
             // the FIRST coins of round r on the source's in-edges [lo, hi); whether one is live
             auto first_row = [&](uint32_t lo, uint32_t hi, uint32_t r) -> bool {
-                if (hi <= lo) return false;
-                const uint32_t qe = ((hi - 1) >> 2) + 1;
+                const uint32_t qe = (lo >> 2) + row_quads(lo, hi);
                 bool any = false;
 #pragma unroll 1
                 for (uint32_t qb = lo >> 2; qb < qe && !ins.overflow; qb += 32) {
                     const uint32_t q = qb + lane;
                     unsigned live = 0;
                     if (q < qe) {
-                        const uint4 x = coin_block(a.rk, q, r, kDomFirst, j);
-                        const uint4 t4 = tau4 ? __ldg(tau4 + q) : make_uint4(rv.tau, rv.tau, rv.tau, rv.tau);
-                        live = coins4(q, x, t4, lo, hi);
+                        const uint4 t4 = a.tau ? __ldg(reinterpret_cast<const uint4*>(a.tau) + q)
+                                               : make_uint4(rv.tau, rv.tau, rv.tau, rv.tau);
+                        live = quad_live(q, coin_block(a.rk, q, r, kDomFirst, j), t4, lo, hi);
                     }
                     any |= live != 0u;
                     list(q, live);
@@ -921,12 +835,11 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_iis_warp(SampleArgs a) {
                 return __any_sync(kFull, any);
             };
 
-            // the conditioned first step (first_step_warp's cases): the bucket
-            // form's pick and the coins after it, RIS's one round, or the
-            // accepted round r of the rejection form
+            // Alg. 1's conditioned first step: the bucket form's picked in-edge
+            // and round-0 coins after it, RIS's one round whatever its coins, or
+            // the first round with a live coin
             const uint32_t s_lo = (uint32_t)rv.off, s_hi = s_lo + rv.deg;
             uint32_t r = 0, from = s_lo;
-            bool failed = false;
             if (a.chain) {
                 uint32_t e = 0;
                 if (lane == 0) {
@@ -935,38 +848,11 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_iis_warp(SampleArgs a) {
                 }
                 npend = 1;
                 from = __shfl_sync(kFull, e, 0) + 1;
-            } else if (!a.ris) {
-                const uint32_t nq = ((s_hi - 1) >> 2) - (s_lo >> 2) + 1;
-                if (nq <= 16) {
-                    // a short row, 32 / nq rounds a pass: lane g draws quad g % nq of round
-                    // r + g / nq; the first lane with a live coin is in the accepted round
-                    const uint32_t rounds = 32u / nq, ri = (uint32_t)lane / nq;
-                    const uint32_t q = (s_lo >> 2) + (uint32_t)lane % nq;
-                    const uint4 t4 = tau4 ? __ldg(tau4 + q) : make_uint4(rv.tau, rv.tau, rv.tau, rv.tau);
-                    for (;; r += rounds) {
-                        if (r >= a.retry_cap) {
-                            failed = true;
-                            r = a.retry_cap;
-                            break;
-                        }
-                        unsigned live = 0;
-                        if (ri < rounds && r + ri < a.retry_cap)
-                            live = coins4(q, coin_block(a.rk, q, r + ri, kDomFirst, j), t4, s_lo, s_hi);
-                        const unsigned bal = __ballot_sync(kFull, live != 0u);
-                        if (bal) {
-                            r += (uint32_t)(__ffs(bal) - 1) / nq;
-                            break;
-                        }
-                    }
-                }
+            } else if (!a.ris && row_quads(s_lo, s_hi) <= kShortRow) {
+                r = accepted_round(a, j, s_lo, s_hi, rv.tau);
             }
-            if (!failed)
-                while (!first_row(from, s_hi, r) && !a.chain && !a.ris) {  // at once for a short row's accepted round
-                    if (++r >= a.retry_cap) {
-                        failed = true;
-                        break;
-                    }
-                }
+            bool failed = r >= a.retry_cap;
+            while (!failed && !first_row(from, s_hi, r) && !a.chain && !a.ris) failed = ++r >= a.retry_cap;
             if (failed) {
                 if (lane == 0) record_retry_failure(a, j, v, r, rv.deg);
                 __syncwarp();
@@ -1006,49 +892,10 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_iis_warp(SampleArgs a) {
                     break;
                 }
                 coins += deg;
-                const uint32_t hi = lo + deg;
-                const uint32_t nq = deg ? ((hi - 1) >> 2) - (lo >> 2) + 1 : 0u;
-                uint32_t incl = nq;
-#pragma unroll
-                for (int d = 1; d < 32; d <<= 1) {
-                    const uint32_t y = __shfl_up_sync(kFull, incl, d);
-                    if (lane >= d) incl += y;
-                }
-                const uint32_t total = __shfl_sync(kFull, incl, 31), excl = incl - nq;
-                const unsigned rowm = __ballot_sync(kFull, nq > 0);
-                if (nq) row[__popc(rowm & lanemask_lt())] = make_uint4(excl, lo, hi, tau_row);
-                __syncwarp();
-                uint32_t started = 0;  // rows that start before this step's quads
+                const RowBatch rb(s_row[wib], lo, lo + deg, tau_row, row_quads(lo, lo + deg));
+                uint32_t st = 0;
 #pragma unroll 1
-                for (uint32_t base = 0; base < total && !ins.overflow; base += 64) {
-                    const uint32_t g0 = base + lane, g1 = g0 + 32;
-                    const uint32_t d0 = excl - base, d1 = d0 - 32;
-                    const unsigned m0 = __reduce_or_sync(kFull, nq && d0 < 32u ? 1u << d0 : 0u);
-                    const unsigned m1 = __reduce_or_sync(kFull, nq && d1 < 32u ? 1u << d1 : 0u);
-                    const unsigned le = lanemask_lt() | (1u << lane);
-                    const uint32_t i0 = started + __popc(m0 & le) - 1;
-                    started += __popc(m0);
-                    const uint32_t i1 = started + __popc(m1 & le) - 1;
-                    started += __popc(m1);
-                    // lanes past the batch's end take its last quad (i0 and i1
-                    // then name the last row) and drop its coins
-                    const uint4 r0 = row[i0], r1 = row[i1];
-                    const uint32_t q0 = (r0.y >> 2) + (min(g0, total - 1) - r0.x);
-                    const uint32_t q1 = (r1.y >> 2) + (min(g1, total - 1) - r1.x);
-                    const bool two = base + 32 < total;  // warp-uniform
-                    const uint4 t0v = tau4 ? __ldg(tau4 + q0) : make_uint4(r0.w, r0.w, r0.w, r0.w);
-                    unsigned l0 = 0, l1 = 0;
-                    if (two) {  // two independent blocks
-                        const uint4 t1v = tau4 ? __ldg(tau4 + q1) : make_uint4(r1.w, r1.w, r1.w, r1.w);
-                        const uint4 x0 = blk(q0, a.rk), x1 = blk(q1, a.rk);
-                        l0 = coins4(q0, x0, t0v, r0.y, r0.z);
-                        if (g1 < total) l1 = coins4(q1, x1, t1v, r1.y, r1.z);
-                    } else if (g0 < total) {
-                        l0 = coins4(q0, blk(q0, a.rk), t0v, r0.y, r0.z);
-                    }
-#pragma unroll 1
-                    for (int h = 0; h < (two ? 2 : 1); ++h) list(h ? q1 : q0, h ? l1 : l0);
-                }
+                for (uint32_t base = 0; base < rb.total && !ins.overflow; base += 64) rb.step(a, blk, base, &st, list);
             }
             if (ins.overflow || heavy) {  // more members or coins than the tier takes: CTA tier
                 if (lane == 0) hand_on(a, j);
@@ -1094,35 +941,60 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_iis_warp(SampleArgs a) {
 // -------------------------------------------------------------- CTA tier
 // One block of kCtaThreads threads per sample, 1024 threads of such blocks per
 // SM (four of 256 by default, or two of 512: the option SKIS_OPT_CTA_THREADS).
+// The reverse BFS goes level by level. The in-rows of a level's first
+// kCtaWin vertices wait in shared memory: a vertex's row is loaded while its
+// visited bit is set, so a level costs two memory latencies (the source
+// gather, then the bit with the row) and one block barrier. Weighted cascade
+// has narrow levels, a few rows each, and is bound by these.
+// A level's rows go to the warps 32 at a time, a batch split over several
+// warps where there are fewer batches than warps (RowBatch); rows of
+// cta_hub_quads edge quads or more are strided over the whole block. Live
+// edges are listed per warp and joined 32 at a time, the rest at the end of
+// the level. Before, each of a quad's four words was inserted in turn (four
+// atomic round trips a level) and every level read its queue and rows back:
+// on Chung-Lu 1M / 17.5M WC the 7670 samples of 1M that run here took 7.4 ms
+// and take 4.4 ms. Where hubs hold the coins it is bound by the coin
+// generator: R-MAT 2^22 / 2^27 WC 355G blocks/s, 2^25 / 2^30 421G (the hub
+// loop alone, with no other work in the kernel, 455G).
+constexpr int kCtaWin = 512;  // rows of a level in shared memory at a time
+
 template <int kCtaThreads>
 __global__ void __launch_bounds__(kCtaThreads, 1024 / kCtaThreads) k_iis_cta(SampleArgs a) {
-    constexpr int kCtaWin = 2 * kCtaThreads;  // queued vertices per load-balanced window
+    constexpr int kWarps = kCtaThreads / 32;
     __shared__ unsigned long long s_j;
-    __shared__ uint32_t s_qlen;
     __shared__ unsigned long long s_coins;
     __shared__ unsigned long long s_base;
-    __shared__ uint32_t s_r, s_failed;
-    __shared__ uint32_t s_pre[kCtaWin], s_lo[kCtaWin], s_hi[kCtaWin], s_tau[kCtaWin];
-    __shared__ uint32_t s_hub[kCtaWin];  // window rows taken by the hub loop
-    __shared__ uint32_t s_nhub;
-    __shared__ uint32_t s_small[3];      // a small window's quad-group shift, quad groups and hub rows
-    __shared__ uint32_t s_wsum[kCtaThreads / 32];
+    __shared__ uint4 s_win[2][kCtaWin];      // rows of this level and the next: first and end edge, threshold
+    __shared__ uint16_t s_hub[2][kCtaWin];   // those of them that the hub loop takes
+    // the previous, this and the next level's joins: vertices, hubs among them
+    // in the window, edge quads of the others and chunks of 64 quads of the hubs
+    struct Level {
+        uint32_t size, hubs, quads, chunks;
+    };
+    __shared__ __align__(16) Level s_lvl[3];
+    __shared__ uint4 s_row[kWarps][32];
+    __shared__ uint32_t s_pend[kWarps][kPend];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    constexpr int kWarps = kCtaThreads / 32;
-    static_assert(kCtaWin == 2 * kCtaThreads, "two window rows per thread");
+    uint32_t* const pend = s_pend[wid];
     uint32_t* bitmap = a.bitmaps + (uint64_t)blockIdx.x * a.bitmap_words;
     int32_t* queue = a.queues + (uint64_t)blockIdx.x * a.queue_cap;
+    const uint4* __restrict__ tau4 = reinterpret_cast<const uint4*>(a.tau);
+    const uint4* __restrict__ rows4 = reinterpret_cast<const uint4*>(a.rows);  // offset (low, high), degree, threshold
     const uint64_t count = input_count(a);
-    if (threadIdx.x == 0) s_nhub = 0;
+    auto is_hub = [&](uint32_t nq) { return a.cta_hub_quads && nq >= a.cta_hub_quads; };
+    unsigned long long claim = 0;  // thread 0: the block's next input
+    if (threadIdx.x == 0) claim = atomicAdd(a.work, 1ull);
 
     for (;;) {
         if (threadIdx.x == 0) {
-            const unsigned long long t = atomicAdd(a.work, 1ull);
-            s_j = t < count ? input_id(a, t) : ~0ull;
+            s_j = claim < count ? input_id(a, claim) : ~0ull;
+            s_coins = 0;
+            s_lvl[0] = s_lvl[1] = s_lvl[2] = Level{0, 0, 0, 0};
         }
         __syncthreads();
         const uint64_t j = s_j;
         if (j == ~0ull) break;
+        if (threadIdx.x == 0) claim = atomicAdd(a.work, 1ull);  // arrives while this sample is drawn
 
         RowInfo rv;
         int64_t pe;
@@ -1131,42 +1003,94 @@ __global__ void __launch_bounds__(kCtaThreads, 1024 / kCtaThreads) k_iis_cta(Sam
         if (threadIdx.x == 0) {
             bitmap[v >> 5] |= 1u << (v & 31);
             queue[0] = (int32_t)v;
-            s_qlen = 1;
-            s_coins = 0;
         }
-        __syncthreads();
-        CtaInserter ins{bitmap, queue, &s_qlen, a.queue_cap, false};
+        __syncthreads();  // the source's bit is set before any other
 
-        // first step: a short source row is searched by warp 0, several
-        // rounds per pass; a long one is split over the warps in whole quads
-        uint32_t r = 0;
-        bool failed = false;
-        const uint64_t nq_src = ((rv.off + rv.deg - 1) >> 2) - (rv.off >> 2) + 1;
-        if (nq_src <= 16 || a.chain) {
-            if (wid == 0) {
-                bool f = false;
-                const uint32_t rr = first_step_warp(a, j, rv, ins, &f, pe, pu);
-                if (lane == 0) {
-                    s_r = rr;
-                    s_failed = f ? 1u : 0u;
+        uint32_t tail = 1;     // members before this level's joins
+        uint64_t coins = 0;    // in-edges of the members that this lane joined
+        int cur = 0, nxt = 1;  // this level's joins, the next level's (zero)
+        int buf = 0;           // half of s_win that this level's joins fill
+        uint32_t npend = 0;
+        // the sources of the last cnt listed edges join the sample, one a lane.
+        // A vertex past the queue's capacity gets its bit back, so that the
+        // bitmap always holds exactly the queued vertices (the counter still
+        // counts it: the sample is then known to have outgrown the slot)
+        auto join = [&](uint32_t cnt) {
+            __syncwarp();
+            npend -= cnt;
+            int32_t u = 0;
+            bool fresh = false;
+            uint4 rw = make_uint4(0, 0, 0, 0);
+            if ((uint32_t)lane < cnt) {
+                u = __ldg(a.src + pend[npend + lane]);
+                rw = __ldg(rows4 + u);  // in flight while the bit is set
+                fresh = (atomicOr(&bitmap[(uint32_t)u >> 5], 1u << (u & 31)) & (1u << (u & 31))) == 0;
+            }
+            const unsigned m = __ballot_sync(kFull, fresh);
+            if (m) {
+                uint32_t at = 0;
+                if (lane == 0) at = atomicAdd(&s_lvl[cur].size, (uint32_t)__popc(m));
+                at = __shfl_sync(kFull, at, 0) + __popc(m & lanemask_lt());
+                const uint32_t nq = fresh ? row_quads(rw.x, rw.x + rw.z) : 0u;
+                const uint32_t quads = __reduce_add_sync(kFull, is_hub(nq) ? 0u : nq);
+                if (lane == 0) atomicAdd(&s_lvl[cur].quads, quads);
+                if (fresh) {
+                    coins += rw.z;
+                    if (tail + at < a.queue_cap) queue[tail + at] = u;
+                    else atomicAnd(&bitmap[(uint32_t)u >> 5], ~(1u << (u & 31)));
+                    if (at < (uint32_t)kCtaWin) {
+                        s_win[buf][at] = make_uint4(rw.x, rw.x + rw.z, rw.w, 0u);
+                        if (is_hub(nq)) {
+                            s_hub[buf][atomicAdd(&s_lvl[cur].hubs, 1u)] = (uint16_t)at;
+                            atomicAdd(&s_lvl[cur].chunks, (nq + 63) / 64);
+                        }
+                    }
                 }
             }
-            __syncthreads();
-            r = s_r;
-            failed = s_failed != 0;
-        } else {
-            const uint64_t q_lo = rv.off >> 2;
-            const uint64_t nq = rv.deg ? ((rv.off + rv.deg - 1) >> 2) - q_lo + 1 : 0;
-            const uint64_t per = (nq + kWarps - 1) / kWarps;
-            const uint64_t a_lo = max(rv.off, (q_lo + (uint64_t)wid * per) << 2);
-            const uint64_t a_hi = min(rv.off + rv.deg, (q_lo + (uint64_t)(wid + 1) * per) << 2);
-            const uint32_t sub_deg = a_hi > a_lo ? (uint32_t)(a_hi - a_lo) : 0u;
-            for (;;) {
-                const bool any_w = expand_rows(a, j, kDomFirst, r, a_lo, lane == 0 ? sub_deg : 0u, rv.tau, ins);
-                const int any = __syncthreads_or(any_w ? 1 : 0);
-                if (any || a.ris) break;
-                if (++r >= a.retry_cap) { failed = true; break; }
+            __syncwarp();
+        };
+        auto list = [&](uint32_t q, unsigned live) {
+            if (!__any_sync(kFull, live != 0u)) return;
+            npend = list_live(pend, npend, q, live);
+#pragma unroll 1
+            while (npend >= 32u) join(32u);
+        };
+
+        // Alg. 1's conditioned first step: the source row is strided over the
+        // block in whole quads (a short row's rounds are searched by every warp
+        // for itself, and its accepted round drawn by the first)
+        const uint32_t s_lo = (uint32_t)rv.off, s_hi = s_lo + rv.deg;
+        uint32_t r = 0, from = s_lo;
+        const bool short_row = !a.chain && !a.ris && row_quads(s_lo, s_hi) <= kShortRow;
+        if (a.chain) {
+            uint32_t e = 0;
+            if (lane == 0) e = pe >= 0 ? (uint32_t)pe : (uint32_t)bucket_pick(a, j, rv.off, rv.deg);
+            e = __shfl_sync(kFull, e, 0);
+            if (wid == 0) {
+                if (lane == 0) pend[0] = e;
+                npend = 1;
             }
+            from = e + 1;
+        } else if (short_row) {
+            r = accepted_round(a, j, s_lo, s_hi, rv.tau);
+        }
+        bool failed = r >= a.retry_cap;
+        while (!failed) {
+            const uint32_t qe = (from >> 2) + row_quads(from, s_hi);
+            bool any = false;
+#pragma unroll 1
+            for (uint32_t qb = (from >> 2) + wid * 32; qb < qe; qb += kCtaThreads) {
+                const uint32_t q = qb + lane;
+                unsigned live = 0;
+                if (q < qe) {
+                    const uint4 t4 = tau4 ? __ldg(tau4 + q) : make_uint4(rv.tau, rv.tau, rv.tau, rv.tau);
+                    live = quad_live(q, coin_block(a.rk, q, r, kDomFirst, j), t4, from, s_hi);
+                }
+                any |= live != 0u;
+                list(q, live);
+            }
+            if (a.chain || a.ris || short_row || __syncthreads_or(any ? 1 : 0)) break;
+            failed = ++r >= a.retry_cap;
         }
         if (failed) {
             if (threadIdx.x == 0) {
@@ -1176,244 +1100,128 @@ __global__ void __launch_bounds__(kCtaThreads, 1024 / kCtaThreads) k_iis_cta(Sam
             __syncthreads();
             continue;
         }
+        if (npend) join(npend);
 
-        // reverse BFS, level by level. A level [head, tail) is taken in
-        // windows of up to kCtaWin queued vertices; the edge quads of a
-        // window's rows are laid end to end and dealt to the warps 32 at a
-        // time, so one long in-row (a hub) is shared by every warp.
-        uint64_t coins = 0;
-        uint32_t head = 1;
-        uint32_t tail = s_qlen;  // after the first step's barrier: its inserts are in
+        // reverse BFS, level by level
+        const SampleBlock blk(a.rk, j, kDomBfs);
         for (;;) {
-            if (head >= tail || tail > a.queue_cap) break;  // done, or the sample outgrew the slot
-            for (uint32_t w0 = head; w0 < tail; w0 += kCtaWin) {
-                const uint32_t nw = min((uint32_t)kCtaWin, tail - w0);
-                uint32_t gsh, total, nhub;  // quad-group shift, quad groups and hub rows of the window
-                if (nw <= 32) {
-                    // a small window (the narrow frontiers of weighted cascade):
-                    // warp 0 loads, classifies and prefixes its rows, one barrier
-                    if (wid == 0) {
-                        uint32_t nq = 0;
-                        bool hub = false;
-                        if ((uint32_t)lane < nw) {
-                            const RowInfo rw = a.rows[queue[w0 + lane]];
-                            coins += rw.deg;
-                            const uint32_t lo = (uint32_t)rw.off, hi = lo + rw.deg;
-                            s_lo[lane] = lo;
-                            s_hi[lane] = hi;
-                            s_tau[lane] = rw.tau;
-                            nq = rw.deg ? ((hi - 1) >> 2) - (lo >> 2) + 1 : 0u;  // edge quads
-                            hub = a.cta_hub_quads && nq >= a.cta_hub_quads;
-                            if (hub) nq = 0;  // the hub loop takes it
-                        }
-                        const unsigned hb = __ballot_sync(kFull, hub);
-                        if (hub) s_hub[__popc(hb & lanemask_lt())] = (uint32_t)lane;
-                        const uint32_t g = __any_sync(kFull, nq >= (uint32_t)kCtaLongRow) ? (uint32_t)kCtaGroupLog2 : 0u;
-                        uint32_t x = (nq + (1u << g) - 1) >> g;
-#pragma unroll
-                        for (int d = 1; d < 32; d <<= 1) {
-                            const uint32_t y = __shfl_up_sync(kFull, x, d);
-                            if (lane >= d) x += y;
-                        }
-                        if ((uint32_t)lane < nw) s_pre[lane] = x;
-                        if (lane == 31) {
-                            s_small[0] = g;
-                            s_small[1] = x;
-                            s_small[2] = (uint32_t)__popc(hb);
+            __syncthreads();  // the last level's joins are in
+            const Level lvl = s_lvl[cur];
+            const uint32_t size = lvl.size, head = tail;
+            tail += size;
+            if (size == 0 || tail > a.queue_cap) break;  // done, or the sample outgrew the slot
+            // the counters rotate: this level fills `nxt` (zero), and the one
+            // after that, read by every thread before this barrier, is cleared
+            const int spare = 3 - cur - nxt;
+            cur = nxt;
+            nxt = spare;
+            if (threadIdx.x == 0) s_lvl[nxt] = Level{0, 0, 0, 0};
+            const uint4* const win = s_win[buf];
+            const uint16_t* const hubs = s_hub[buf];
+            buf ^= 1;
+#pragma unroll 1
+            for (uint32_t w0 = 0; w0 < size; w0 += kCtaWin) {
+                const uint32_t nw = min((uint32_t)kCtaWin, size - w0);
+                uint32_t nhub = lvl.hubs, chunks = lvl.chunks;
+                if (w0) {  // a wide level's later rows: loaded from the queue
+                    __shared__ uint32_t s_whub[2];
+                    __syncthreads();
+                    if (threadIdx.x < 2) s_whub[threadIdx.x] = 0;
+                    __syncthreads();
+                    for (uint32_t i = threadIdx.x; i < nw; i += kCtaThreads) {
+                        const uint4 rw = __ldg(rows4 + queue[head + w0 + i]);
+                        const uint32_t nq = row_quads(rw.x, rw.x + rw.z);
+                        s_win[buf ^ 1][i] = make_uint4(rw.x, rw.x + rw.z, rw.w, 0u);
+                        if (is_hub(nq)) {
+                            s_hub[buf ^ 1][atomicAdd(&s_whub[0], 1u)] = (uint16_t)i;
+                            atomicAdd(&s_whub[1], (nq + 63) / 64);
                         }
                     }
                     __syncthreads();
-                    gsh = s_small[0];
-                    total = s_small[1];
-                    nhub = s_small[2];
-                } else {
-                uint32_t nq2[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const uint32_t i = 2u * threadIdx.x + h;
-                    nq2[h] = 0;
-                    if (i < nw) {
-                        const RowInfo rw = a.rows[queue[w0 + i]];
-                        coins += rw.deg;
-                        const uint32_t lo = (uint32_t)rw.off, hi = lo + rw.deg;
-                        s_lo[i] = lo;
-                        s_hi[i] = hi;
-                        s_tau[i] = rw.tau;
-                        nq2[h] = rw.deg ? ((hi - 1) >> 2) - (lo >> 2) + 1 : 0u;  // edge quads
-                        if (a.cta_hub_quads && nq2[h] >= a.cta_hub_quads) {  // the hub loop takes it
-                            s_hub[atomicAdd(&s_nhub, 1u)] = i;
-                            nq2[h] = 0;
-                        }
+                    nhub = s_whub[0];
+                    chunks = s_whub[1];
+                }
+                // batches of 32 rows, each dealt to 2^sh warps while warps are left
+                // over (a narrow level's few quads go to the first warps, the
+                // others do not look at its rows)
+                const int batches = (int)((nw + 31) / 32);
+                const int sh = max(0, 31 - __clz(kWarps) - (batches > 1 ? 32 - __clz(batches - 1) : 0));
+                const uint32_t part = (uint32_t)wid & ((1u << sh) - 1u);
+#pragma unroll 1
+                for (int b = 64u * part < lvl.quads ? wid >> sh : batches; b < batches; b += kWarps >> sh) {
+                    const uint32_t i = 32u * b + lane;
+                    uint4 w = make_uint4(0, 0, 0, 0);
+                    if (i < nw) w = win[i];
+                    uint32_t nq = row_quads(w.x, w.y);
+                    if (is_hub(nq)) nq = 0;  // the hub loop takes it
+                    const RowBatch rb(s_row[wid], w.x, w.y, w.z, nq);
+#pragma unroll 1
+                    for (uint32_t base = 64u * part; base < rb.total; base += 64u << sh) {
+                        uint32_t st = rb.started(base);
+                        rb.step(a, blk, base, &st, list);
                     }
                 }
-                // a window with a long row (a hub) deals its quads kCtaGroup at
-                // a time to amortise the row search; others one at a time, so
-                // that short rows keep every lane busy
-                gsh = __syncthreads_or(nq2[0] >= (uint32_t)kCtaLongRow || nq2[1] >= (uint32_t)kCtaLongRow)
-                          ? (uint32_t)kCtaGroupLog2 : 0u;  // group of 2^gsh quads
-                const uint32_t grp0 = 1u << gsh;
-#pragma unroll
-                for (int h = 0; h < 2; ++h) nq2[h] = (nq2[h] + grp0 - 1) >> gsh;
-                // block-wide inclusive prefix of the quad-group counts
-                const uint32_t pair = nq2[0] + nq2[1];
-                uint32_t x = pair;
-#pragma unroll
-                for (int d = 1; d < 32; d <<= 1) {
-                    const uint32_t y = __shfl_up_sync(kFull, x, d);
-                    if (lane >= d) x += y;
-                }
-                if (lane == 31) s_wsum[wid] = x;
-                __syncthreads();
-                // every thread reads the hub count between these two barriers,
-                // and it is cleared after the second, before any thread can
-                // classify the next window's rows
-                nhub = s_nhub;
-                if (wid == 0) {
-                    uint32_t w = lane < kWarps ? s_wsum[lane] : 0u;
-#pragma unroll
-                    for (int d = 1; d < 32; d <<= 1) {
-                        const uint32_t y = __shfl_up_sync(kFull, w, d);
-                        if (lane >= d) w += y;
-                    }
-                    if (lane < kWarps) s_wsum[lane] = w;
-                }
-                __syncthreads();
-                if (threadIdx.x == 0) s_nhub = 0;
-                const uint32_t before = (wid ? s_wsum[wid - 1] : 0u) + x - pair;
-                if (2u * threadIdx.x < nw) s_pre[2u * threadIdx.x] = before + nq2[0];
-                if (2u * threadIdx.x + 1 < nw) s_pre[2u * threadIdx.x + 1] = before + pair;
-                __syncthreads();
-                total = s_pre[nw - 1];
-                }
-                const uint32_t grp = 1u << gsh;
-                // quad group g (nothing when g is past the window): quads q ..
-                // q + grp - 1 of one row, independent Philox blocks; a
-                // quad inside the row skips the edge bounds. Returns the live
-                // edges as a bit mask (bit 4h + k: edge k of quad q + h).
-                auto draw = [&](uint32_t g, uint32_t* q_out) -> unsigned {
-                    *q_out = 0;
-                    if (g >= total) return 0u;
-                    uint32_t i = 0;  // the row of group g: entries with prefix <= g
-                    // (steps from the window's own size: a lone hub row needs none)
-                    for (uint32_t b = nw > 1 ? 1u << (31 - __clz(nw - 1)) : 0u; b; b >>= 1)
-                        if (i + b - 1 < nw && s_pre[i + b - 1] <= g) i += b;
-                    const uint32_t lo = s_lo[i], hi = s_hi[i], tr = s_tau[i];
-                    const uint32_t q = (lo >> 2) + ((g - (i ? s_pre[i - 1] : 0u)) << gsh);
-                    const uint32_t q_last = (hi - 1) >> 2;
-                    *q_out = q;
-                    unsigned live = 0;
-#pragma unroll
-                    for (int h = 0; h < kCtaGroup; ++h) {
-                        const uint32_t qh = q + h;
-                        if ((uint32_t)h >= grp || qh > q_last) break;
-                        const uint4 x = coin_block(a.rk, qh, 0, kDomBfs, j);
-                        const uint4 t4 = a.tau ? __ldg(reinterpret_cast<const uint4*>(a.tau) + qh)
-                                               : make_uint4(tr, tr, tr, tr);
-                        const uint32_t e0 = qh << 2;
-                        unsigned l4 = 0;
-                        if (e0 >= lo && e0 + 4 <= hi) {
-                            l4 |= coin_live(x.x, t4.x) ? 1u : 0u;
-                            l4 |= coin_live(x.y, t4.y) ? 2u : 0u;
-                            l4 |= coin_live(x.z, t4.z) ? 4u : 0u;
-                            l4 |= coin_live(x.w, t4.w) ? 8u : 0u;
-                        } else {
-                            l4 |= (e0 + 0 >= lo && e0 + 0 < hi && coin_live(x.x, t4.x)) ? 1u : 0u;
-                            l4 |= (e0 + 1 >= lo && e0 + 1 < hi && coin_live(x.y, t4.y)) ? 2u : 0u;
-                            l4 |= (e0 + 2 >= lo && e0 + 2 < hi && coin_live(x.z, t4.z)) ? 4u : 0u;
-                            l4 |= (e0 + 3 >= lo && e0 + 3 < hi && coin_live(x.w, t4.w)) ? 8u : 0u;
+                // hub rows: their chunks of 64 quads laid end to end and cut into one
+                // run a warp, so a warp goes straight down a row with no search,
+                // two independent blocks a lane and step. For one threshold a row
+                // (never the sentinel: a hub has many edges) a step is one compare
+                // of the blocks' minimum, as a live coin is rare there (weighted
+                // cascade expects one a row)
+                const uint32_t per = (chunks + kWarps - 1) / kWarps, run0 = wid * per;
+                const uint32_t run1 = run0 < chunks ? min(chunks, run0 + per) : 0u;
+                uint32_t before = 0;  // chunks of the hubs before h
+#pragma unroll 1
+                for (uint32_t h = 0; h < nhub && before < run1; ++h) {
+                    const uint4 w = win[hubs[h]];
+                    const uint32_t lo = w.x, hi = w.y, tr = w.z, nq = row_quads(lo, hi), n = (nq + 63) / 64;
+                    const uint32_t c0 = max(run0, before) - before, c1 = min(run1, before + n) - before;
+                    const bool mine = run0 < before + n;
+                    before += n;
+                    if (!mine) continue;
+                    uint32_t q = (lo >> 2) + 64 * c0 + lane;  // this lane's quads: q and q + 32
+                    const uint32_t qe = (lo >> 2) + nq;
+                    // the live coins of one step join the list (quads past the row's end dropped)
+                    auto draw = [&]() {
+                        const uint4 tr4 = make_uint4(tr, tr, tr, tr);
+#pragma unroll 1
+                        for (uint32_t k = 0; k < 64 && q - lane + k < qe; k += 32) {
+                            const uint32_t qk = q + k;
+                            const uint4 x = blk(qk, a.rk);
+                            if (!tau4 && !__any_sync(kFull, min4(x) < tr)) continue;
+                            unsigned live = 0;
+                            if (qk < qe) live = quad_live(qk, x, tau4 ? __ldg(tau4 + qk) : tr4, lo, hi);
+                            list(qk, live);
                         }
-                        live |= l4 << (4 * h);
-                    }
-                    return live;
-                };
-                // one group (32 grp quads) per warp step; the
-                // sources of live edges are loaded only when some lane has one
-                for (uint32_t c = wid; c * 32u < total; c += kWarps) {
-                    uint32_t q;
-                    const unsigned live = draw(c * 32u + lane, &q);
-                    if (!__any_sync(kFull, live != 0u)) continue;
-#pragma unroll
-                    for (int h = 0; h < kCtaGroup; ++h) {
-                        const unsigned lh = (live >> (4 * h)) & 15u;
-                        if (!__any_sync(kFull, lh != 0u)) continue;
-                        int4 s4 = make_int4(-1, -1, -1, -1);
-                        if (lh) s4 = __ldg(reinterpret_cast<const int4*>(a.src) + q + h);
-                        const int32_t cand[4] = {s4.x, s4.y, s4.z, s4.w};
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const int32_t u = ((lh >> k) & 1u) ? cand[k] : -1;
-                            if (__any_sync(kFull, u >= 0)) ins.insert(u);
-                        }
-                    }
-                }
-                // hub rows: their quads laid end to end and strided over the
-                // block, so a thread runs straight down a row with no search
-                // and no per-edge bounds; a live coin is rare there (WC: one
-                // expected per row) and is inserted by its lane alone
-                if (nhub) {
-                    const SampleBlock blk(a.rk, j, kDomBfs);
-                    const uint4* __restrict__ tau4 = reinterpret_cast<const uint4*>(a.tau);
-                    // the live coins of quad q (Philox block x) within [lo, hi) join the sample
-                    auto take = [&](uint32_t q, const uint4& x, const uint4& t4, uint32_t lo, uint32_t hi) {
-                        const uint32_t e0 = q << 2;
-                        unsigned l4 = 0;
-                        l4 |= (e0 + 0 >= lo && e0 + 0 < hi && coin_live(x.x, t4.x)) ? 1u : 0u;
-                        l4 |= (e0 + 1 >= lo && e0 + 1 < hi && coin_live(x.y, t4.y)) ? 2u : 0u;
-                        l4 |= (e0 + 2 >= lo && e0 + 2 < hi && coin_live(x.z, t4.z)) ? 4u : 0u;
-                        l4 |= (e0 + 3 >= lo && e0 + 3 < hi && coin_live(x.w, t4.w)) ? 8u : 0u;
-                        if (l4) {
-                            const int4 s4 = __ldg(reinterpret_cast<const int4*>(a.src) + q);
-                            if (l4 & 1u) cta_insert_one(bitmap, queue, &s_qlen, a.queue_cap, s4.x);
-                            if (l4 & 2u) cta_insert_one(bitmap, queue, &s_qlen, a.queue_cap, s4.y);
-                            if (l4 & 4u) cta_insert_one(bitmap, queue, &s_qlen, a.queue_cap, s4.z);
-                            if (l4 & 8u) cta_insert_one(bitmap, queue, &s_qlen, a.queue_cap, s4.w);
-                        }
+                        q += 64;
                     };
-                    auto min4 = [](const uint4& x) { return min(min(x.x, x.y), min(x.z, x.w)); };
-                    uint32_t g = threadIdx.x;
-                    for (uint32_t h = 0; h < nhub; ++h) {
-                        const uint32_t i = s_hub[h];
-                        const uint32_t lo = s_lo[i], hi = s_hi[i], tr = s_tau[i];
-                        const uint32_t qf = lo >> 2, nq = ((hi - 1) >> 2) - qf + 1;
+                    uint32_t full = max(c0, min(c1, nq / 64)) - c0;  // steps without a ragged end
+#pragma unroll 1
+                    while (full) {
                         if (!tau4) {
-                            // one threshold for the row (never the sentinel: a hub row has many
-                            // edges): two independent blocks a step, one compare of their minimum
-                            const uint4 tr4 = make_uint4(tr, tr, tr, tr);
-                            for (; g + kCtaThreads < nq; g += 2 * kCtaThreads) {
-                                const uint32_t q0 = qf + g, q1 = q0 + kCtaThreads;
-                                const uint4 x0 = blk(q0, a.rk), x1 = blk(q1, a.rk);
-                                if (min(min4(x0), min4(x1)) < tr || tr == kSentinel) {
-                                    take(q0, x0, tr4, lo, hi);
-                                    take(q1, x1, tr4, lo, hi);
-                                }
-                            }
-                            for (; g < nq; g += kCtaThreads) {
-                                const uint32_t q = qf + g;
-                                const uint4 x = blk(q, a.rk);
-                                if (min4(x) < tr || tr == kSentinel) take(q, x, tr4, lo, hi);
-                            }
+                            // nothing but blocks and the compare until a lane may have a
+                            // live coin, whose step is then drawn again
+                            bool hit;
+                            do {
+                                hit = __any_sync(kFull, min8(blk(q, a.rk), blk(q + 32, a.rk)) < tr);
+                                q += 64;
+                                --full;
+                            } while (!hit && full);
+                            if (!hit) break;
+                            q -= 64;
                         } else {
-                            for (; g < nq; g += kCtaThreads) {
-                                const uint32_t q = qf + g;
-                                const uint4 x = blk(q, a.rk);
-                                const uint4 t4 = __ldg(tau4 + q);
-                                if (coin_live(x.x, t4.x) | coin_live(x.y, t4.y) | coin_live(x.z, t4.z) |
-                                    coin_live(x.w, t4.w))
-                                    take(q, x, t4, lo, hi);
-                            }
+                            --full;
                         }
-                        g -= nq;
+                        draw();
                     }
+                    if (c1 == n && nq % 64) draw();
                 }
-                __syncthreads();  // the window's shared arrays are reused
             }
-            head = tail;
-            tail = s_qlen;  // after the level's last barrier: every insert of the level is in
+            if (npend) join(npend);
         }
+        const uint32_t len = tail;
         coins = warp_sum_u64(coins);
         if (lane == 0 && coins) atomicAdd(&s_coins, (unsigned long long)coins);
         __syncthreads();
-        const uint32_t len = s_qlen;
         const bool outgrown = len > a.queue_cap;  // the queue kept its first queue_cap members only
         if (threadIdx.x == 0) {
             const unsigned long long base = outgrown ? 0ull : atomicAdd(a.arena_cursor, (unsigned long long)len);
