@@ -116,8 +116,8 @@ typedef struct skis_stats {
  * (up to 32 members, in-rows up to THREAD_MAX_DEG edges, up to
  * THREAD_MAX_STEPS edge quads, up to THREAD_MAX_RETRIES rejected rounds;
  * the "thread" names below refer to this tier), one warp per sample (up to
- * 1536 members, the first 256 in shared memory; up to WARP_MAX_COINS
- * in-edges), one CTA per sample (any size). Options tune the split; they
+ * 1536 members, 4096 on graphs of 24,576 vertices and more, the first 256 in
+ * shared memory; up to WARP_MAX_COINS in-edges), one CTA per sample (any size). Options tune the split; they
  * never change the samples. */
 typedef enum skis_option {
     SKIS_OPT_RETRY_CAP = 0,      /* cap on rejected first-step rounds (default 2^24) */

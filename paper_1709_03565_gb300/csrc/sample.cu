@@ -12,7 +12,7 @@
 //
 // Warp tier: one warp per sample. The member list (256 entries) and an
 // open-addressing hash set (the visited set R_j) live in shared memory; a
-// larger sample moves to the warp's slot in global memory (up to 1536
+// larger sample moves to the warp's slot in global memory (1536 or 4096
 // members). Edges of up to 32 queued vertices are spread over the lanes one
 // edge quad at a time. A sample that outgrows it is handed, by id, to the CTA
 // tier.
@@ -36,9 +36,17 @@ constexpr int kQCap = 256;         // warp-tier members held in shared memory
 constexpr int kHashBits = 9;
 constexpr int kHCap = 1 << kHashBits;  // their hash slots (load <= 1/2 + one insert round)
 constexpr int kIdBatch = 16;       // most sample ids a warp takes per work-cursor atomic
-constexpr int kSpillCap = 1536;    // warp-tier members in all: past kQCap in the warp's global spill slot
-constexpr int kSpillHashBits = 12;
-constexpr int kSpillHash = 1 << kSpillHashBits;  // its hash slots (load under 2/5)
+// Members a sample may have in the warp tier, past kQCap in the warp's global
+// spill slot, and the slot's hash bits (load at most 1/2). The longest samples
+// that are still narrow (a few rows a level) belong here, where 32 of them
+// share an SM, and not on the CTA tier, where four do: on Chung-Lu 1M / 17.5M
+// WC (levels of 13 rows) the two tiers take 10.6 ms with 1536 members and
+// 7.5 ms with 4096. A sample that holds a sixth of the graph has levels wide
+// enough for a block, so a small graph keeps the smaller slot.
+struct SpillSize {
+    uint32_t cap, hash_bits;
+};
+inline SpillSize spill_size(int64_t n) { return n >= 6 * 4096 ? SpillSize{4096, 13} : SpillSize{1536, 12}; }
 constexpr int kRing = 64;          // queued members whose in-rows wait in shared memory
 constexpr int kPend = 32 + 128;    // live edges waiting for an insert round: under 32, plus one quad a lane
 // entries reserved per arena atomic; once a warp's reservation did not fit it
@@ -96,9 +104,10 @@ struct SampleArgs {
     const uint4* up_rec;
     const uint2* up_pick;
     uint64_t up_first, up_count;
-    // warp tier: a spill slot a warp, kSpillHash table words and kSpillCap members
+    // warp tier: a spill slot a warp, 2^hash_bits table words and cap members
     uint32_t* spill_hash;
     int32_t* spill_queue;
+    SpillSize spill;
 };
 
 
@@ -192,7 +201,7 @@ __device__ __forceinline__ uint32_t source_of(const SampleArgs& a, uint64_t j, R
 // Warp tier: the members of the warp's sample (which are also its BFS queue)
 // and their hash set. Up to kQCap members live in shared memory; a larger
 // sample moves both to the warp's spill slot in global memory (L2) and goes
-// on there, up to kSpillCap members. A candidate's in-row is loaded while its
+// on there, up to spill.cap members. A candidate's in-row is loaded while its
 // hash slot is probed, and kept in a shared ring if it joins within kRing
 // places of the queue's head, so that a pop finds the row without going
 // through the queue and the row table (a chain of two memory latencies per
@@ -204,6 +213,7 @@ struct WarpInserter {
     uint32_t* ghash;  // the spill slot
     int32_t* gqueue;
     const RowInfo* rows;
+    SpillSize spill;
     uint32_t qlen, head;
     bool big;         // the sample lives in the spill slot
     bool overflow;
@@ -222,14 +232,14 @@ struct WarpInserter {
         return put(hash, (u * 2654435761u) >> (32 - kHashBits), kHCap - 1, u);
     }
     __device__ __forceinline__ bool put_spill(uint32_t u) {
-        return put(ghash, (u * 2654435761u) >> (32 - kSpillHashBits), kSpillHash - 1, u);
+        return put(ghash, (u * 2654435761u) >> (32 - spill.hash_bits), (1u << spill.hash_bits) - 1, u);
     }
 
     // The sample outgrew shared memory: its members (qlen of them, and the
     // lanes' fresh ones) go to the spill slot, whose table is cleared first.
-    __device__ __forceinline__ void spill(int32_t u, bool fresh) {
+    __device__ __forceinline__ void move(int32_t u, bool fresh) {
         const int lane = threadIdx.x & 31;
-        for (int i = lane; i < kSpillHash / 4; i += 32)
+        for (uint32_t i = lane; i < (1u << spill.hash_bits) / 4; i += 32)
             reinterpret_cast<uint4*>(ghash)[i] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
         __syncwarp();
         for (uint32_t i = lane; i < qlen; i += 32) {
@@ -254,8 +264,8 @@ struct WarpInserter {
         if (m) {
             const uint32_t pos = qlen + __popc(m & lanemask_lt());
             const uint32_t len = qlen + __popc(m);
-            if (len > (uint32_t)kQCap && !big) spill(u, fresh);
-            if (len > (uint32_t)kSpillCap) {
+            if (len > (uint32_t)kQCap && !big) move(u, fresh);
+            if (len > spill.cap) {
                 overflow = true;
             } else if (fresh) {
                 if (big) gqueue[pos] = u;
@@ -750,11 +760,9 @@ __global__ void __launch_bounds__(kLaneBlock, 4) k_iis_lane(SampleArgs a) {
 // the source gather, the probe and the row load of 32 candidates overlap and
 // an insert round has every lane busy.
 // Two thirds of a weighted-cascade sketch's members lie in samples of more
-// than 256 members, so the tier goes on past shared memory: the spill slots
-// of 1536 members keep all but 1 in 130 samples of Chung-Lu 1M / 17.5M off
-// the CTA tier, which pays block barriers on every narrow level (100 us and
-// more a sample). On 1M samples of that graph this tier and the CTA tier
-// took 29 ms when samples left here at 256 members and 13.5 ms now.
+// than 256 members, so the tier goes on past shared memory. On 1M samples of
+// Chung-Lu 1M / 17.5M WC this tier and the CTA tier took 29 ms when samples
+// left here at 256 members and 7.5 ms now.
 __global__ void __launch_bounds__(kWarpThreads, 4) k_iis_warp(SampleArgs a) {
     __shared__ __align__(16) uint32_t s_hash[kWarpThreads / 32][kHCap];
     __shared__ __align__(16) int32_t s_queue[kWarpThreads / 32][kQCap];
@@ -794,8 +802,8 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_iis_warp(SampleArgs a) {
             int64_t pe;
             int32_t pu;
             const uint32_t v = source_of(a, j, &rv, &pe, &pu);
-            WarpInserter ins{hash, s_queue[wib], s_ring[wib], a.spill_hash + wid * kSpillHash,
-                             a.spill_queue + wid * kSpillCap, a.rows, 1u, 1u, false, false};
+            WarpInserter ins{hash, s_queue[wib], s_ring[wib], a.spill_hash + (wid << a.spill.hash_bits),
+                             a.spill_queue + wid * a.spill.cap, a.rows, a.spill, 1u, 1u, false, false};
             if (lane == 0) {
                 ins.put_shared(v);
                 s_queue[wib][0] = (int32_t)v;
@@ -1654,8 +1662,8 @@ static int ensure_sample_buffers(skis_sketch* s, uint64_t count, uint64_t slack,
         s->spill_hash = nullptr;
         s->spill_queue = nullptr;
         s->spill_warps = 0;
-        SK_CUDA(dev_alloc_t(&s->spill_hash, (size_t)(warps * kSpillHash), st));
-        SK_CUDA(dev_alloc_t(&s->spill_queue, (size_t)(warps * kSpillCap), st));
+        SK_CUDA(dev_alloc_t(&s->spill_hash, (size_t)(warps << spill_size(g->n).hash_bits), st));
+        SK_CUDA(dev_alloc_t(&s->spill_queue, (size_t)(warps * spill_size(g->n).cap), st));
         s->spill_warps = warps;
     }
     // CTA-tier slots: an n-bit visited bitmap and a queue of min(n, cta_queue_cap)
@@ -1784,6 +1792,7 @@ int sketch_sample(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* 
     base.lt_cum = g->lt_cum;
     base.spill_hash = s->spill_hash;
     base.spill_queue = s->spill_queue;
+    base.spill = spill_size(g->n);
     // per-vertex member counts, kept while they describe exactly samples
     // [0, T): invalid until this call succeeds
     const bool counting = s->vcount_ok && s->vcount_T == s->T;

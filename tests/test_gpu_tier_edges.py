@@ -1,6 +1,7 @@
 """Samples whose sizes and shapes sit at the edges of the deeper sampling tiers: every edge is live, so a sample is its
-source's ancestor set and its size is known. The warp tier keeps 256 members in shared memory and 1536 in all, batches
-32 rows and joins 32 live edges at a time; the CTA tier holds 512 rows of a level in shared memory. All against the
+source's ancestor set and its size is known. The warp tier keeps 256 members in shared memory and 1536 in all (4096 on
+graphs of 24,576 vertices and more), batches 32 rows and joins 32 live edges at a time; the CTA tier holds 512 rows of
+a level in shared memory. All against the
 oracle, sample by sample (integers and sets: equal)."""
 import numpy as np
 import pytest
@@ -39,26 +40,28 @@ TIERS = {"default": {}, "warp": {skis.SKIS_OPT_THREAD_MAX_DEG: 0},
 
 
 @pytest.mark.parametrize("tier", sorted(TIERS))
-@pytest.mark.parametrize("shape,n", [("star", 33), ("star", 257), ("star", 258), ("star", 1536), ("star", 1537),
-                                     ("path", 300), ("path", 1600), ("tree", 256), ("tree", 1537), ("broom", 1027),
-                                     ("broom", 2501)])
+@pytest.mark.parametrize("shape,size,n", [
+    ("star", 33, 33), ("star", 257, 257), ("star", 258, 258), ("star", 1536, 1536), ("star", 1537, 1537),
+    ("path", 300, 300), ("path", 1600, 1600), ("tree", 256, 256), ("tree", 1537, 1537), ("broom", 1027, 1027),
+    ("broom", 2501, 2501), ("star", 1537, 24_575), ("star", 4096, 24_576), ("star", 4097, 24_576),
+    ("broom", 4095, 24_576), ("broom", 4097, 24_576), ("path", 1700, 24_576)])
 @pytest.mark.parametrize("bucket", [False, True])
-def test_sizes_at_the_tiers_edges(shape, n, tier, bucket):
+def test_sizes_at_the_tiers_edges(shape, size, n, tier, bucket):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
-    src, dst = (np.ascontiguousarray(x, dtype=np.int32) for x in SHAPES[shape](n))
+    src, dst = (np.ascontiguousarray(x, dtype=np.int32) for x in SHAPES[shape](size))
     tau = np.full(len(src), 0xFFFFFFFF, np.uint32)
     g = skis.skis_load_graph(n, src, dst, tau, skis.SKIS_W_EXPLICIT_TAU)
     o = oracle.OracleGraph(n, src, dst, weights=tau, model=oracle.W_TAU)
-    T, seed = 2000, 0xED6E + n
+    T, seed = 2000, 0xED6E + size
     s = skis.skis_sketch_create(g, seed)
     skis.skis_sketch_set_option(s, skis.SKIS_OPT_FIRST_STEP, 1 if bucket else 0)
     for k, v in TIERS[tier].items():
         skis.skis_sketch_set_option(s, k, v)
     skis.skis_sample(s, T)
     ora = o.sample_ids(seed, np.arange(T, dtype=np.uint64), bucket=bucket)
-    assert shape not in ("star", "path") or ora["len"].max() >= n - 4  # a sample of (nearly) all vertices is among them
+    assert shape not in ("star", "path") or ora["len"].max() >= size - 4  # a sample of (nearly) everything is among them
     assert_samples_equal(skis.skis_sketch_export(s, 0, T), ora)
     s.close()
     g.close()
