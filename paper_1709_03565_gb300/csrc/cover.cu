@@ -11,8 +11,6 @@
 // coverage Delta_v, then per round an exact argmax of the integer key
 // Delta_v W + T (2^f - w_v) (ties to the lowest id), and the samples of the
 // chosen vertex are marked covered and their members' Delta decremented.
-#include <cooperative_groups.h>
-
 #include <algorithm>
 #include <string>
 
@@ -89,23 +87,18 @@ __device__ __forceinline__ void add_aggregated(uint32_t* counter, int32_t u, int
 
 // Greedy's cover walk: a block-local table merges the decrements of vertices
 // that recur across the samples a seed covers (hubs), so that each such
-// vertex takes one global atomic per block and round instead of one per
-// warp step. A vertex that finds its slot held by another goes straight to
-// the global counter.
+// vertex takes one global atomic per block and round. A vertex that finds its
+// slot held by another goes straight to the global counter.
 constexpr int kHotBits = 10;
 constexpr int kHotSlots = 1 << kHotBits;
 constexpr uint32_t kHotEmpty = 0xFFFFFFFFu;
 
 __device__ __forceinline__ void sub_merged(uint32_t* counter, int32_t u, uint32_t* hkey, uint32_t* hcnt) {
-    const unsigned active = __activemask();
-    const unsigned peers = __match_any_sync(active, u);
-    if ((threadIdx.x & 31) != __ffs(peers) - 1) return;
-    const uint32_t c = (uint32_t)__popc(peers);
     const uint32_t slot = ((uint32_t)u * 2654435761u) >> (32 - kHotBits);
     uint32_t old = hkey[slot];
     if (old == kHotEmpty) old = atomicCAS(&hkey[slot], kHotEmpty, (uint32_t)u);
-    if (old == kHotEmpty || old == (uint32_t)u) atomicAdd(&hcnt[slot], c);
-    else atomicSub(&counter[u], c);
+    if (old == kHotEmpty || old == (uint32_t)u) atomicAdd(&hcnt[slot], 1u);
+    else atomicSub(&counter[u], 1u);
 }
 
 // ------------------------------------------------------------- coverage
@@ -760,17 +753,6 @@ __device__ __forceinline__ KeyId shfl_down_keyid(const KeyId& x, int d) {
     return y;
 }
 
-__device__ __forceinline__ KeyId shfl_keyid(const KeyId& x, int src) {
-    KeyId y;
-    y.key = ((u128)__shfl_sync(kFull, (unsigned long long)(x.key >> 64), src) << 64) |
-            (u128)__shfl_sync(kFull, (unsigned long long)x.key, src);
-    y.id = __shfl_sync(kFull, x.id, src);
-    y.valid = __shfl_sync(kFull, x.valid, src);
-    y.d = __shfl_sync(kFull, x.d, src);
-    y.pad = 0;
-    return y;
-}
-
 __device__ KeyId block_best(KeyId b, KeyId* s_part) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
 #pragma unroll
@@ -791,12 +773,60 @@ __device__ KeyId block_best(KeyId b, KeyId* s_part) {
     return b;  // valid in thread 0
 }
 
+// One candidate of the greedy argmax: the exact key Delta W + T (2^f - w)
+// (below 2^94: T < 2^32, W <= 2^61) in three words, the vertex (~0: none),
+// its Delta, and its inverted list where the holder knows it.
+struct __align__(16) Cand {
+    uint32_t k2, k1, k0, id;
+    uint32_t d, cnt;
+    uint64_t lo;
+};
+constexpr uint32_t kNone = 0xFFFFFFFFu;
+
+__device__ __forceinline__ Cand no_cand() { return Cand{0, 0, 0, kNone, 0, 0, 0}; }
+
+__device__ __forceinline__ bool cand_better(const Cand& a, const Cand& b) {  // larger key, then lower id
+    if (a.k2 != b.k2) return a.k2 > b.k2;
+    if (a.k1 != b.k1) return a.k1 > b.k1;
+    if (a.k0 != b.k0) return a.k0 > b.k0;
+    return a.id < b.id;
+}
+
+// The lane that holds the warp's best candidate, by word-wise reductions.
+__device__ __forceinline__ int warp_best_lane(const Cand& c) {
+    const uint32_t m2 = __reduce_max_sync(kFull, c.k2);
+    bool e = c.k2 == m2;
+    const uint32_t m1 = __reduce_max_sync(kFull, e ? c.k1 : 0u);
+    e = e && c.k1 == m1;
+    const uint32_t m0 = __reduce_max_sync(kFull, e ? c.k0 : 0u);
+    e = e && c.k0 == m0;
+    const uint32_t id = __reduce_min_sync(kFull, e ? c.id : kNone);
+    return __ffs(__ballot_sync(kFull, e && c.id == id)) - 1;
+}
+
+__device__ __forceinline__ Cand ldcg_cand(const Cand* p) {
+    const uint4* q = reinterpret_cast<const uint4*>(p);
+    const uint4 x = __ldcg(q), y = __ldcg(q + 1);
+    return Cand{x.x, x.y, x.z, x.w, y.x, y.y, (uint64_t)y.z | ((uint64_t)y.w << 32)};
+}
+
+// Control words of one greedy call, zero at its start.
+struct GreedyCtl {
+    unsigned int arrived;  // grid barrier arrivals
+    unsigned int pool_n;
+    unsigned int gave_up;  // a barrier wait ran out (it cannot while every block runs)
+    unsigned int pad[29];
+    unsigned int reached;  // the last grid barrier that every block arrived at, on a line of its own
+    unsigned int pad2[31];
+};
+
 struct GreedyArgs {
     const uint64_t* w;
     uint8_t* inS;
     uint32_t* delta;
     int64_t n;
     uint64_t W, T;
+    double ratio;     // T / W, for the pool's buckets
     int f;
     int32_t k;
     const uint64_t* inv_off;
@@ -805,53 +835,145 @@ struct GreedyArgs {
     const uint32_t* h_len;
     const int32_t* arena;
     uint32_t* covered;
-    KeyId* partial;
-    KeyId* seg_best;  // per segment of kGreedySeg vertices: its best of the last scan
+    Cand* partial;
+    Cand* seg_best;   // per segment of kGreedySeg vertices: its best of the last scan
     int64_t nseg;
+    uint32_t* pool;   // kGreedyThreads vertices
+    uint32_t* hist;   // kBuckets counters of the vertices by rounded key (k_greedy_init)
+    GreedyCtl* ctl;
     int32_t* seeds;
     int64_t* cov_out;
     double* est_out;
     int ris;
 };
 
-
-__device__ __forceinline__ KeyId ldcg_keyid(const KeyId* p) {
-    const unsigned long long* q = reinterpret_cast<const unsigned long long*>(p);
-    KeyId c;
-    c.key = ((u128)__ldcg(q + 1) << 64) | (u128)__ldcg(q);
-    const unsigned long long tail = __ldcg(q + 2);
-    c.id = (uint32_t)tail;
-    c.valid = (uint32_t)(tail >> 32);
-    c.d = (uint32_t)__ldcg(q + 3);
-    c.pad = 0;
-    return c;
-}
-
-// All k rounds of Alg. 3 in one cooperative launch, one block per SM. Per
-// round: every block scans its share of the vertices for the exact key
-// Delta_v W + T (2^f - w_v) (v outside S, ties to the lowest id) and writes
-// its best; a grid barrier; every block reduces all the blocks' bests itself
-// (the same winner everywhere, no atomic hand-off) and block 0 records it;
-// every warp walks the winner's inverted list, marking uncovered samples and
-// decrementing their members' Delta (hub decrements merged per block); a grid
-// barrier. Every block executes the same sequence of barriers. Data that
-// other blocks change during the launch (Delta, the block bests) is read
-// through L2 (ld.global.cg), never from a possibly stale L1 line.
+// All k rounds of Alg. 3 in one cooperative launch, one block per SM. A round
+// is a chain of memory latencies and grid barriers far more than it is work,
+// so:
+//   - The argmax comes from a pool: the vertices outside S with the largest
+//     keys, up to one a thread, which every block holds alike, and the exact
+//     best key outside the pool. Keys only decrease, so while the pool's best
+//     beats that bound it is the argmax (ties to the lowest id), and every
+//     block finds it by itself, with no exchange. When it no longer does, the
+//     pool is refilled from all vertices (a histogram of rounded keys picks
+//     how far down it goes; membership decides nothing but speed).
+//   - Where too many vertices tie for a pool, rounds scan segments of 256
+//     vertices instead: a segment whose best is still outside S with an
+//     unchanged Delta keeps it, the others are rescanned, one warp each.
+//   - A block may change Delta only after every block has read it; that grid
+//     barrier is entered before the walk and left after the walk's first
+//     loads (list, covered bits, headers), which do not touch Delta.
+//   - The walk: a thread takes an entry of the winner's inverted list, and the
+//     members of the block's uncovered samples are dealt to its threads end
+//     to end, whatever their sizes.
+// Data that other blocks change during the launch is read through L2
+// (ld.global.cg), never from a possibly stale L1 line.
+// Chung-Lu 1M / 17.5M WC, 1M samples, k = 1000: 20 -> 8 ms, 8 us a round, of
+// which the grid barrier at its end 3 us, the argmax 1.8 us, the list and the
+// headers 1.7 us, the members 1.2 us (the argmax over the segments with two
+// grid barriers a round, each list run of 32 entries on one warp, before).
 constexpr int kGreedyThreads = 1024;
 constexpr int kGreedySegLog = 8;  // vertices per segment: 256
 constexpr int64_t kGreedySeg = 1ll << kGreedySegLog;
-constexpr uint32_t kBigLen = 256;   // covered samples longer than this are walked by the whole block
-constexpr int kBigQueue = 64;
+constexpr int kBuckets = 8192;           // exponent and five mantissa bits of a rounded key / W
+constexpr uint32_t kPoolMin = 64;        // a smaller pool does not pay for its refill
+constexpr uint32_t kSegRounds = 64;      // segment rounds before a pool is tried again
+constexpr unsigned int kBarSpins = 1u << 23;  // polls of a grid barrier before giving up (~10 s)
+
+// key / W, rounded: where a vertex stands in the pool's histogram
+__device__ __forceinline__ uint32_t greedy_bucket(uint32_t d, uint64_t gap, double ratio, int ris) {
+    const float x = ris ? (float)d : (float)((double)d + (double)gap * ratio);
+    return __float_as_uint(x) >> 18;
+}
+
+// Delta_R(v, {}) = number of samples containing v = length of v's list, and
+// the histogram of the first pool.
+__global__ void __launch_bounds__(kGreedyThreads) k_greedy_init(GreedyArgs a) {
+    __shared__ uint32_t s_hist[kBuckets];
+    for (int i = threadIdx.x; i < kBuckets; i += kGreedyThreads) s_hist[i] = 0;
+    __syncthreads();
+    const int64_t stride = (int64_t)gridDim.x * kGreedyThreads;
+    for (int64_t v0 = (int64_t)blockIdx.x * kGreedyThreads + (threadIdx.x & ~31); v0 < a.n; v0 += stride) {
+        const int64_t v = v0 + (threadIdx.x & 31);
+        uint32_t b = kBuckets;
+        if (v < a.n) {
+            const uint32_t d = (uint32_t)(a.inv_off[v + 1] - a.inv_off[v]);
+            a.delta[v] = d;
+            b = greedy_bucket(d, (1ull << a.f) - a.w[v], a.ratio, a.ris);
+        }
+        // most vertices share a few low buckets: one atomic a warp for each
+        const unsigned peers = __match_any_sync(kFull, b);
+        if (b < kBuckets && (threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&s_hist[b], (uint32_t)__popc(peers));
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kBuckets; i += kGreedyThreads)
+        if (s_hist[i]) atomicAdd(&a.hist[i], s_hist[i]);
+}
+
+// Grid barrier in two halves (the grid is launched cooperatively): an arrival
+// is one atomic a block, the last of them publishes the barrier's number, and
+// one thread a block polls that word. Few pollers and no sequentially
+// consistent fence: with every block polling a word of every other, or with
+// __threadfence() at each end, a barrier took 9,000 to 17,000 cycles, with the
+// cooperative-groups one 9,000, with this one 5,900 (800 where the walk's
+// first loads hide it).
+struct GridBar {
+    GreedyCtl* ctl;
+    uint32_t* failed;  // shared
+    uint32_t goal;
+
+    // After a block barrier. ordered: the block's writes before it are seen by
+    // the other blocks after their wait (else only its reads are over).
+    __device__ __forceinline__ void arrive(bool ordered) {
+        ++goal;
+        if (threadIdx.x != 0) return;
+        uint32_t old;
+        if (ordered) {
+            asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(&ctl->arrived) : "memory");
+            if (old + 1u == goal * gridDim.x)
+                asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&ctl->reached), "r"(goal) : "memory");
+        } else {
+            asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(&ctl->arrived) : "memory");
+            if (old + 1u == goal * gridDim.x)
+                asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(&ctl->reached), "r"(goal) : "memory");
+        }
+    }
+    // false: the wait ran out
+    __device__ __forceinline__ bool wait(bool ordered) {
+        if (threadIdx.x == 0) {
+            uint32_t x;
+            for (uint32_t spins = 0;;) {
+                if (ordered)
+                    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(&ctl->reached) : "memory");
+                else
+                    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(&ctl->reached) : "memory");
+                if ((int)(x - goal) >= 0) break;
+                if (++spins > kBarSpins) {
+                    atomicOr(&ctl->gave_up, 1u);
+                    *failed = 1;
+                    break;
+                }
+            }
+        }
+        __syncthreads();
+        return *failed == 0;
+    }
+    __device__ __forceinline__ bool sync() {
+        __syncthreads();
+        arrive(true);
+        return wait(true);
+    }
+};
 
 __global__ void __launch_bounds__(kGreedyThreads, 1) k_greedy_rounds(GreedyArgs a) {
-    namespace cg = cooperative_groups;
-    cg::grid_group grid = cg::this_grid();
-    __shared__ KeyId s_part[kGreedyThreads / 32];
-    __shared__ KeyId s_win;
+    __shared__ Cand s_part[2][kGreedyThreads / 32];
+    __shared__ __align__(16) uint32_t s_hist[kBuckets];  // a refill's histogram, or
+    uint64_t* const s_off = reinterpret_cast<uint64_t*>(s_hist);  // the walk's samples: arena offset,
+    uint64_t* const s_end = s_off + kGreedyThreads;               // and members of the block up to its end
+    static_assert(kBuckets * sizeof(uint32_t) >= 2 * kGreedyThreads * sizeof(uint64_t), "the walk's arrays fit");
     __shared__ uint32_t s_hkey[kHotSlots], s_hcnt[kHotSlots];
-    __shared__ uint64_t s_big_off[kBigQueue];
-    __shared__ uint32_t s_big_len[kBigQueue];
-    __shared__ uint32_t s_nbig;
+    __shared__ uint64_t s_wsum[kGreedyThreads / 32];
+    __shared__ uint32_t s_cut, s_failed;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const uint64_t one_f = 1ull << a.f;
     const int nw = kGreedyThreads / 32;
@@ -859,34 +981,168 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) k_greedy_rounds(GreedyArgs 
         s_hkey[i] = kHotEmpty;
         s_hcnt[i] = 0;
     }
-    if (threadIdx.x == 0) s_nbig = 0;
-    uint64_t cov = 0, sum_c = 0;  // running totals, kept by block 0
-    __syncthreads();
-    for (int32_t round = 0; round < a.k; ++round) {
-        // the best outside S: each lane holds one segment's best at a time.
-        // Keys only decrease, so a segment whose best is still outside S
-        // with an unchanged Delta keeps it (every other key is at most what
-        // it was; ties keep the lowest id), and a segment with no vertex
-        // outside S stays so; the others are rescanned, one warp each.
-        // warp gw of W takes segments gw + W i, 32 of them at a time (lane l:
-        // gw + W (32 i + l)); the block index varies fastest over gw, so a
-        // few segments already spread over every SM
-        KeyId wbest{0, 0xFFFFFFFFu, 0};
+    if (threadIdx.x == 0) s_failed = 0;
+    GridBar bar{a.ctl, &s_failed, 0u};
+    int par = 0;  // half of s_part of the next block reduction
+
+    auto make = [&](uint32_t v, uint32_t d, uint64_t w) -> Cand {
+        const u128 key = a.ris ? (u128)d : (u128)d * a.W + (u128)a.T * (one_f - w);
+        return Cand{(uint32_t)(key >> 64), (uint32_t)(key >> 32), (uint32_t)key, v, d, 0u, 0ull};
+    };
+    // the block's best of the threads' candidates, known to every thread; a
+    // block barrier stands between the candidates' loads and the return
+    auto block_cand = [&](const Cand& c) -> Cand {
+        const int src = warp_best_lane(c);
+        if (lane == src) s_part[par][wib] = c;
+        __syncthreads();
+        const int win = warp_best_lane(s_part[par][lane]);
+        const Cand r = s_part[par][win];
+        par ^= 1;
+        return r;
+    };
+    // the grid's best, known to every thread (one grid barrier)
+    auto grid_cand = [&](const Cand& c) -> Cand {
+        const Cand b = block_cand(c);
+        if (threadIdx.x == 0) a.partial[blockIdx.x] = b;
+        bar.sync();
+        Cand r = no_cand();
+        for (unsigned i = lane; i < gridDim.x; i += 32) {
+            const Cand x = ldcg_cand(a.partial + i);
+            if (cand_better(x, r)) r = x;
+        }
+        const int src = warp_best_lane(r);
+        r.k2 = __shfl_sync(kFull, r.k2, src);
+        r.k1 = __shfl_sync(kFull, r.k1, src);
+        r.k0 = __shfl_sync(kFull, r.k0, src);
+        r.id = __shfl_sync(kFull, r.id, src);
+        r.d = __shfl_sync(kFull, r.d, src);
+        return r;
+    };
+    auto bucket = [&](uint32_t d, uint64_t w) { return greedy_bucket(d, one_f - w, a.ratio, a.ris); };
+
+    // the pool entry of this thread
+    uint32_t p_id = kNone, p_cnt = 0;
+    uint64_t p_w = 0, p_lo = 0;
+    auto pool_best = [&]() -> Cand {
+        Cand c = no_cand();
+        if (p_id != kNone) {
+            c = make(p_id, __ldcg(a.delta + p_id), p_w);
+            c.cnt = p_cnt;
+            c.lo = p_lo;
+        }
+        return block_cand(c);
+    };
+    // Fills the pool from the vertices outside S; returns the best of the others.
+    bool hist_ready = true;  // k_greedy_init's
+    auto refill = [&]() -> Cand {
+        const int64_t stride = (int64_t)gridDim.x * kGreedyThreads;
+        const int64_t first = (int64_t)blockIdx.x * kGreedyThreads + threadIdx.x;
+        if (threadIdx.x == 0) s_cut = kBuckets;
+        __syncthreads();
+        if (!hist_ready) {
+            for (int i = threadIdx.x; i < kBuckets; i += kGreedyThreads) s_hist[i] = 0;
+            __syncthreads();
+            for (int64_t v0 = first - lane; v0 < a.n; v0 += stride) {  // warp-uniform
+                const int64_t v = v0 + lane;
+                uint32_t b = kBuckets;
+                if (v < a.n && !__ldcg(a.inS + v)) b = bucket(__ldcg(a.delta + v), a.w[v]);
+                const unsigned peers = __match_any_sync(kFull, b);
+                if (b < kBuckets && lane == __ffs(peers) - 1) atomicAdd(&s_hist[b], (uint32_t)__popc(peers));
+            }
+            __syncthreads();
+            for (int i = threadIdx.x; i < kBuckets; i += kGreedyThreads)
+                if (s_hist[i]) atomicAdd(&a.hist[i], s_hist[i]);
+            bar.sync();
+        }
+        hist_ready = false;
+        // the lowest bucket down to which the pool has room: thread t counts
+        // buckets 8 (1023 - t) + 7 .. 8 (1023 - t), in descending order over t
+        constexpr int kPer = kBuckets / kGreedyThreads;
+        const int top = kPer * (kGreedyThreads - 1 - threadIdx.x) + kPer - 1;
+        uint32_t c[kPer], sum = 0;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            c[i] = __ldcg(a.hist + top - i);
+            sum += c[i];
+        }
+        uint32_t incl = sum;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(kFull, incl, d);
+            if (lane >= d) incl += y;
+        }
+        if (lane == 31) s_wsum[wib] = incl;
+        __syncthreads();
+        uint32_t before = incl - sum;
+        for (int q = 0; q < wib; ++q) before += (uint32_t)s_wsum[q];
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            before += c[i];
+            if (before <= (uint32_t)kGreedyThreads) atomicMin(&s_cut, (uint32_t)(top - i));
+        }
+        __syncthreads();
+        const uint32_t cut = s_cut;
+        Cand out = no_cand();
+        for (int64_t v0 = first; v0 < a.n; v0 += 4 * stride) {  // four vertices a pass, their loads together
+            uint8_t in4[4];
+            uint32_t d4[4];
+            uint64_t w4[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int64_t v = v0 + q * stride;
+                in4[q] = 1;
+                if (v < a.n) {
+                    in4[q] = __ldcg(a.inS + v);
+                    d4[q] = __ldcg(a.delta + v);
+                    w4[q] = a.w[v];
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (in4[q]) continue;
+                const uint32_t v = (uint32_t)(v0 + q * stride);
+                if (bucket(d4[q], w4[q]) >= cut) {
+                    const uint32_t slot = atomicAdd(&a.ctl->pool_n, 1u);
+                    if (slot < (uint32_t)kGreedyThreads) a.pool[slot] = v;
+                } else {
+                    const Cand x = make(v, d4[q], w4[q]);
+                    if (cand_better(x, out)) out = x;
+                }
+            }
+        }
+        out = grid_cand(out);
+        const uint32_t np = min(__ldcg(&a.ctl->pool_n), (uint32_t)kGreedyThreads);
+        p_id = kNone;
+        if (threadIdx.x < np) {
+            p_id = __ldcg(a.pool + threadIdx.x);
+            p_w = a.w[p_id];
+            p_lo = a.inv_off[p_id];
+            p_cnt = (uint32_t)(a.inv_off[p_id + 1] - p_lo);
+        }
+        return out;
+    };
+    // The best vertex outside S by segments. Warp gw of W takes segments
+    // gw + W i, 32 of them at a time (lane l: gw + W (32 i + l)); the block
+    // index varies fastest over gw, so a few segments already spread over
+    // every SM.
+    bool seg_init = false;
+    auto seg_scan = [&]() -> Cand {
+        Cand wbest = no_cand();
         const int64_t W = (int64_t)gridDim.x * nw, gw = (int64_t)wib * gridDim.x + blockIdx.x;
         for (int64_t g0 = gw; g0 < a.nseg; g0 += 32 * W) {
             const int64_t sg = g0 + lane * W;
-            KeyId b{0, 0xFFFFFFFFu, 0};
+            Cand b = no_cand();
             bool ok = sg >= a.nseg;
-            if (!ok && round > 0) {
-                b = ldcg_keyid(a.seg_best + sg);
-                ok = !b.valid || (!__ldcg(a.inS + b.id) && __ldcg(a.delta + b.id) == b.d);
+            if (!ok && seg_init) {
+                b = ldcg_cand(a.seg_best + sg);
+                ok = b.id == kNone || (!__ldcg(a.inS + b.id) && __ldcg(a.delta + b.id) == b.d);
             }
             unsigned redo = __ballot_sync(kFull, !ok);
             while (redo) {
                 const int src = __ffs(redo) - 1;
                 redo &= redo - 1;
                 const int64_t v_lo = (g0 + src * W) << kGreedySegLog, v_hi = min(a.n, v_lo + kGreedySeg);
-                KeyId r{0, 0xFFFFFFFFu, 0};
+                Cand r = no_cand();
                 // four of the lane's vertices per pass, their loads issued together
                 for (int64_t v0 = v_lo + lane; v0 < v_hi; v0 += 128) {
                     uint8_t in4[4];
@@ -905,94 +1161,123 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) k_greedy_rounds(GreedyArgs 
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         if (in4[q]) continue;
-                        const u128 dv = (u128)d4[q];
-                        const KeyId c{a.ris ? dv : dv * a.W + (u128)a.T * (one_f - w4[q]), (uint32_t)(v0 + 32 * q),
-                                      1u, d4[q], 0u};
-                        if (better(c, r)) r = c;
+                        const Cand c = make((uint32_t)(v0 + 32 * q), d4[q], w4[q]);
+                        if (cand_better(c, r)) r = c;
                     }
                 }
-#pragma unroll
-                for (int d = 16; d > 0; d >>= 1) {
-                    const KeyId o = shfl_down_keyid(r, d);
-                    if (better(o, r)) r = o;
-                }
-                r = shfl_keyid(r, 0);
+                const int best = warp_best_lane(r);
+                r.k2 = __shfl_sync(kFull, r.k2, best);
+                r.k1 = __shfl_sync(kFull, r.k1, best);
+                r.k0 = __shfl_sync(kFull, r.k0, best);
+                r.id = __shfl_sync(kFull, r.id, best);
+                r.d = __shfl_sync(kFull, r.d, best);
                 if (lane == src) b = r;
                 if (lane == 0) a.seg_best[g0 + src * W] = r;
             }
-            if (better(b, wbest)) wbest = b;
+            if (cand_better(b, wbest)) wbest = b;
         }
-        const KeyId best = block_best(wbest, s_part);
-        if (threadIdx.x == 0) a.partial[blockIdx.x] = best;
-        grid.sync();
-        if (wib == 0) {
-            KeyId b{0, 0xFFFFFFFFu, 0};
-            for (unsigned i = lane; i < gridDim.x; i += 32) {
-                const KeyId c = ldcg_keyid(a.partial + i);
-                if (better(c, b)) b = c;
-            }
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) {
-                const KeyId o = shfl_down_keyid(b, d);
-                if (better(o, b)) b = o;
-            }
-            if (lane == 0) s_win = b;
+        seg_init = true;
+        return grid_cand(wbest);
+    };
+
+    uint64_t cov = 0, sum_c = 0;  // running totals, kept by one thread
+    bool pool_on = false;
+    uint32_t seg_left = 0;
+    Cand bound = no_cand();  // the best outside the pool when it was filled
+    __syncthreads();
+    for (int32_t round = 0; round < a.k; ++round) {
+        Cand win = no_cand();
+        bool found = false, refilled = false;
+        if (pool_on) {
+            win = pool_best();
+            found = cand_better(win, bound);
         }
-        __syncthreads();
-        const uint32_t v = s_win.id;
-        if (threadIdx.x == 0) {
-            if (blockIdx.x == 0) {
-                a.inS[v] = 1;  // read (through L2) after the round's last grid barrier
-                cov += s_win.d;  // Delta_v as scanned, before any walk of this round
-                sum_c += one_f - a.w[v];
-                a.seeds[round] = (int32_t)v;
-                a.cov_out[round] = (int64_t)cov;
-                const u128 N = a.ris ? (u128)cov * (uint64_t)a.n : (u128)cov * a.W + (u128)a.T * sum_c;
-                const u128 D = a.ris ? (u128)a.T : (u128)a.T << a.f;
-                a.est_out[round] = u128_to_double(N) / u128_to_double(D);
-            }
+        if (!found && seg_left) {
+            --seg_left;
+            win = seg_scan();
+        } else if (!found) {
+            bound = refill();
+            refilled = true;
+            win = pool_best();
+            if (!cand_better(win, bound)) win = bound;
+            pool_on = __syncthreads_count(p_id != kNone) >= (int)kPoolMin;
+            if (!pool_on) seg_left = kSegRounds;
         }
-        __syncthreads();
-        // cover the uncovered samples of the committed vertex
-        // a warp takes spw list entries at a time, spw the power of two that
-        // spreads the list over every warp (up to 32), so a short list is
-        // not walked by a few warps one member at a time
-        const uint64_t lo = a.inv_off[v], cnt = a.inv_off[v + 1] - lo;
-        const uint64_t nwarps = (uint64_t)gridDim.x * (kGreedyThreads / 32);
-        uint32_t spw = 1;
-        while (spw < 32 && (uint64_t)spw * nwarps < cnt) spw <<= 1;
-        for (uint64_t base = ((uint64_t)blockIdx.x * (kGreedyThreads / 32) + wib) * spw; base < cnt;
-             base += nwarps * spw) {
-            const uint64_t x = base + lane;
+        const uint32_t v = win.id;
+        // every read of Delta in this block is done: changes may start once
+        // all blocks are here
+        bar.arrive(false);
+        if (p_id == v) p_id = kNone;
+        uint64_t lo = win.lo, cnt = win.cnt;
+        if (cnt == 0) {  // not a pool entry's (or an empty list)
+            lo = a.inv_off[v];
+            cnt = a.inv_off[v + 1] - lo;
+        }
+        // the uncovered samples of the committed vertex, an entry a thread: a
+        // list of up to one entry a thread of the grid is dealt over the blocks
+        // entry by entry, a longer one in runs of 1024
+        const bool spread = cnt <= (uint64_t)gridDim.x * kGreedyThreads;
+        const uint64_t step = (uint64_t)gridDim.x * kGreedyThreads;
+        for (uint64_t base = 0; base < cnt || base == 0; base += step) {
+            const uint64_t x = spread ? (uint64_t)threadIdx.x * gridDim.x + blockIdx.x
+                                      : base + (uint64_t)blockIdx.x * kGreedyThreads + threadIdx.x;
             uint64_t off = 0;
             uint32_t len = 0;
-            if ((uint32_t)lane < spw && x < cnt) {
+            if (x < cnt) {
                 const uint32_t j = a.inv[lo + x];
                 const uint32_t bit = 1u << (j & 31);
+                const uint64_t o = a.h_off[j];  // with the bit, not after it
+                const uint32_t l = a.h_len[j];
                 if ((atomicOr(&a.covered[j >> 5], bit) & bit) == 0) {
-                    off = a.h_off[j];
-                    len = a.h_len[j];
-                    if (len > kBigLen) {  // a large sample: the whole block walks it below
-                        const uint32_t q = atomicAdd(&s_nbig, 1u);
-                        if (q < (uint32_t)kBigQueue) {
-                            s_big_off[q] = off;
-                            s_big_len[q] = len;
-                            len = 0;
-                        }
-                    }
+                    off = o;
+                    len = l;
                 }
             }
-            warp_members(off, len, a.arena, [&](int, int32_t u) { sub_merged(a.delta, u, s_hkey, s_hcnt); });
+            // the block's members end to end: inclusive prefix of the lengths
+            uint64_t incl = len;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint64_t y = __shfl_up_sync(kFull, incl, d);
+                if (lane >= d) incl += y;
+            }
+            if (lane == 31) s_wsum[wib] = incl;
+            if (base == 0) {
+                if (!bar.wait(false)) return;  // the host reports it
+                if (refilled && blockIdx.x == 0) {  // every block has read these
+                    for (int i = threadIdx.x; i < kBuckets; i += kGreedyThreads) a.hist[i] = 0;
+                    if (threadIdx.x == 0) a.ctl->pool_n = 0;
+                }
+                // read (through L2) after the round's last grid barrier
+                if (blockIdx.x == 0 && threadIdx.x == 0) a.inS[v] = 1;
+            } else {
+                __syncthreads();
+            }
+            uint64_t before = 0, total = 0;
+            {
+                uint64_t wsum = s_wsum[lane];
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint64_t y = __shfl_up_sync(kFull, wsum, d);
+                    if (lane >= d) wsum += y;
+                }
+                total = __shfl_sync(kFull, wsum, 31);
+                before = __shfl_sync(kFull, wsum, wib > 0 ? wib - 1 : 0);
+                if (wib == 0) before = 0;
+            }
+            if (total) {
+                s_off[threadIdx.x] = off - (before + incl - len);  // + a member's place in the block
+                s_end[threadIdx.x] = before + incl;
+                __syncthreads();
+                for (uint64_t p = threadIdx.x; p < total; p += kGreedyThreads) {
+                    int owner = 0;  // the sample that holds member p: entries that end at or before it
+#pragma unroll
+                    for (int b = kGreedyThreads / 2; b; b >>= 1)
+                        if (s_end[owner + b - 1] <= p) owner += b;
+                    sub_merged(a.delta, a.arena[s_off[owner] + p], s_hkey, s_hcnt);
+                }
+            }
+            __syncthreads();  // s_wsum, s_off and s_end are free again
         }
-        __syncthreads();
-        const uint32_t nbig = min(s_nbig, (uint32_t)kBigQueue);
-        for (uint32_t b = 0; b < nbig; ++b) {
-            const uint64_t boff = s_big_off[b];
-            const uint32_t blen = s_big_len[b];
-            for (uint32_t i = threadIdx.x; i < blen; i += blockDim.x) sub_merged(a.delta, a.arena[boff + i], s_hkey, s_hcnt);
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) s_nbig = 0;
         for (int i = threadIdx.x; i < kHotSlots; i += blockDim.x) {
             const uint32_t key = s_hkey[i];
             if (key != kHotEmpty) {
@@ -1001,13 +1286,19 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) k_greedy_rounds(GreedyArgs 
                 s_hcnt[i] = 0;
             }
         }
-        grid.sync();
+        __syncthreads();
+        bar.arrive(true);
+        if (blockIdx.x == 0 && threadIdx.x == kGreedyThreads - 1) {  // while the barrier is waited for
+            cov += win.d;  // Delta_v as read, before any walk of this round
+            sum_c += one_f - a.w[v];
+            a.seeds[round] = (int32_t)v;
+            a.cov_out[round] = (int64_t)cov;
+            const u128 N = a.ris ? (u128)cov * (uint64_t)a.n : (u128)cov * a.W + (u128)a.T * sum_c;
+            const u128 D = a.ris ? (u128)a.T : (u128)a.T << a.f;
+            a.est_out[round] = u128_to_double(N) / u128_to_double(D);
+        }
+        if (!bar.wait(true)) return;  // the host reports it
     }
-}
-
-__global__ void k_delta_from_index(const uint64_t* __restrict__ inv_off, int64_t n, uint32_t* __restrict__ delta) {
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
-        delta[v] = (uint32_t)(inv_off[v + 1] - inv_off[v]);
 }
 
 int sketch_inverted(skis_sketch* s, cudaStream_t st, std::string* err) {
@@ -1065,8 +1356,9 @@ int sketch_greedy(skis_sketch* s, int32_t k, int32_t* h_seeds, int64_t* h_cov, d
     if (rc != SKIS_OK) return rc;
     uint32_t *delta = nullptr, *covered = nullptr;
     uint8_t* inS = nullptr;
-    KeyId* partial = nullptr;
-    KeyId* seg_best = nullptr;
+    Cand *partial = nullptr, *seg_best = nullptr;
+    uint32_t *pool = nullptr, *hist = nullptr;
+    GreedyCtl *ctl = nullptr, h_ctl{};
     int32_t* d_seeds = nullptr;
     int64_t* d_cov = nullptr;
     double* d_est = nullptr;
@@ -1084,15 +1376,17 @@ int sketch_greedy(skis_sketch* s, int32_t k, int32_t* h_seeds, int64_t* h_cov, d
         CV_CUDA(dev_alloc_t(&partial, (size_t)gblocks, st));
         const int64_t nseg = (n + kGreedySeg - 1) / kGreedySeg;
         CV_CUDA(dev_alloc_t(&seg_best, (size_t)nseg, st));
+        CV_CUDA(dev_alloc_t(&pool, (size_t)kGreedyThreads, st));
+        // one allocation zeroed at once: the histogram and the control words
+        const size_t words = kBuckets + sizeof(GreedyCtl) / sizeof(uint32_t);
+        CV_CUDA(dev_alloc_t(&hist, words, st));
+        CV_CUDA(cudaMemsetAsync(hist, 0, words * sizeof(uint32_t), st));
+        ctl = reinterpret_cast<GreedyCtl*>(hist + kBuckets);
         CV_CUDA(dev_alloc_t(&d_seeds, (size_t)k, st));
         CV_CUDA(dev_alloc_t(&d_cov, (size_t)k, st));
         CV_CUDA(dev_alloc_t(&d_est, (size_t)k, st));
         CV_CUDA(cudaMemsetAsync(inS, 0, (size_t)n, st));
         CV_CUDA(cudaMemsetAsync(covered, 0, (size_t)((T + 31) / 32) * sizeof(uint32_t), st));
-        // Delta_R(v, {}) = number of samples containing v = length of v's list
-        const int b1 = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)sm_count() * 8));
-        k_delta_from_index<<<b1, 256, 0, st>>>(s->inv_off, n, delta); note_launch();
-        CV_CUDA(cudaGetLastError());
         GreedyArgs ga;
         ga.w = g->w;
         ga.inS = inS;
@@ -1100,6 +1394,7 @@ int sketch_greedy(skis_sketch* s, int32_t k, int32_t* h_seeds, int64_t* h_cov, d
         ga.n = n;
         ga.W = g->W;
         ga.T = T;
+        ga.ratio = g->W ? (double)T / (double)g->W : 0.0;
         ga.f = g->f;
         ga.k = k;
         ga.inv_off = s->inv_off;
@@ -1111,17 +1406,29 @@ int sketch_greedy(skis_sketch* s, int32_t k, int32_t* h_seeds, int64_t* h_cov, d
         ga.partial = partial;
         ga.seg_best = seg_best;
         ga.nseg = nseg;
+        ga.pool = pool;
+        ga.hist = hist;
+        ga.ctl = ctl;
         ga.seeds = d_seeds;
         ga.cov_out = d_cov;
         ga.est_out = d_est;
         ga.ris = s->ris;
+        const int b1 = (int)std::max<int64_t>(1, std::min<int64_t>((n + kGreedyThreads - 1) / kGreedyThreads,
+                                                                   (int64_t)sm_count() * 2));
+        k_greedy_init<<<b1, kGreedyThreads, 0, st>>>(ga); note_launch();
+        CV_CUDA(cudaGetLastError());
         void* kargs[] = {&ga};
         CV_CUDA(cudaLaunchCooperativeKernel((const void*)k_greedy_rounds, gblocks, kGreedyThreads, kargs, 0, st));
         note_launch();
         CV_CUDA(cudaMemcpyAsync(h_seeds, d_seeds, (size_t)k * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
         if (h_cov) CV_CUDA(cudaMemcpyAsync(h_cov, d_cov, (size_t)k * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
         if (h_est) CV_CUDA(cudaMemcpyAsync(h_est, d_est, (size_t)k * sizeof(double), cudaMemcpyDeviceToHost, st));
+        CV_CUDA(cudaMemcpyAsync(&h_ctl, ctl, sizeof(GreedyCtl), cudaMemcpyDeviceToHost, st));
         CV_CUDA(cudaStreamSynchronize(st));
+        if (h_ctl.gave_up) {
+            *err = "skis_greedy_maxcover: internal error: a grid barrier ran out";
+            return SKIS_ERR_INTERNAL;
+        }
         return SKIS_OK;
     };
     rc = body();
@@ -1130,6 +1437,8 @@ int sketch_greedy(skis_sketch* s, int32_t k, int32_t* h_seeds, int64_t* h_cov, d
     dev_free(inS, st);
     dev_free(partial, st);
     dev_free(seg_best, st);
+    dev_free(pool, st);
+    dev_free(hist, st);
     dev_free(d_seeds, st);
     dev_free(d_cov, st);
     dev_free(d_est, st);
