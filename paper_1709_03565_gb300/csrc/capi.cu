@@ -563,6 +563,7 @@ void skis::sketch_release(skis_sketch* s) {
     dev_free(s->spill_hash, st);
     dev_free(s->spill_queue, st);
     dev_free(s->bitmaps, st);
+    dev_free(s->slot_clean, st);
     dev_free(s->queues, st);
     dev_free(s->big_queues, st);
     dev_free(s->big_ids, st);

@@ -90,6 +90,7 @@ struct SampleArgs {
     uint64_t arena_cap;
     DevStatus* status;
     uint32_t* bitmaps;
+    uint32_t* slot_clean;    // CTA tier: the slot's bitmap has been cleared
     int32_t* queues;
     uint64_t bitmap_words;
     uint32_t queue_cap;      // CTA tier: entries of a slot's queue (also the slots' stride); a sample
@@ -948,7 +949,12 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_iis_warp(SampleArgs a) {
 
 // -------------------------------------------------------------- CTA tier
 // One block of kCtaThreads threads per sample, 1024 threads of such blocks per
-// SM (four of 256 by default, or two of 512: the option SKIS_OPT_CTA_THREADS).
+// SM: eight blocks of 128 by default, or two of 512 (SKIS_OPT_CTA_THREADS).
+// Four warps a sample pay a level's fixed cost half as often as eight, and
+// twice as many samples hide one another's latencies. R-MAT 2^22 / 2^27 WC,
+// 200K samples: 47.2 ms with blocks of 256, 44.7 with 128, 48.0 with 64;
+// 2^25 / 2^30, 10^6 samples: 614, 600, 607; Chung-Lu 4M / 140M WC, 262K
+// samples: 4.2, 2.9, 2.8.
 // The reverse BFS goes level by level. The in-rows of a level's first
 // kCtaWin vertices wait in shared memory: a vertex's row is loaded while its
 // visited bit is set, so a level costs two memory latencies (the source
@@ -962,8 +968,9 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_iis_warp(SampleArgs a) {
 // atomic round trips a level) and every level read its queue and rows back:
 // on Chung-Lu 1M / 17.5M WC the 7670 samples of 1M that run here took 7.4 ms
 // and take 4.4 ms. Where hubs hold the coins it is bound by the coin
-// generator: R-MAT 2^22 / 2^27 WC 355G blocks/s, 2^25 / 2^30 421G (the hub
+// generator: R-MAT 2^22 / 2^27 WC 372G blocks/s, 2^25 / 2^30 431G (the hub
 // loop alone, with no other work in the kernel, 455G).
+constexpr int kCtaBlock = 128;  // threads of the default blocks
 constexpr int kCtaWin = 512;  // rows of a level in shared memory at a time
 
 template <int kCtaThreads>
@@ -990,6 +997,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1024 / kCtaThreads) k_iis_cta(Sam
     const uint4* __restrict__ rows4 = reinterpret_cast<const uint4*>(a.rows);  // offset (low, high), degree, threshold
     const uint64_t count = input_count(a);
     auto is_hub = [&](uint32_t nq) { return a.cta_hub_quads && nq >= a.cta_hub_quads; };
+    bool clean = a.slot_clean[blockIdx.x] != 0;
     unsigned long long claim = 0;  // thread 0: the block's next input
     if (threadIdx.x == 0) claim = atomicAdd(a.work, 1ull);
 
@@ -1003,6 +1011,12 @@ __global__ void __launch_bounds__(kCtaThreads, 1024 / kCtaThreads) k_iis_cta(Sam
         const uint64_t j = s_j;
         if (j == ~0ull) break;
         if (threadIdx.x == 0) claim = atomicAdd(a.work, 1ull);  // arrives while this sample is drawn
+        if (!clean) {  // the slot's first sample: its bitmap is cleared once, and kept clear by every sample
+            for (uint64_t i = threadIdx.x; i < a.bitmap_words; i += kCtaThreads) bitmap[i] = 0;
+            __syncthreads();
+            if (threadIdx.x == 0) a.slot_clean[blockIdx.x] = 1;
+            clean = true;
+        }
 
         RowInfo rv;
         int64_t pe;
@@ -1587,6 +1601,9 @@ static cudaError_t grow_copy(T** p, uint64_t old_n, uint64_t new_n, cudaStream_t
     return cudaSuccess;
 }
 
+// threads of a CTA-tier block
+static int cta_block(const skis_sketch* s) { return s->cta_threads == 512 ? 512 : kCtaBlock; }
+
 // slack: arena entries that the tiers' warps may leave unused at the ends of their chunks;
 // warps: the warp tier's warps (0: no such tier)
 static int ensure_sample_buffers(skis_sketch* s, uint64_t count, uint64_t slack, uint64_t warps, cudaStream_t st,
@@ -1668,23 +1685,29 @@ static int ensure_sample_buffers(skis_sketch* s, uint64_t count, uint64_t slack,
     }
     // CTA-tier slots: an n-bit visited bitmap and a queue of min(n, cta_queue_cap)
     // entries each (a sample with more members moves to a pass over slots with
-    // n-entry queues), 1024 threads of blocks per SM within ~8 GB
+    // n-entry queues), 1024 threads of blocks per SM within ~12 GB. A block
+    // clears its bitmap when it takes its first sample (few of them do where few
+    // samples come this far)
     const uint32_t qcap = (uint32_t)std::min<uint64_t>((uint64_t)g->n, s->cta_queue_cap);
     int slots = s->cta_slots;
     if (slots <= 0) {
         const uint64_t per_slot = (uint64_t)qcap * 4 + ((uint64_t)g->n + 31) / 32 * 4;
-        const uint64_t budget = 8ull << 30;
-        const uint64_t per_sm = g->lt ? 2 : 1024 / s->cta_threads;
+        const uint64_t budget = 12ull << 30;
+        const uint64_t per_sm = g->lt ? 2 : 1024 / cta_block(s);
         slots = (int)std::min<uint64_t>((uint64_t)sm_count() * per_sm, std::max<uint64_t>(1, budget / per_slot));
     }
     if (slots != s->cta_slots_alloc || qcap != s->queue_cap) {
         dev_free(s->bitmaps, st);
         dev_free(s->queues, st);
-        s->bitmaps = nullptr;
+        dev_free(s->slot_clean, st);
+        s->bitmaps = s->slot_clean = nullptr;
         s->queues = nullptr;
+        s->cta_slots_alloc = 0;
         s->bitmap_words = ((uint64_t)g->n + 31) / 32;
         SK_CUDA(dev_alloc_t(&s->bitmaps, (size_t)(s->bitmap_words * slots), st));
-        SK_CUDA(cudaMemsetAsync(s->bitmaps, 0, s->bitmap_words * slots * sizeof(uint32_t), st));
+        SK_CUDA(dev_alloc_t(&s->slot_clean, (size_t)slots, st));
+        if (g->lt) SK_CUDA(cudaMemsetAsync(s->bitmaps, 0, s->bitmap_words * slots * sizeof(uint32_t), st));
+        else SK_CUDA(cudaMemsetAsync(s->slot_clean, 0, (size_t)slots * sizeof(uint32_t), st));
         SK_CUDA(dev_alloc_t(&s->queues, (size_t)((uint64_t)qcap * slots), st));
         s->cta_slots_alloc = slots;
         s->queue_cap = qcap;
@@ -1703,6 +1726,12 @@ static int ensure_big_slots(skis_sketch* s, cudaStream_t st, std::string* err) {
     SK_CUDA(dev_alloc_t(&s->big_queues, (size_t)(n * slots), st));
     s->big_slots = slots;
     return SKIS_OK;
+}
+
+static void launch_cta(const skis_sketch* s, const SampleArgs& a, int slots, cudaStream_t st) {
+    if (cta_block(s) == 512) k_iis_cta<512><<<slots, 512, 0, st>>>(a);
+    else k_iis_cta<kCtaBlock><<<slots, kCtaBlock, 0, st>>>(a);
+    note_launch();
 }
 
 static int occupancy_grid(const void* kernel, int threads, int override_blocks, uint64_t max_useful,
@@ -1780,6 +1809,7 @@ int sketch_sample(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* 
     base.arena_cap = s->arena_cap;
     base.status = s->status;
     base.bitmaps = s->bitmaps;
+    base.slot_clean = s->slot_clean;
     base.queues = s->queues;
     base.bitmap_words = s->bitmap_words;
     base.queue_cap = s->queue_cap;
@@ -1877,9 +1907,7 @@ int sketch_sample(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* 
             k_iis_warp<<<warp_blocks, kWarpThreads, 0, st>>>(aw); note_launch();
             SK_CUDA(cudaGetLastError());
             SK_CUDA(cudaEventRecord(s->ev[2], st));
-            if (s->cta_threads == 512) k_iis_cta<512><<<s->cta_slots_alloc, 512, 0, st>>>(ac);
-            else k_iis_cta<256><<<s->cta_slots_alloc, 256, 0, st>>>(ac);
-            note_launch();
+            launch_cta(s, ac, s->cta_slots_alloc, st);
             SK_CUDA(cudaGetLastError());
             SK_CUDA(cudaEventRecord(s->ev[3], st));
         }
@@ -1905,9 +1933,7 @@ int sketch_sample(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* 
             if (g->lt) {
                 k_lt_long<<<s->big_slots, 32, 0, st>>>(ab); note_launch();
             } else {
-                if (s->cta_threads == 512) k_iis_cta<512><<<s->big_slots, 512, 0, st>>>(ab);
-                else k_iis_cta<256><<<s->big_slots, 256, 0, st>>>(ab);
-                note_launch();
+                launch_cta(s, ab, s->big_slots, st);
             }
             SK_CUDA(cudaGetLastError());
             SK_CUDA(cudaEventRecord(s->ev[3], st));
