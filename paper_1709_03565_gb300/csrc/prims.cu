@@ -176,15 +176,23 @@ cudaError_t scan_u128(const u128* in, u128* out, int64_t n, cudaStream_t st) {
 // index as value (so equal keys keep input order), in 8-bit digits. One
 // kernel reads the edges once and counts every digit of every pass; then one
 // kernel a pass ("onesweep"): each CTA claims the next tile from a ticket,
-// ranks its items per warp (match_any, warp-striped loads: positions in warp
-// order, so the ranking is stable), publishes the tile's per-digit counts and
-// looks back over the previous tiles' published counts for its global
-// offsets (decoupled look-back), then writes the tile out through shared
-// memory in digit order, so that each digit's items leave as a contiguous
-// run. The first pass builds the keys from the edge arrays in registers.
-constexpr int kOsThreads = 256;
-constexpr int kOsItems = 16;
-constexpr int kOsTile = kOsThreads * kOsItems;  // 4096 items
+// ranks its items per warp (one vote a digit bit, warp-striped loads: positions
+// in warp order, so the ranking is stable), publishes the tile's per-digit
+// counts, lays the tile out in shared memory in digit order, looks back over
+// the previous tiles' published counts for its global offsets (decoupled
+// look-back), and writes the tile out, so that each digit's items leave as a
+// contiguous run. The first pass builds the keys from the edge arrays in
+// registers.
+// A pass is bound by instruction issue (the votes: 0.7 of the ALU pipe) and by
+// the look-back's latency, at about half of the copy bandwidth. 7 10^7 edges,
+// 44-bit keys in five passes, whole graph load: 5.71 ms with match_any ranks
+// and tiles of 4096 items on 256 threads, 4.46 with votes and 6144 items on
+// 512 threads, two CTAs an SM (4096 items, three CTAs: 4.7; 7168: 4.6; 8192 on
+// one CTA: 6.4); 1.4 10^8 edges 10.7 -> 8.2 ms.
+constexpr int kOsThreads = 512;
+constexpr int kOsItems = 12;
+constexpr int kOsGroup = 4;                     // of a thread's items ranked at a time
+constexpr int kOsTile = kOsThreads * kOsItems;  // 6144 items
 constexpr int kOsWarps = kOsThreads / 32;
 constexpr int kOsMaxPasses = 8;
 // status word of (tile, digit): state in bits 62-63 (1: the tile's own
@@ -266,164 +274,168 @@ struct OsOut {
 };
 
 template <bool kFirst, bool kLast, int kBits>
-__global__ void __launch_bounds__(kOsThreads, 3) k_os_pass(
+__global__ void __launch_bounds__(kOsThreads, 2) k_os_pass(
     const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int src_bits,
     const uint64_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in, OsOut out, int64_t n, int shift,
     unsigned long long tag,
     const unsigned long long* __restrict__ base, unsigned long long* __restrict__ status,
     unsigned int* __restrict__ ticket, unsigned int* __restrict__ gave_up) {
-    constexpr int kDigits = 1 << kBits, kPer = kDigits / kOsThreads;  // digits a thread owns
+    constexpr int kDigits = 1 << kBits;  // thread t < kDigits owns digit t
     constexpr uint32_t kMask = kDigits - 1;
+    static_assert(kDigits <= kOsThreads && kOsTile <= 65536, "a digit a thread; positions in the tile fit 16 bits");
     extern __shared__ __align__(16) unsigned char os_smem[];
     uint64_t* s_keys = reinterpret_cast<uint64_t*>(os_smem);
     uint32_t* s_vals = reinterpret_cast<uint32_t*>(s_keys + kOsTile);
-    __shared__ uint32_t s_wcnt[kOsWarps][kDigits];   // per warp: digit counts, then the warp's start in the digit
-    __shared__ uint32_t s_tstart[kDigits];           // digit start within the tile
-    __shared__ unsigned long long s_gbase[kDigits];  // output position of the digit's first item of the tile
-    __shared__ uint32_t s_wsum[kPer][kOsWarps];
+    // per warp: digit counts, then the tile position of the warp's first (16 bits each, two a word)
+    __shared__ uint32_t s_wcnt[kOsWarps][kDigits / 2];
+    __shared__ uint32_t s_out[kDigits];  // output position of a digit's items less their tile position
+    __shared__ uint32_t s_wsum[kOsWarps];
     __shared__ uint32_t s_tile, s_bad;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const bool owner = tid < kDigits;
+    uint16_t* const my_cnt = reinterpret_cast<uint16_t*>(&s_wcnt[0][0]) + tid;  // + w kDigits: warp w's
     if (tid == 0) {
         s_tile = atomicAdd(ticket, 1u);
         s_bad = 0;
     }
-    unsigned long long digit_base[kPer];  // in flight while the tile loads
-#pragma unroll
-    for (int r = 0; r < kPer; ++r) digit_base[r] = base[tid + r * kOsThreads];
-#pragma unroll
-    for (int w = 0; w < kOsWarps; ++w)
-#pragma unroll
-        for (int r = 0; r < kPer; ++r) s_wcnt[w][tid + r * kOsThreads] = 0;
+    const unsigned long long digit_base = owner ? base[tid] : 0;  // in flight while the tile loads
+    for (int i = tid; i < kOsWarps * kDigits / 2; i += kOsThreads) (&s_wcnt[0][0])[i] = 0;
     __syncthreads();
     const uint32_t tile = s_tile;
     const int64_t t0 = (int64_t)tile * kOsTile;
-    const int64_t wb = t0 + (int64_t)wid * (32 * kOsItems);
+    const int64_t wb = t0 + (int64_t)wid * (32 * kOsItems) + lane;  // this lane's items: wb + 32 c
+    const int left = (int)max((int64_t)0, min((int64_t)(32 * kOsItems), n - wb));  // item c is there if 32 c < left
     uint64_t key[kOsItems];
-    uint32_t val[kOsItems], rnk[kOsItems];
 #pragma unroll
     for (int c = 0; c < kOsItems; ++c) {
-        const int64_t i = wb + c * 32 + lane;
-        if (kFirst) {
-            key[c] = i < n ? edge_key(src, dst, i, src_bits) : 0;
-            val[c] = (uint32_t)i;
-        } else {
-            key[c] = i < n ? keys_in[i] : 0;
-            val[c] = i < n ? vals_in[i] : 0;
+        key[c] = 0;
+        if (32 * c < left) key[c] = kFirst ? edge_key(src, dst, wb + 32 * c, src_bits) : keys_in[wb + 32 * c];
+    }
+    // rank within the warp: earlier chunks, then lower lanes. The lanes with a
+    // lane's digit by one vote a bit (a match instruction is slower); then the
+    // counter updates in chunk order, none waiting for the one before, and the
+    // broadcasts, kOsGroup of each in flight
+    uint32_t rnk[kOsItems];  // digit << 16 | rank
+#pragma unroll
+    for (int g = 0; g < kOsItems; g += kOsGroup) {
+        uint32_t peers[kOsGroup], old[kOsGroup];
+#pragma unroll
+        for (int q = 0; q < kOsGroup; ++q) {
+            const int c = g + q;
+            const uint32_t d = (uint32_t)(key[c] >> shift) & kMask;
+            rnk[c] = d << 16;
+            peers[q] = __ballot_sync(kFull, 32 * c < left);
+#pragma unroll
+            for (int b = 0; b < kBits; ++b) {
+                const uint32_t ones = __ballot_sync(kFull, (d >> b) & 1u);
+                const uint32_t mine = (uint32_t)((int32_t)(d << (31 - b)) >> 31);  // all bits as the lane's bit b
+                peers[q] &= ~(ones ^ mine);
+            }
+            old[q] = 0;
+            if (32 * c < left && (peers[q] & lanemask_lt()) == 0)
+                old[q] = atomicAdd(&s_wcnt[wid][d >> 1], (uint32_t)__popc(peers[q]) << (16 * (d & 1u)));
+            __syncwarp();  // this chunk's counts come before the next chunk's
+        }
+#pragma unroll
+        for (int q = 0; q < kOsGroup; ++q) {
+            const uint32_t d = rnk[g + q] >> 16;
+            const uint32_t before = __shfl_sync(kFull, old[q], __ffs(peers[q]) - 1) >> (16 * (d & 1u));
+            rnk[g + q] += (before & 0xFFFFu) + (uint32_t)__popc(peers[q] & lanemask_lt());
         }
     }
-    // rank within the warp: earlier chunks, then lower lanes
+    uint32_t val[kOsItems];  // arrive while the counts are scanned
 #pragma unroll
     for (int c = 0; c < kOsItems; ++c) {
-        const bool valid = wb + c * 32 + lane < n;
-        const uint32_t d = valid ? (uint32_t)((key[c] >> shift) & kMask) : (uint32_t)kDigits;
-        const unsigned peers = __match_any_sync(kFull, d);
-        const int leader = __ffs(peers) - 1;
-        uint32_t before = 0;
-        if (lane == leader && valid) {
-            before = s_wcnt[wid][d];
-            s_wcnt[wid][d] = before + (uint32_t)__popc(peers);
-        }
-        __syncwarp();  // this chunk's counts are in before the next chunk's leaders read them
-        before = __shfl_sync(kFull, before, leader);
-        rnk[c] = before + (uint32_t)__popc(peers & lanemask_lt());
+        val[c] = 0;
+        if (32 * c < left) val[c] = kFirst ? (uint32_t)(wb + 32 * c) : vals_in[wb + 32 * c];
     }
     __syncthreads();
-    // thread tid owns digits tid + r kOsThreads: the tile's count and each warp's start
-    uint32_t cnt[kPer], x[kPer];
+    // the owned digit's count in the tile, published at once
+    uint32_t cnt = 0;
+    if (owner) {
 #pragma unroll
-    for (int r = 0; r < kPer; ++r) {
-        const int dd = tid + r * kOsThreads;
-        uint32_t run = 0;
+        for (int w = 0; w < kOsWarps; ++w) cnt += my_cnt[w * kDigits];
+        st_relaxed_u64(status + (size_t)tile * kDigits + tid, (tile == 0 ? kOsIncl : kOsAgg) | tag | cnt);
+    }
+    // tile-local digit starts: exclusive scan of the counts in digit order, and
+    // from them each warp's start in the digit
+    uint32_t start = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t z = __shfl_up_sync(kFull, start, o);
+        if (lane >= o) start += z;
+    }
+    if (lane == 31) s_wsum[wid] = start;
+    __syncthreads();
+    start -= cnt;
+    for (int w = 0; w < wid; ++w) start += s_wsum[w];
+    if (owner) {
+        uint32_t run = start;
 #pragma unroll
         for (int w = 0; w < kOsWarps; ++w) {
-            const uint32_t c2 = s_wcnt[w][dd];
-            s_wcnt[w][dd] = run;
+            const uint32_t c2 = my_cnt[w * kDigits];
+            my_cnt[w * kDigits] = (uint16_t)run;
             run += c2;
         }
-        cnt[r] = run;
-        st_relaxed_u64(status + (size_t)tile * kDigits + dd, (tile == 0 ? kOsIncl : kOsAgg) | tag | run);
-        // tile-local digit starts: exclusive scan of the counts in digit order
-        uint32_t y = run;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t z = __shfl_up_sync(kFull, y, o);
-            if (lane >= o) y += z;
-        }
-        x[r] = y;
-        if (lane == 31) s_wsum[r][wid] = y;
-    }
-    // look back over the earlier tiles for each owned digit's items before
-    // the tile, kOsWindow tiles a read: sum their own counts back to the first
-    // inclusive prefix, waiting on the first tile not yet published
-#pragma unroll
-    for (int r = 0; r < kPer; ++r) {
-        const int dd = tid + r * kOsThreads;
-        unsigned long long excl = 0;
-        if (tile > 0) {
-            int64_t t = (int64_t)tile - 1;  // the next tile to account for
-            uint32_t spins = 0;
-            bool done = false;
-            while (!done) {
-                unsigned long long v[kOsWindow];
-#pragma unroll
-                for (int k = 0; k < kOsWindow; ++k)
-                    v[k] = t - k >= 0 ? ld_relaxed_u64(status + (size_t)(t - k) * kDigits + dd) : 0;
-                int k = 0;
-#pragma unroll
-                for (int q = 0; q < kOsWindow; ++q) {
-                    const bool ready = (v[q] & (63ull << 56)) == tag && (v[q] >> 62) != 0;
-                    if (!ready) break;
-                    excl += v[q] & kOsCount;
-                    ++k;
-                    if ((v[q] >> 62) == 2) {
-                        done = true;
-                        break;
-                    }
-                }
-                if (done) break;
-                t -= k;  // tile 0 is always inclusive, so t stays >= 0
-                if (k < kOsWindow) {  // tile t is not published yet
-                    if (++spins > kOsSpinLimit) {  // cannot happen while every claimed tile runs; never hang
-                        atomicOr(gave_up, 1u);
-                        s_bad = 1;
-                        break;
-                    }
-                    __nanosleep(64);
-                }
-            }
-            st_relaxed_u64(status + (size_t)tile * kDigits + dd, kOsIncl | tag | ((excl + cnt[r]) & kOsCount));
-        }
-        s_gbase[dd] = digit_base[r] + excl;
-    }
-    __syncthreads();
-    uint32_t lower = 0;  // items of the tile in the digits owned before this pass of r
-#pragma unroll
-    for (int r = 0; r < kPer; ++r) {
-        uint32_t before = lower;
-        for (int w = 0; w < wid; ++w) before += s_wsum[r][w];
-        s_tstart[tid + r * kOsThreads] = before + x[r] - cnt[r];
-#pragma unroll
-        for (int w = 0; w < kOsWarps; ++w) lower += s_wsum[r][w];
     }
     __syncthreads();
     // the tile in shared memory in digit order
 #pragma unroll
     for (int c = 0; c < kOsItems; ++c) {
-        if (wb + c * 32 + lane < n) {
-            const uint32_t d = (uint32_t)((key[c] >> shift) & kMask);
-            const uint32_t pos = s_tstart[d] + s_wcnt[wid][d] + rnk[c];
+        if (32 * c < left) {
+            const uint32_t pos = reinterpret_cast<const uint16_t*>(s_wcnt[wid])[rnk[c] >> 16] + (rnk[c] & 0xFFFFu);
             s_keys[pos] = key[c];
             s_vals[pos] = val[c];
         }
+    }
+    // (the keys' registers are free, and the earlier tiles have had the placement's
+    // time to publish) look back over them for the owned digit's items before the
+    // tile, kOsWindow tiles a read: sum their own counts back to the first
+    // inclusive prefix, waiting on the first tile not yet published
+    if (owner) {
+        unsigned long long excl = 0;
+        int64_t t = (int64_t)tile - 1;  // the next tile to account for
+        uint32_t spins = 0;
+        bool done = tile == 0;
+        while (!done) {
+            unsigned long long v[kOsWindow];
+#pragma unroll
+            for (int k = 0; k < kOsWindow; ++k)
+                v[k] = t - k >= 0 ? ld_relaxed_u64(status + (size_t)(t - k) * kDigits + tid) : 0;
+            int k = 0;
+#pragma unroll
+            for (int q = 0; q < kOsWindow; ++q) {
+                const bool ready = (v[q] & (63ull << 56)) == tag && (v[q] >> 62) != 0;
+                if (!ready) break;
+                excl += v[q] & kOsCount;
+                ++k;
+                if ((v[q] >> 62) == 2) {
+                    done = true;
+                    break;
+                }
+            }
+            if (done) break;
+            t -= k;  // tile 0 is always inclusive, so t stays >= 0
+            if (k < kOsWindow) {  // tile t is not published yet
+                if (++spins > kOsSpinLimit) {  // cannot happen while every claimed tile runs; never hang
+                    atomicOr(gave_up, 1u);
+                    s_bad = 1;
+                    break;
+                }
+                __nanosleep(32);
+            }
+        }
+        if (tile > 0)
+            st_relaxed_u64(status + (size_t)tile * kDigits + tid, kOsIncl | tag | ((excl + cnt) & kOsCount));
+        s_out[tid] = (uint32_t)(digit_base + excl) - start;  // positions are below 2^32
     }
     __syncthreads();
     if (s_bad) return;  // offsets unknown: write nothing (the host reports the failure)
     const int tile_n = (int)min((int64_t)kOsTile, n - t0);
     for (int i = tid; i < tile_n; i += kOsThreads) {
         const uint64_t k = s_keys[i];
-        const uint32_t d = (uint32_t)((k >> shift) & kMask);
-        const unsigned long long g = s_gbase[d] + (unsigned long long)(i - (int)s_tstart[d]);
-        if (g >= (unsigned long long)n) {  // inconsistent counts (cannot happen): never write out of bounds
+        const uint32_t g = s_out[(uint32_t)((k >> shift) & kMask)] + (uint32_t)i;
+        if ((int64_t)g >= n) {  // inconsistent counts (cannot happen): never write out of bounds
             atomicOr(gave_up, 2u);
             continue;
         }
