@@ -336,37 +336,46 @@ static int estimate_call(const char* name, skis_sketch* s, int32_t num_queries, 
         if (off[b + 1] < off[b]) return fail(SKIS_EINVAL, where + ": seed offsets decrease");
     if (off[num_queries] > 0 && !seeds) return fail(SKIS_EINVAL, where + ": seeds is NULL");
     std::string err;
-    auto run = [&](const int64_t* d_off, const int32_t* d_seeds, int64_t* d_cov, double* d_est) {
+    // exch: the sharded form (its own status copy); pack: one copy back of status and answers
+    auto run = [&](const int64_t* d_off, const int32_t* d_seeds, int64_t* d_cov, double* d_est, void* d_pack,
+                   void* h_pack, size_t bytes) {
         return exch ? sketch_estimate_sharded(s, num_queries, d_off, d_seeds, off.data(), d_cov, d_est, exch, fn, ctx,
                                               st, &err)
-                    : sketch_estimate(s, num_queries, d_off, d_seeds, off.data(), d_cov, d_est, st, &err);
+                    : sketch_estimate(s, num_queries, d_off, d_seeds, off.data(), d_cov, d_est, st, &err, d_pack,
+                                      h_pack, bytes);
     };
     int rc;
     if (mem_space == SKIS_MEM_DEVICE) {
-        rc = run(seed_offsets, seeds, coverage_out, estimate_out);
+        rc = run(seed_offsets, seeds, coverage_out, estimate_out, nullptr, nullptr, 0);
     } else {
-        const int64_t nseeds = off[num_queries];
-        int64_t* d_off = nullptr;
-        int32_t* d_seeds = nullptr;
-        int64_t* d_cov = nullptr;
-        double* d_est = nullptr;
-        API_CUDA(name, dev_alloc_t(&d_off, (size_t)num_queries + 1, st));
-        API_CUDA(name, dev_alloc_t(&d_seeds, (size_t)std::max<int64_t>(nseeds, 1), st));
-        API_CUDA(name, dev_alloc_t(&d_cov, (size_t)num_queries, st));
-        API_CUDA(name, dev_alloc_t(&d_est, (size_t)num_queries, st));
-        API_CUDA(name, cudaMemcpyAsync(d_off, off.data(), (num_queries + 1) * 8, cudaMemcpyHostToDevice, st));
-        if (nseeds) API_CUDA(name, cudaMemcpyAsync(d_seeds, seeds, nseeds * 4, cudaMemcpyHostToDevice, st));
-        rc = run(d_off, d_seeds, d_cov, d_est);
-        if (rc == SKIS_OK) {
-            if (coverage_out)
-                API_CUDA(name, cudaMemcpyAsync(coverage_out, d_cov, num_queries * 8, cudaMemcpyDeviceToHost, st));
-            API_CUDA(name, cudaMemcpyAsync(estimate_out, d_est, num_queries * 8, cudaMemcpyDeviceToHost, st));
-            API_CUDA(name, cudaStreamSynchronize(st));
-        }
-        dev_free(d_off, st);
-        dev_free(d_seeds, st);
-        dev_free(d_cov, st);
-        dev_free(d_est, st);
+        // one device buffer: the status, the answers (these come back together),
+        // the offsets and the seeds
+        const size_t q = (size_t)num_queries, nseeds = (size_t)off[num_queries];
+        const size_t pack = sizeof(DevStatus) + 16 * q;
+        unsigned char* buf = nullptr;
+        API_CUDA(name, dev_alloc((void**)&buf, pack + (q + 1) * 8 + nseeds * 4, st));
+        double* d_est = reinterpret_cast<double*>(buf + sizeof(DevStatus));
+        int64_t* d_cov = reinterpret_cast<int64_t*>(d_est + q);
+        int64_t* d_off = d_cov + q;
+        int32_t* d_seeds = reinterpret_cast<int32_t*>(d_off + q + 1);
+        std::vector<unsigned char> back(pack);
+        auto body = [&]() -> int {
+            API_CUDA(name, cudaMemcpyAsync(d_off, off.data(), (q + 1) * 8, cudaMemcpyHostToDevice, st));
+            if (nseeds) API_CUDA(name, cudaMemcpyAsync(d_seeds, seeds, nseeds * 4, cudaMemcpyHostToDevice, st));
+            const int r = run(d_off, d_seeds, d_cov, d_est, exch ? nullptr : buf, back.data(), pack);
+            if (r != SKIS_OK) return fail(r, err);
+            if (exch) {
+                API_CUDA(name, cudaMemcpyAsync(back.data(), buf, pack, cudaMemcpyDeviceToHost, st));
+                API_CUDA(name, cudaStreamSynchronize(st));
+            }
+            return SKIS_OK;
+        };
+        rc = body();
+        dev_free(buf, st);
+        if (rc != SKIS_OK) return rc;
+        const unsigned char* ans = back.data() + sizeof(DevStatus);
+        std::copy(ans, ans + 8 * q, reinterpret_cast<unsigned char*>(estimate_out));
+        if (coverage_out) std::copy(ans + 8 * q, ans + 16 * q, reinterpret_cast<unsigned char*>(coverage_out));
     }
     if (rc != SKIS_OK) return fail(rc, err);
     return SKIS_OK;

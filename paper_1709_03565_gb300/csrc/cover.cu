@@ -22,53 +22,50 @@ namespace skis {
 constexpr int kCovThreads = 256;
 
 // Calls f(owner_lane, member) for every member of the samples held by the
-// lanes (lane i: arena offset off, length len), spread over the warp.
+// lanes (lane i: arena offset off, length len), spread over the warp: the
+// members laid end to end, kRuns runs of 32 a pass with their loads in flight
+// together, each lane finding the sample that holds its member by a search of
+// the prefix sums.
 template <int kRuns = 2, class F>
 __device__ __forceinline__ void warp_members(uint64_t off, uint32_t len, const int32_t* __restrict__ arena, F&& f) {
-    static_assert(kRuns == 1 || kRuns == 2, "one or two runs of 32 members per pass");
     const int lane = threadIdx.x & 31;
-    uint64_t incl = len;
+    uint64_t sum = len;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-        const uint64_t y = __shfl_up_sync(kFull, incl, d);
-        if (lane >= d) incl += y;
+        const uint64_t y = __shfl_up_sync(kFull, sum, d);
+        if (lane >= d) sum += y;
     }
-    const uint64_t total = __shfl_sync(kFull, incl, 31);
-    const uint64_t excl = incl - len;
-    if constexpr (kRuns == 1) {
-        for (uint64_t base = 0; base < total; base += 32) {
-            const uint64_t p = base + lane;
-            int owner = 0;
-#pragma unroll
-            for (int step = 16; step >= 1; step >>= 1) {
-                const uint64_t v = __shfl_sync(kFull, incl, owner + step - 1);
-                if (v <= p) owner += step;
-            }
-            const uint64_t o_off = __shfl_sync(kFull, off, owner);
-            const uint64_t o_excl = __shfl_sync(kFull, excl, owner);
-            if (p < total) f(owner, arena[o_off + (p - o_excl)]);
+    const uint64_t all = __shfl_sync(kFull, sum, 31);
+    if (all >= (1ull << 32) - 32 * kRuns) {  // past 32-bit places: one sample after another
+        for (int o = 0; o < 32; ++o) {
+            const uint64_t o_off = __shfl_sync(kFull, off, o);
+            const uint32_t o_len = __shfl_sync(kFull, len, o);
+            for (uint64_t i = lane; i < o_len; i += 32) f(o, arena[o_off + i]);
         }
-    } else {
-        // two runs of 32 members per pass: both member loads are in flight
-        // before either member is handed to f
-        for (uint64_t base = 0; base < total; base += 64) {
-            const uint64_t p0 = base + lane, p1 = base + 32 + lane;
-            int own0 = 0, own1 = 0;
+        return;
+    }
+    const uint32_t incl = (uint32_t)sum, total = (uint32_t)all;
+    const uint64_t rel = off - (incl - len);  // + a member's place: its arena position
+    for (uint32_t base = 0; base < total; base += 32 * kRuns) {
+        int own[kRuns];
+        int32_t u[kRuns];
 #pragma unroll
-            for (int step = 16; step >= 1; step >>= 1) {
-                const uint64_t v0 = __shfl_sync(kFull, incl, own0 + step - 1);
-                const uint64_t v1 = __shfl_sync(kFull, incl, own1 + step - 1);
-                if (v0 <= p0) own0 += step;
-                if (v1 <= p1) own1 += step;
-            }
-            const uint64_t off0 = __shfl_sync(kFull, off, own0), ex0 = __shfl_sync(kFull, excl, own0);
-            const uint64_t off1 = __shfl_sync(kFull, off, own1), ex1 = __shfl_sync(kFull, excl, own1);
-            int32_t u0 = 0, u1 = 0;
-            if (p0 < total) u0 = arena[off0 + (p0 - ex0)];
-            if (p1 < total) u1 = arena[off1 + (p1 - ex1)];
-            if (p0 < total) f(own0, u0);
-            if (p1 < total) f(own1, u1);
+        for (int k = 0; k < kRuns; ++k) own[k] = 0;
+#pragma unroll
+        for (int step = 16; step >= 1; step >>= 1)
+#pragma unroll
+            for (int k = 0; k < kRuns; ++k)
+                if (__shfl_sync(kFull, incl, own[k] + step - 1) <= base + 32 * k + lane) own[k] += step;
+#pragma unroll
+        for (int k = 0; k < kRuns; ++k) {
+            const uint64_t o_rel = __shfl_sync(kFull, rel, own[k]);
+            const uint32_t p = base + 32 * k + lane;
+            u[k] = 0;
+            if (p < total) u[k] = arena[o_rel + p];
         }
+#pragma unroll
+        for (int k = 0; k < kRuns; ++k)
+            if (base + 32 * k + lane < total) f(own[k], u[k]);
     }
 }
 
@@ -119,8 +116,9 @@ __device__ __forceinline__ uint32_t filter_index(uint32_t v, int hashed) {
 }
 __global__ void k_qmask_set(const int64_t* __restrict__ off, const int32_t* __restrict__ seeds, int32_t q0,
                             int32_t qn, int64_t n, uint64_t* __restrict__ qmask, uint32_t* __restrict__ qbits,
-                            DevStatus* st) {
+                            DevStatus* st, unsigned long long* __restrict__ reset3) {
     const int lane = threadIdx.x & 31;
+    if (reset3 && blockIdx.x == 0 && threadIdx.x < 3) reset3[threadIdx.x] = 0;  // the ordered scan's counters
     const int32_t b = q0 + (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (b >= q0 + qn) return;
     const int64_t lo = off[b], hi = off[b + 1];
@@ -144,28 +142,17 @@ __global__ void k_qmask_set(const int64_t* __restrict__ off, const int32_t* __re
     }
 }
 
-__global__ void k_qmask_clear(const int64_t* __restrict__ off, const int32_t* __restrict__ seeds, int32_t q0,
-                              int32_t qn, int64_t n, uint64_t* __restrict__ qmask, uint32_t* __restrict__ qbits,
-                              unsigned long long* __restrict__ reset2) {
-    const int lane = threadIdx.x & 31;
-    if (reset2 && blockIdx.x == 0 && threadIdx.x < 3) reset2[threadIdx.x] = 0;  // the ordered scan's counters
-    const int32_t b = q0 + (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    if (b >= q0 + qn) return;
-    for (int64_t i = off[b] + lane; i < off[b + 1]; i += 32) {
-        const int32_t v = seeds[i];
-        if (v >= 0 && v < n) {
-            qmask[v] = 0;
-            // every bit set in the filter belongs to a seed of this batch
-            if (qbits) qbits[filter_index((uint32_t)v, n > ((int64_t)1 << kFilterLog2)) >> 5] = 0;
-        }
-    }
-}
-
+// A warp takes 2^glog consecutive samples at a time. Bound by the chain of
+// header, member and filter loads of the longest group: with 32 samples a warp
+// a small sketch left most warp slots empty (ER 10k / 100k, 100K samples, 60
+// members on average and up to 1,700: 3,125 groups for 9,728 slots, 76 us), so
+// a group is only as large as keeps every slot supplied (coverage_shape), and
+// four runs of 32 members are in flight.
 __global__ void __launch_bounds__(kCovThreads) k_coverage(const uint64_t* __restrict__ h_off,
                                                           const uint32_t* __restrict__ h_len, uint64_t T,
                                                           const int32_t* __restrict__ arena,
                                                           const uint64_t* __restrict__ qmask,
-                                                          const uint32_t* __restrict__ qbits, int hashed,
+                                                          const uint32_t* __restrict__ qbits, int hashed, int glog,
                                                           unsigned long long* __restrict__ cov) {
     __shared__ unsigned long long s_acc[kCovThreads / 32][32];
     __shared__ unsigned long long s_cnt[64];
@@ -174,25 +161,29 @@ __global__ void __launch_bounds__(kCovThreads) k_coverage(const uint64_t* __rest
     __syncthreads();
     unsigned long long c_lo = 0, c_hi = 0;  // counts of queries `lane` and `lane + 32`
     const uint64_t nwarps = (uint64_t)gridDim.x * (kCovThreads / 32);
-    const uint64_t groups = (T + 31) / 32;
+    const uint64_t groups = (T + (1u << glog) - 1) >> glog;
+    unsigned long long* acc_row = s_acc[wib];
     for (uint64_t gidx = (uint64_t)blockIdx.x * (kCovThreads / 32) + wib; gidx < groups; gidx += nwarps) {
-        const uint64_t j = gidx * 32 + lane;
-        const bool valid = j < T;
+        const uint64_t j = (gidx << glog) + lane;
+        const bool valid = lane < (1 << glog) && j < T;
         const uint64_t off = valid ? h_off[j] : 0;
         const uint32_t len = valid ? h_len[j] : 0;
-        s_acc[wib][lane] = 0;
+        acc_row[lane] = 0;
         __syncwarp();
-        unsigned long long* acc_row = s_acc[wib];
-        warp_members(off, len, arena, [&](int owner, int32_t u) {
+        bool hit = false;
+        warp_members<4>(off, len, arena, [&](int owner, int32_t u) {
             if (qbits) {  // not a seed
                 const uint32_t f = filter_index((uint32_t)u, hashed);
                 if (!((__ldg(qbits + (f >> 5)) >> (f & 31)) & 1u)) return;
             }
             const uint64_t msk = qmask[u];
-            if (msk) atomicOr(&acc_row[owner], (unsigned long long)msk);
+            if (msk) {
+                atomicOr(&acc_row[owner], (unsigned long long)msk);
+                hit = true;
+            }
         });
-        __syncwarp();
-        const uint64_t acc = s_acc[wib][lane];
+        if (!__any_sync(kFull, hit)) continue;
+        const uint64_t acc = acc_row[lane];
         uint64_t present = acc;
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) present |= __shfl_xor_sync(kFull, present, d);
@@ -349,22 +340,13 @@ __global__ void __launch_bounds__(256) k_scan_hits(const unsigned long long* __r
     if (threadIdx.x < 64 && s_cnt[threadIdx.x]) atomicAdd(&cov[threadIdx.x], (unsigned long long)s_cnt[threadIdx.x]);
 }
 
-__global__ void k_unmark(const uint32_t* __restrict__ touched, const unsigned long long* __restrict__ ntouched,
-                         unsigned long long* __restrict__ smask) {
-    const uint64_t cnt = *ntouched;
-    for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < cnt; k += (uint64_t)gridDim.x * blockDim.x)
-        smask[touched[k]] = 0;
-}
-
 // Eq. 21 with exact integers: N = Cov W + T sum_{v in S} (2^f - w_v),
-// D = T 2^f, estimate = N / D.
-__global__ void k_estimate(const int64_t* __restrict__ off, const int32_t* __restrict__ seeds, int32_t q0,
-                           int32_t qn, int64_t n, const uint64_t* __restrict__ w, int f, uint64_t W, uint64_t T,
-                           const unsigned long long* __restrict__ cov, int64_t* __restrict__ cov_out,
-                           double* __restrict__ est_out, int ris) {
+// D = T 2^f, estimate = N / D, of query b by one warp (Cov = c).
+__device__ __forceinline__ void estimate_query(const int64_t* __restrict__ off, const int32_t* __restrict__ seeds,
+                                               int32_t b, int64_t n, const uint64_t* __restrict__ w, int f, uint64_t W,
+                                               uint64_t T, uint64_t c, int64_t* __restrict__ cov_out,
+                                               double* __restrict__ est_out, int ris) {
     const int lane = threadIdx.x & 31;
-    const int32_t b = q0 + (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    if (b >= q0 + qn) return;
     const uint64_t one_f = 1ull << f;
     uint64_t s = 0;  // <= |S| 2^f <= 2^61
     for (int64_t i = off[b] + lane; i < off[b + 1]; i += 32) {
@@ -374,12 +356,55 @@ __global__ void k_estimate(const int64_t* __restrict__ off, const int32_t* __res
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) s += __shfl_down_sync(kFull, s, d);
     if (lane == 0) {
-        const uint64_t c = cov[b - q0];
         // RIS (Lemma 1): n Cov / T; SKIS (Eq. 21): (Cov W + T sum) / (T 2^f)
         const u128 N = ris ? (u128)c * (uint64_t)n : (u128)c * W + (u128)T * s;
         const u128 D = ris ? (u128)T : (u128)T << f;
         if (cov_out) cov_out[b] = (int64_t)c;
         est_out[b] = u128_to_double(N) / u128_to_double(D);
+    }
+}
+
+__global__ void k_estimate(const int64_t* __restrict__ off, const int32_t* __restrict__ seeds, int32_t q0,
+                           int32_t qn, int64_t n, const uint64_t* __restrict__ w, int f, uint64_t W, uint64_t T,
+                           const unsigned long long* __restrict__ cov, int64_t* __restrict__ cov_out,
+                           double* __restrict__ est_out, int ris) {
+    const int32_t b = q0 + (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (b >= q0 + qn) return;
+    estimate_query(off, seeds, b, n, w, f, W, T, cov[b - q0], cov_out, est_out, ris);
+}
+
+// The end of a batch of queries, a warp each: the estimate, and everything the
+// batch set goes back to zero (its seeds' masks and filter bits, its coverage
+// counts and, by the blocks past the queries', the samples' query words).
+// status_out (nullable) receives the status word.
+__global__ void k_finish(const int64_t* __restrict__ off, const int32_t* __restrict__ seeds, int32_t q0, int32_t qn,
+                         int64_t n, const uint64_t* __restrict__ w, int f, uint64_t W, uint64_t T,
+                         unsigned long long* __restrict__ cov, int64_t* __restrict__ cov_out,
+                         double* __restrict__ est_out, int ris, uint64_t* __restrict__ qmask,
+                         uint32_t* __restrict__ qbits, int qblocks, const uint32_t* __restrict__ touched,
+                         const unsigned long long* __restrict__ ntouched, unsigned long long* __restrict__ smask,
+                         const DevStatus* __restrict__ status, DevStatus* __restrict__ status_out) {
+    if ((int)blockIdx.x >= qblocks) {
+        const uint64_t cnt = *ntouched;
+        for (uint64_t k = (uint64_t)(blockIdx.x - qblocks) * blockDim.x + threadIdx.x; k < cnt;
+             k += (uint64_t)(gridDim.x - qblocks) * blockDim.x)
+            smask[touched[k]] = 0;
+        return;
+    }
+    if (status_out && blockIdx.x == 0 && threadIdx.x == 0) *status_out = *status;
+    const int lane = threadIdx.x & 31;
+    const int32_t b = q0 + (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (b >= q0 + qn) return;
+    const uint64_t c = cov[b - q0];
+    estimate_query(off, seeds, b, n, w, f, W, T, c, cov_out, est_out, ris);
+    if (lane == 0) cov[b - q0] = 0;
+    for (int64_t i = off[b] + lane; i < off[b + 1]; i += 32) {
+        const int32_t v = seeds[i];
+        if (v >= 0 && v < n) {
+            qmask[v] = 0;
+            // every bit set in the filter belongs to a seed of this batch
+            if (qbits) qbits[filter_index((uint32_t)v, n > ((int64_t)1 << kFilterLog2)) >> 5] = 0;
+        }
     }
 }
 
@@ -396,6 +421,17 @@ static int coverage_blocks(uint64_t T) {
     const uint64_t groups = (T + 31) / 32;
     const uint64_t want = (groups + (kCovThreads / 32) - 1) / (kCovThreads / 32);
     return (int)std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)sm_count() * 8));
+}
+
+// k_coverage's grid and group size: the largest groups (at most 32 samples)
+// that still give two to each of the GPU's warps.
+void coverage_shape(uint64_t T, int* blocks, int* glog) {
+    const uint64_t warps = (uint64_t)sm_count() * 8 * (kCovThreads / 32);
+    *glog = 5;
+    while (*glog > 0 && (T >> *glog) < 2 * warps) --*glog;
+    const uint64_t groups = (T + (1u << *glog) - 1) >> *glog;
+    const uint64_t want = (groups + kCovThreads / 32 - 1) / (kCovThreads / 32);
+    *blocks = (int)std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)sm_count() * 8));
 }
 
 // ------------------------------------------- coverage by inverted index
@@ -564,7 +600,8 @@ int sketch_order_arena(skis_sketch* s, cudaStream_t st, std::string* err) {
 }
 
 int sketch_estimate(skis_sketch* s, int32_t q, const int64_t* d_off, const int32_t* d_seeds, const int64_t* h_off,
-                    int64_t* d_cov, double* d_est, cudaStream_t st, std::string* err) {
+                    int64_t* d_cov, double* d_est, cudaStream_t st, std::string* err, void* d_pack, void* h_pack,
+                    size_t pack_bytes) {
     const char* where = "skis_estimate";
     const skis_graph* g = s->g;
     if (s->T == 0) {
@@ -591,8 +628,12 @@ int sketch_estimate(skis_sketch* s, int32_t q, const int64_t* d_off, const int32
         CV_CUDA(cudaMemsetAsync(s->qmask, 0, (size_t)g->n * sizeof(uint64_t), st));
         CV_CUDA(dev_alloc_t(&s->qbits, (size_t)fwords, st));
         CV_CUDA(cudaMemsetAsync(s->qbits, 0, (size_t)fwords * sizeof(uint32_t), st));
+        // coverage counts and status, zero (first_bad all ones) between calls
         CV_CUDA(dev_alloc_t(&s->qcov, 64, st));
         CV_CUDA(dev_alloc_t(&s->qstatus, 1, st));
+        CV_CUDA(cudaMemsetAsync(s->qcov, 0, 64 * sizeof(unsigned long long), st));
+        CV_CUDA(cudaMemsetAsync(s->qstatus, 0, sizeof(DevStatus), st));
+        CV_CUDA(cudaMemsetAsync(&s->qstatus->first_bad, 0xFF, sizeof(unsigned long long), st));
         CV_CUDA(cudaEventCreate(&s->qev[0]));
         CV_CUDA(cudaEventCreate(&s->qev[1]));
     }
@@ -602,9 +643,8 @@ int sketch_estimate(skis_sketch* s, int32_t q, const int64_t* d_off, const int32
         dev_free(s->touched, st);
         s->touched = nullptr;
         CV_CUDA(dev_alloc_t(&s->touched, (size_t)s->T, st));
-        if (!s->ntouched) {  // list count, task cursor and hit count, zero between calls (k_qmask_clear resets them)
+        if (!s->ntouched) {  // list count, task cursor and hit count (k_qmask_set resets them)
             CV_CUDA(dev_alloc_t(&s->ntouched, 3, st));
-            CV_CUDA(cudaMemsetAsync(s->ntouched, 0, 3 * sizeof(unsigned long long), st));
             CV_CUDA(dev_alloc_t(&s->hits, (size_t)kHitCap, st));
         }
         s->touched_cap = s->T;
@@ -628,15 +668,14 @@ int sketch_estimate(skis_sketch* s, int32_t q, const int64_t* d_off, const int32
     if (ordered_scan)  // the filter takes up to 128 KiB of dynamic shared memory
         CV_CUDA(cudaFuncSetAttribute(k_scan_ordered, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)(kFilterMaxWords * sizeof(uint32_t))));
-    CV_CUDA(cudaMemsetAsync(s->qstatus, 0, sizeof(DevStatus), st));
-    CV_CUDA(cudaMemsetAsync(&s->qstatus->first_bad, 0xFF, sizeof(unsigned long long), st));
-    const int cblocks = coverage_blocks(s->T);
+    int cblocks = 0, glog = 0;
+    coverage_shape(s->T, &cblocks, &glog);
     float query_ms = 0;
     for (int32_t q0 = 0; q0 < q; q0 += 64) {
         const int32_t qn = std::min<int32_t>(64, q - q0);
         const int wb = div_up((int64_t)qn * 32, 256);
-        CV_CUDA(cudaMemsetAsync(s->qcov, 0, 64 * sizeof(unsigned long long), st));
-        k_qmask_set<<<wb, 256, 0, st>>>(d_off, d_seeds, q0, qn, g->n, s->qmask, s->qbits, s->qstatus); note_launch();
+        k_qmask_set<<<wb, 256, 0, st>>>(d_off, d_seeds, q0, qn, g->n, s->qmask, s->qbits, s->qstatus,
+                                        ordered_scan ? s->ntouched : nullptr); note_launch();
         CV_CUDA(cudaGetLastError());
         CV_CUDA(cudaEventRecord(s->qev[0], st));
         if (by_index) {
@@ -654,34 +693,34 @@ int sketch_estimate(skis_sketch* s, int32_t q, const int64_t* d_off, const int32
                                                         s->touched, s->ntouched, s->qcov);
             note_launch();
             CV_CUDA(cudaGetLastError());
-            k_unmark<<<sm_count() * 4, 256, 0, st>>>(s->touched, s->ntouched,
-                                                     reinterpret_cast<unsigned long long*>(s->smask));
-            note_launch();
-            CV_CUDA(cudaGetLastError());
         } else {
             k_coverage<<<cblocks, kCovThreads, 0, st>>>(s->h_off, s->h_len, s->T, s->arena, s->qmask, s->qbits, hashed,
-                                                        s->qcov);
+                                                        glog, s->qcov);
             note_launch();
             CV_CUDA(cudaGetLastError());
         }
         CV_CUDA(cudaEventRecord(s->qev[1], st));
-        k_estimate<<<wb, 256, 0, st>>>(d_off, d_seeds, q0, qn, g->n, g->w, g->f, g->W, s->T, s->qcov, d_cov, d_est,
-                                       s->ris); note_launch();
-        CV_CUDA(cudaGetLastError());
-        k_qmask_clear<<<wb, 256, 0, st>>>(d_off, d_seeds, q0, qn, g->n, s->qmask, s->qbits,
-                                          ordered_scan ? s->ntouched : nullptr); note_launch();
+        k_finish<<<wb + (ordered_scan ? sm_count() : 0), 256, 0, st>>>(
+            d_off, d_seeds, q0, qn, g->n, g->w, g->f, g->W, s->T, s->qcov, d_cov, d_est, s->ris, s->qmask, s->qbits, wb,
+            s->touched, s->ntouched, reinterpret_cast<unsigned long long*>(s->smask), s->qstatus,
+            static_cast<DevStatus*>(d_pack));
+        note_launch();
         CV_CUDA(cudaGetLastError());
     }
     dev_free(chunk_cnt, st);
     dev_free(chunk_off, st);
     DevStatus h;
-    CV_CUDA(cudaMemcpyAsync(&h, s->qstatus, sizeof(DevStatus), cudaMemcpyDeviceToHost, st));
+    if (d_pack) CV_CUDA(cudaMemcpyAsync(h_pack, d_pack, pack_bytes, cudaMemcpyDeviceToHost, st));
+    else CV_CUDA(cudaMemcpyAsync(&h, s->qstatus, sizeof(DevStatus), cudaMemcpyDeviceToHost, st));
     CV_CUDA(cudaStreamSynchronize(st));
+    if (d_pack) h = *static_cast<const DevStatus*>(h_pack);
     if (q > 0 && q <= 64) {  // the device time of the coverage launches (one chunk of queries)
         cudaEventElapsedTime(&query_ms, s->qev[0], s->qev[1]);
         s->last_query_ms = query_ms;
     }
     if (h.flags & kStInval) {
+        CV_CUDA(cudaMemsetAsync(s->qstatus, 0, sizeof(DevStatus), st));
+        CV_CUDA(cudaMemsetAsync(&s->qstatus->first_bad, 0xFF, sizeof(unsigned long long), st));
         *err = "skis_estimate: query " + std::to_string(h.first_bad) +
                " is empty, has a seed outside [0, n) or repeats a seed";
         return SKIS_EINVAL;

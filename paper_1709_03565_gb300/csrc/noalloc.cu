@@ -108,13 +108,10 @@ extern "C" int skis_estimate_noalloc(const skis_sketch* s, int32_t num_queries, 
     if (e != cudaSuccess) return noalloc_fail(error_buf, error_len, SKIS_ERR_CUDA, "skis_estimate_noalloc: ", cudaGetErrorString(e));
 
     const int wb = (int)((num_queries * 32 + 255) / 256);
-    const uint64_t groups = (s->T + 31) / 32;
-    uint64_t cb = (groups + 7) / 8;
-    const uint64_t cap = (uint64_t)sm_count() * 8;
-    if (cb > cap) cb = cap;
-    if (cb < 1) cb = 1;
-    k_qmask_set<<<wb, 256, 0, st>>>(seed_offsets, seeds, 0, num_queries, g->n, qmask, nullptr, status); note_launch();
-    k_coverage<<<(unsigned)cb, 256, 0, st>>>(s->h_off, s->h_len, s->T, s->arena, qmask, nullptr, 0, qcov); note_launch();
+    int cb = 0, glog = 0;
+    coverage_shape(s->T, &cb, &glog);
+    k_qmask_set<<<wb, 256, 0, st>>>(seed_offsets, seeds, 0, num_queries, g->n, qmask, nullptr, status, nullptr); note_launch();
+    k_coverage<<<cb, 256, 0, st>>>(s->h_off, s->h_len, s->T, s->arena, qmask, nullptr, 0, glog, qcov); note_launch();
     k_estimate<<<wb, 256, 0, st>>>(seed_offsets, seeds, 0, num_queries, g->n, g->w, g->f, g->W, s->T, qcov,
                                    coverage_out, estimate_out, s->ris); note_launch();
     e = cudaGetLastError();

@@ -373,8 +373,12 @@ namespace skis {
 int sketch_sample(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* err);
 int sketch_sample_to_size(skis_sketch* s, uint64_t target, uint64_t max_count, cudaStream_t st, uint64_t* appended,
                           std::string* err);
+// d_pack (nullable): a device buffer whose first word receives the call's
+// DevStatus and whose pack_bytes come back to h_pack in the one copy that ends
+// the call (d_cov and d_est may lie in it).
 int sketch_estimate(skis_sketch* s, int32_t q, const int64_t* d_off, const int32_t* d_seeds, const int64_t* h_off,
-                    int64_t* d_cov, double* d_est, cudaStream_t st, std::string* err);
+                    int64_t* d_cov, double* d_est, cudaStream_t st, std::string* err, void* d_pack = nullptr,
+                    void* h_pack = nullptr, size_t pack_bytes = 0);
 int sketch_greedy(skis_sketch* s, int32_t k, int32_t* h_seeds, int64_t* h_cov, double* h_est, cudaStream_t st,
                   std::string* err);
 // Eq. 21 and Alg. 3 over a sketch split by sample id across ranks; exch is
@@ -410,13 +414,12 @@ int set_last_error(int code, const std::string& msg);
 // Coverage kernels (defined in cover.cu).
 __global__ void k_qmask_set(const int64_t* __restrict__ off, const int32_t* __restrict__ seeds, int32_t q0,
                             int32_t qn, int64_t n, uint64_t* __restrict__ qmask, uint32_t* __restrict__ qbits,
-                            DevStatus* st);
-__global__ void k_qmask_clear(const int64_t* __restrict__ off, const int32_t* __restrict__ seeds, int32_t q0,
-                              int32_t qn, int64_t n, uint64_t* __restrict__ qmask, uint32_t* __restrict__ qbits,
-                              unsigned long long* __restrict__ reset2);
+                            DevStatus* st, unsigned long long* __restrict__ reset3);
 __global__ void __launch_bounds__(256) k_coverage(const uint64_t* __restrict__ h_off, const uint32_t* __restrict__ h_len, uint64_t T,
                            const int32_t* __restrict__ arena, const uint64_t* __restrict__ qmask,
-                           const uint32_t* __restrict__ qbits, int hashed, unsigned long long* __restrict__ cov);
+                           const uint32_t* __restrict__ qbits, int hashed, int glog,
+                           unsigned long long* __restrict__ cov);
+void coverage_shape(uint64_t T, int* blocks, int* glog);
 __global__ void k_estimate(const int64_t* __restrict__ off, const int32_t* __restrict__ seeds, int32_t q0,
                            int32_t qn, int64_t n, const uint64_t* __restrict__ w, int f, uint64_t W, uint64_t T,
                            const unsigned long long* __restrict__ cov, int64_t* __restrict__ cov_out,
