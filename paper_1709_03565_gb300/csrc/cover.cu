@@ -391,7 +391,10 @@ __global__ void k_finish(const int64_t* __restrict__ off, const int32_t* __restr
             smask[touched[k]] = 0;
         return;
     }
-    if (status_out && blockIdx.x == 0 && threadIdx.x == 0) *status_out = *status;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (status_out) *status_out = *status;
+        cov[64] = 0;  // the index walk's queue
+    }
     const int lane = threadIdx.x & 31;
     const int32_t b = q0 + (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (b >= q0 + qn) return;
@@ -437,82 +440,145 @@ void coverage_shape(uint64_t T, int* blocks, int* glog) {
 // ------------------------------------------- coverage by inverted index
 // Cov_R(S) for small seed sets: walk the sample list of every seed and set
 // the query's bit in a per-sample mask; the first setter of (sample, query)
-// counts it. Lists are cut into chunks of kInvChunk entries; one warp takes
-// one chunk, found by binary search over the batch's chunk prefix sums.
-constexpr uint32_t kInvChunk = 2048;
+// counts it. A warp takes a seed and the first kInvChunk entries of its list;
+// the further chunks of a long list (a hub's) are queued and dealt over the
+// grid by the next launch, or, past the queue's capacity, walked on the spot.
+// Bound by latency: seed, list bounds, list and mask are one dependent load
+// after another, so the lists are short work in many warps, four entries a
+// lane in flight. 64 queries, 13,800 seeds, lists of 93 entries on average
+// (Chung-Lu 4M / 70M WC, 5M samples): set and reset 117 us with a chunk table,
+// its prefix sums and a search of it per chunk of 2048, in seven launches; 154,
+// 66 and 50 us like this with chunks of 2048, 512 and 256.
+constexpr uint32_t kInvChunk = 256;
 
-__global__ void k_seed_chunks(const int32_t* __restrict__ seeds, int64_t seed_base, int64_t nseeds, int64_t n,
-                              const uint64_t* __restrict__ inv_off, uint32_t* __restrict__ chunk_cnt) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nseeds; i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t v = seeds[seed_base + i];
-        uint32_t c = 0;
-        if (v >= 0 && v < n) c = (uint32_t)((inv_off[v + 1] - inv_off[v] + kInvChunk - 1) / kInvChunk);
-        chunk_cnt[i] = c;
-    }
-}
+struct InvWalk {
+    const int64_t* off;     // the batch's seed offsets and seeds
+    const int32_t* seeds;
+    int32_t q0, qn;
+    int64_t seed_base, nseeds, n;
+    const uint64_t* inv_off;
+    const uint32_t* inv;
+    unsigned long long* smask;
+    unsigned long long* cov;      // qn counts
+    uint64_t* queue;              // seed << 32 | chunk
+    uint64_t queue_cap;
+    unsigned long long* nqueue;   // chunks queued or past the capacity
+};
 
-__global__ void __launch_bounds__(kCovThreads) k_cover_inv(const int64_t* __restrict__ off,
-                                                           const int32_t* __restrict__ seeds, int32_t q0, int32_t qn,
-                                                           int64_t seed_base, int64_t nseeds,
-                                                           const uint64_t* __restrict__ chunk_off,
-                                                           const uint64_t* __restrict__ inv_off,
-                                                           const uint32_t* __restrict__ inv,
-                                                           uint64_t* __restrict__ smask,
-                                                           unsigned long long* __restrict__ cov, int clear) {
-    const int lane = threadIdx.x & 31;
-    const uint64_t C = chunk_off[nseeds];
-    const uint64_t nwarps = (uint64_t)gridDim.x * (blockDim.x / 32);
-    for (uint64_t c = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32; c < C; c += nwarps) {
-        int64_t lo = 0, hi = nseeds - 1;  // last seed i with chunk_off[i] <= c
-        while (lo < hi) {
-            const int64_t mid = (lo + hi + 1) / 2;
-            if (chunk_off[mid] <= c) lo = mid;
-            else hi = mid - 1;
-        }
-        const int64_t i = lo;
-        int32_t blo = q0, bhi = q0 + qn - 1;  // last query b with off[b] <= seed_base + i
-        while (blo < bhi) {
-            const int32_t mid = (blo + bhi + 1) / 2;
-            if (off[mid] <= seed_base + i) blo = mid;
-            else bhi = mid - 1;
-        }
-        const uint64_t bit = 1ull << (blo - q0);
-        const int32_t v = seeds[seed_base + i];
-        const uint64_t start = inv_off[v] + (c - chunk_off[i]) * kInvChunk;
-        const uint64_t end = min(start + kInvChunk, inv_off[v + 1]);
-        uint32_t fresh = 0;
-        for (uint64_t x = start + lane; x < end; x += 32) {
-            const uint32_t j = inv[x];
-            if (clear) {
-                smask[j] = 0;
-            } else {
-                const unsigned long long old = atomicOr((unsigned long long*)&smask[j], (unsigned long long)bit);
-                fresh += (old & bit) ? 0u : 1u;
+// Sets `bit` in the masks of list entries [x0, x1) (clear: zeroes the masks);
+// returns how many masks of the lane's entries did not have it.
+__device__ __forceinline__ uint32_t walk_list(const InvWalk& a, uint64_t x0, uint64_t x1, unsigned long long bit, bool clear) {
+    uint32_t fresh = 0;
+    for (uint64_t x = x0 + (threadIdx.x & 31); x < x1; x += 128) {
+        uint32_t j[4];
+        unsigned long long old[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (x + 32 * q < x1) j[q] = a.inv[x + 32 * q];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            old[q] = bit;
+            if (x + 32 * q < x1) {
+                if (clear) a.smask[j[q]] = 0;
+                else old[q] = atomicOr(&a.smask[j[q]], bit);
             }
         }
-        if (!clear) {
 #pragma unroll
-            for (int d = 16; d > 0; d >>= 1) fresh += __shfl_down_sync(kFull, fresh, d);
-            if (lane == 0 && fresh) atomicAdd(&cov[blo - q0], (unsigned long long)fresh);
+        for (int q = 0; q < 4; ++q) fresh += (old[q] & bit) ? 0u : 1u;
+    }
+    return fresh;
+}
+
+// mode 0: the lists' first chunks (the others queued); 1: the queued chunks;
+// 2: every mask they set back to zero
+__global__ void __launch_bounds__(kCovThreads) k_cover_inv(InvWalk a, int mode) {
+    __shared__ int64_t s_off[65];
+    __shared__ unsigned int s_cov[64];
+    const int lane = threadIdx.x & 31;
+    for (int i = threadIdx.x; i <= a.qn; i += kCovThreads) s_off[i] = a.off[a.q0 + i];
+    if (threadIdx.x < 64) s_cov[threadIdx.x] = 0;
+    __syncthreads();
+    auto query_of = [&](int64_t i) -> int {  // the last query b with off[b] <= seed_base + i
+        int lo = 0, hi = a.qn - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) / 2;
+            if (s_off[mid] <= a.seed_base + i) lo = mid;
+            else hi = mid - 1;
+        }
+        return lo;
+    };
+    auto add = [&](int b, uint32_t fresh) {
+        fresh = __reduce_add_sync(kFull, fresh);
+        if (lane == 0 && fresh) atomicAdd(&s_cov[b], fresh);
+    };
+    const int64_t nwarps = (int64_t)gridDim.x * (kCovThreads / 32);
+    const int64_t w0 = ((int64_t)blockIdx.x * kCovThreads + threadIdx.x) / 32;
+    const uint64_t queued = mode ? min((uint64_t)*a.nqueue, a.queue_cap) : 0;
+    const bool past = mode == 2 && *a.nqueue > a.queue_cap;
+    if (mode != 1) {
+        for (int64_t i = w0; i < a.nseeds; i += nwarps) {
+            const int32_t v = a.seeds[a.seed_base + i];
+            if (v < 0 || v >= a.n) continue;
+            const uint64_t lo = a.inv_off[v], len = a.inv_off[v + 1] - lo;
+            const int b = query_of(i);
+            const unsigned long long bit = 1ull << b;
+            uint64_t rest = len;  // entries [rest, len) are walked here as well
+            if (len > kInvChunk) {
+                if (mode == 2) {
+                    if (past) rest = kInvChunk;  // whichever were queued, all of it
+                } else {
+                    const uint64_t more = (len - 1) / kInvChunk;
+                    unsigned long long at = 0;
+                    if (lane == 0) at = atomicAdd(a.nqueue, (unsigned long long)more);
+                    at = __shfl_sync(kFull, at, 0);
+                    const uint64_t fit = at < a.queue_cap ? min(more, (uint64_t)(a.queue_cap - at)) : 0;
+                    for (uint64_t c = lane; c < fit; c += 32) a.queue[at + c] = ((uint64_t)i << 32) | (c + 1);
+                    rest = min(len, (fit + 1) * kInvChunk);
+                }
+            }
+            uint32_t fresh = walk_list(a, lo, lo + min(len, (uint64_t)kInvChunk), bit, mode == 2);
+            if (rest < len) fresh += walk_list(a, lo + rest, lo + len, bit, mode == 2);
+            if (mode == 0) add(b, fresh);
         }
     }
+    for (uint64_t k = w0; k < queued; k += nwarps) {
+        const uint64_t item = a.queue[k];
+        const int64_t i = (int64_t)(item >> 32);
+        const int32_t v = a.seeds[a.seed_base + i];
+        const uint64_t x = a.inv_off[v] + (item & 0xFFFFFFFFu) * kInvChunk;
+        const int b = query_of(i);
+        const uint32_t fresh = walk_list(a, x, min(x + kInvChunk, a.inv_off[v + 1]), 1ull << b, mode == 2);
+        if (mode == 1) add(b, fresh);
+    }
+    if (mode == 2) return;
+    __syncthreads();
+    if (threadIdx.x < 64 && s_cov[threadIdx.x]) atomicAdd(&a.cov[threadIdx.x], (unsigned long long)s_cov[threadIdx.x]);
 }
 
 cudaError_t coverage_by_index(const skis_sketch* s, const int64_t* off, const int32_t* seeds, int32_t q0,
-                              int32_t qn, int64_t seed_base, int64_t nseeds, uint32_t* chunk_cnt,
-                              uint64_t* chunk_off, uint64_t* smask, unsigned long long* cov, cudaStream_t st) {
+                              int32_t qn, int64_t seed_base, int64_t nseeds, uint64_t* queue, uint64_t queue_cap,
+                              uint64_t* smask, unsigned long long* cov, cudaStream_t st) {
     if (nseeds <= 0) return cudaSuccess;
-    const int b1 = (int)std::max<int64_t>(1, std::min<int64_t>((nseeds + 255) / 256, (int64_t)sm_count() * 4));
-    k_seed_chunks<<<b1, 256, 0, st>>>(seeds, seed_base, nseeds, s->g->n, s->inv_off, chunk_cnt); note_launch();
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    e = scan_u32_to_u64(chunk_cnt, chunk_off, nseeds, st);
-    if (e != cudaSuccess) return e;
-    const int b2 = sm_count() * 8;
-    k_cover_inv<<<b2, kCovThreads, 0, st>>>(off, seeds, q0, qn, seed_base, nseeds, chunk_off, s->inv_off, s->inv,
-                                            smask, cov, 0); note_launch();
-    k_cover_inv<<<b2, kCovThreads, 0, st>>>(off, seeds, q0, qn, seed_base, nseeds, chunk_off, s->inv_off, s->inv,
-                                            smask, cov, 1); note_launch();
+    InvWalk a;
+    a.off = off;
+    a.seeds = seeds;
+    a.q0 = q0;
+    a.qn = qn;
+    a.seed_base = seed_base;
+    a.nseeds = nseeds;
+    a.n = s->g->n;
+    a.inv_off = s->inv_off;
+    a.inv = s->inv;
+    a.smask = reinterpret_cast<unsigned long long*>(smask);
+    a.cov = cov;
+    a.queue = queue;
+    a.queue_cap = queue_cap;
+    a.nqueue = cov + 64;
+    const int full = sm_count() * 8;
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((nseeds + kCovThreads / 32 - 1) / (kCovThreads / 32), full));
+    k_cover_inv<<<blocks, kCovThreads, 0, st>>>(a, 0); note_launch();
+    k_cover_inv<<<full, kCovThreads, 0, st>>>(a, 1); note_launch();
+    k_cover_inv<<<full, kCovThreads, 0, st>>>(a, 2); note_launch();
     return cudaGetLastError();
 }
 
@@ -628,17 +694,18 @@ int sketch_estimate(skis_sketch* s, int32_t q, const int64_t* d_off, const int32
         CV_CUDA(cudaMemsetAsync(s->qmask, 0, (size_t)g->n * sizeof(uint64_t), st));
         CV_CUDA(dev_alloc_t(&s->qbits, (size_t)fwords, st));
         CV_CUDA(cudaMemsetAsync(s->qbits, 0, (size_t)fwords * sizeof(uint32_t), st));
-        // coverage counts and status, zero (first_bad all ones) between calls
-        CV_CUDA(dev_alloc_t(&s->qcov, 64, st));
+        // coverage counts, the index walk's queue length and the status, zero
+        // (first_bad all ones) between calls
+        CV_CUDA(dev_alloc_t(&s->qcov, 65, st));
         CV_CUDA(dev_alloc_t(&s->qstatus, 1, st));
-        CV_CUDA(cudaMemsetAsync(s->qcov, 0, 64 * sizeof(unsigned long long), st));
+        CV_CUDA(cudaMemsetAsync(s->qcov, 0, 65 * sizeof(unsigned long long), st));
         CV_CUDA(cudaMemsetAsync(s->qstatus, 0, sizeof(DevStatus), st));
         CV_CUDA(cudaMemsetAsync(&s->qstatus->first_bad, 0xFF, sizeof(unsigned long long), st));
         CV_CUDA(cudaEventCreate(&s->qev[0]));
         CV_CUDA(cudaEventCreate(&s->qev[1]));
     }
-    uint32_t* chunk_cnt = nullptr;
-    uint64_t* chunk_off = nullptr;
+    uint64_t* queue = nullptr;
+    uint64_t queue_cap = 0;
     if (ordered_scan && s->touched_cap < s->T) {
         dev_free(s->touched, st);
         s->touched = nullptr;
@@ -662,8 +729,8 @@ int sketch_estimate(skis_sketch* s, int32_t q, const int64_t* d_off, const int32
         int64_t most = 1;
         for (int32_t q0 = 0; q0 < q; q0 += 64)
             most = std::max<int64_t>(most, h_off[std::min<int32_t>(q, q0 + 64)] - h_off[q0]);
-        CV_CUDA(dev_alloc_t(&chunk_cnt, (size_t)most, st));
-        CV_CUDA(dev_alloc_t(&chunk_off, (size_t)most + 1, st));
+        queue_cap = (uint64_t)most + kInvQueueExtra;
+        CV_CUDA(dev_alloc_t(&queue, (size_t)queue_cap, st));
     }
     if (ordered_scan)  // the filter takes up to 128 KiB of dynamic shared memory
         CV_CUDA(cudaFuncSetAttribute(k_scan_ordered, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -679,8 +746,8 @@ int sketch_estimate(skis_sketch* s, int32_t q, const int64_t* d_off, const int32
         CV_CUDA(cudaGetLastError());
         CV_CUDA(cudaEventRecord(s->qev[0], st));
         if (by_index) {
-            CV_CUDA(coverage_by_index(s, d_off, d_seeds, q0, qn, h_off[q0], h_off[q0 + qn] - h_off[q0], chunk_cnt,
-                                      chunk_off, s->smask, s->qcov, st));
+            CV_CUDA(coverage_by_index(s, d_off, d_seeds, q0, qn, h_off[q0], h_off[q0 + qn] - h_off[q0], queue,
+                                      queue_cap, s->smask, s->qcov, st));
         } else if (ordered_scan) {
             k_scan_ordered<<<sm_count(), kScanThreads, fwords * sizeof(uint32_t), st>>>(
                 s->h_off, s->h_len, s->T, s->arena, s->qbits, fwords, hashed, s->qmask,
@@ -707,8 +774,7 @@ int sketch_estimate(skis_sketch* s, int32_t q, const int64_t* d_off, const int32
         note_launch();
         CV_CUDA(cudaGetLastError());
     }
-    dev_free(chunk_cnt, st);
-    dev_free(chunk_off, st);
+    dev_free(queue, st);
     DevStatus h;
     if (d_pack) CV_CUDA(cudaMemcpyAsync(h_pack, d_pack, pack_bytes, cudaMemcpyDeviceToHost, st));
     else CV_CUDA(cudaMemcpyAsync(&h, s->qstatus, sizeof(DevStatus), cudaMemcpyDeviceToHost, st));

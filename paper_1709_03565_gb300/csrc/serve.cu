@@ -38,8 +38,7 @@ struct Slot {
     int64_t* d_cov = nullptr;
     double* d_est = nullptr;
     uint64_t* d_smask = nullptr;   // T per-sample query bits, zero between batches
-    uint32_t* d_chunk_cnt = nullptr;
-    uint64_t* d_chunk_off = nullptr;
+    uint64_t* d_queue = nullptr;   // chunks of long sample lists
     unsigned long long* d_qcov = nullptr;
     DevStatus* d_status = nullptr;
     std::vector<uint64_t> tickets;
@@ -92,8 +91,7 @@ static void release_slot(Slot& sl) {
     cudaFree(sl.d_cov);
     cudaFree(sl.d_est);
     cudaFree(sl.d_smask);
-    cudaFree(sl.d_chunk_cnt);
-    cudaFree(sl.d_chunk_off);
+    cudaFree(sl.d_queue);
     cudaFree(sl.d_qcov);
     cudaFree(sl.d_status);
     if (sl.done) cudaEventDestroy(sl.done);
@@ -150,9 +148,8 @@ extern "C" int skis_server_create(skis_server** out, skis_sketch* s, int32_t slo
             chk(dev_malloc((void**)&sl.d_cov, 64 * sizeof(int64_t)));
             chk(dev_malloc((void**)&sl.d_est, 64 * sizeof(double)));
             chk(dev_malloc((void**)&sl.d_smask, (size_t)s->T * sizeof(uint64_t)));
-            chk(dev_malloc((void**)&sl.d_chunk_cnt, seed_capacity * sizeof(uint32_t)));
-            chk(dev_malloc((void**)&sl.d_chunk_off, (seed_capacity + 1) * sizeof(uint64_t)));
-            chk(dev_malloc((void**)&sl.d_qcov, 64 * sizeof(unsigned long long)));
+            chk(dev_malloc((void**)&sl.d_queue, (seed_capacity + kInvQueueExtra) * sizeof(uint64_t)));
+            chk(dev_malloc((void**)&sl.d_qcov, 65 * sizeof(unsigned long long)));
             chk(dev_malloc((void**)&sl.d_status, sizeof(DevStatus)));
             if (e == cudaSuccess) e = cudaMemsetAsync(sl.d_smask, 0, (size_t)s->T * sizeof(uint64_t), sl.stream);
             if (e == cudaSuccess) e = cudaStreamSynchronize(sl.stream);
@@ -218,10 +215,10 @@ static int launch_batch(skis_server* srv, Slot& sl) {
     cudaStream_t st = sl.stream;
     SV_CUDA(cudaMemcpyAsync(sl.d_off, sl.h_off, (size_t)(q + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, st));
     SV_CUDA(cudaMemcpyAsync(sl.d_seeds, sl.h_seeds, used * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-    SV_CUDA(cudaMemsetAsync(sl.d_qcov, 0, 64 * sizeof(unsigned long long), st));
+    SV_CUDA(cudaMemsetAsync(sl.d_qcov, 0, 65 * sizeof(unsigned long long), st));
     SV_CUDA(cudaMemsetAsync(sl.d_status, 0, sizeof(DevStatus), st));
     const int wb = (q * 32 + 255) / 256;
-    SV_CUDA(coverage_by_index(s, sl.d_off, sl.d_seeds, 0, q, 0, (int64_t)used, sl.d_chunk_cnt, sl.d_chunk_off,
+    SV_CUDA(coverage_by_index(s, sl.d_off, sl.d_seeds, 0, q, 0, (int64_t)used, sl.d_queue, srv->seed_cap + kInvQueueExtra,
                               sl.d_smask, sl.d_qcov, st));
     k_estimate<<<wb, 256, 0, st>>>(sl.d_off, sl.d_seeds, 0, q, g->n, g->w, g->f, g->W, s->T, sl.d_qcov, sl.d_cov,
                                    sl.d_est, s->ris); note_launch();

@@ -358,7 +358,7 @@ struct skis_sketch {
     uint64_t smask_cap = 0;
     uint64_t* qmask = nullptr;           // n per-vertex query bits
     uint32_t* qbits = nullptr;           // n bits: the vertex is a seed of the current batch
-    unsigned long long* qcov = nullptr;  // 64 coverage counters
+    unsigned long long* qcov = nullptr;  // 64 coverage counters, the index walk's queue length
     uint32_t* touched = nullptr;         // ordered scan: samples whose query word was set (for the reset)
     unsigned long long* ntouched = nullptr;  // [0] touched count, [1] task cursor, [2] hit count
     unsigned long long* hits = nullptr;      // ordered scan: (task, position) of members that may be seeds
@@ -397,10 +397,12 @@ int sketch_order_arena(skis_sketch* s, cudaStream_t st, std::string* err);
 int sketch_inverted(skis_sketch* s, cudaStream_t st, std::string* err);
 // Coverage of queries [q0, q0 + qn) of a CSR batch through the inverted
 // index: cov[b - q0] = #samples meeting S_b. smask (T words, all zero on
-// entry) is restored to zero; chunk_cnt/chunk_off hold nseeds (+1) entries.
+// entry) is restored to zero; cov holds 65 words, zero on entry (the last one
+// counts the queue of long lists' chunks, which holds queue_cap entries).
+constexpr uint64_t kInvQueueExtra = 1u << 19;  // callers' queues hold one chunk a seed and this many more
 cudaError_t coverage_by_index(const skis_sketch* s, const int64_t* off, const int32_t* seeds, int32_t q0,
-                              int32_t qn, int64_t seed_base, int64_t nseeds, uint32_t* chunk_cnt,
-                              uint64_t* chunk_off, uint64_t* smask, unsigned long long* cov, cudaStream_t st);
+                              int32_t qn, int64_t seed_base, int64_t nseeds, uint64_t* queue, uint64_t queue_cap,
+                              uint64_t* smask, unsigned long long* cov, cudaStream_t st);
 void sketch_release(skis_sketch* s);
 int sketch_autotune(skis_sketch* s, uint64_t pilot, cudaStream_t st, double* cand_ms, int cand_cap, int* ncand,
                     std::string* err);
