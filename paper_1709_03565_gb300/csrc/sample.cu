@@ -1286,32 +1286,47 @@ __global__ void __launch_bounds__(kCtaThreads, 1024 / kCtaThreads) k_iis_cta(Sam
 // sums P, none when y >= P_d); the walk ends when none is picked or the
 // picked vertex is already in R_j. Step t of sample j draws the Philox block
 // (q = t, domain LT, sample j): step 0 conditioned (64-bit U, y = floor(U S
-// / 2^64)), later steps y = its word 0. Two tiers: one lane per sample with
-// up to kLtQ members in shared memory, then one warp per CTA-tier slot with
-// the slot's global visited bitmap and queue.
+// / 2^64)), later steps y = its word 0. Three tiers: a lane a walk with up to
+// kLtQ members in shared memory, a lane a walk with up to kLtMidCap members in
+// global memory, then one warp per CTA-tier slot with the slot's global
+// visited bitmap and queue.
+// A step is a chain of two loads (the vertex's row, the picked in-neighbour);
+// the next row is loaded while the visited check runs. The lane tiers keep
+// their warps together: walks start and end in batches of kLtRefill lanes or
+// more, and members are written out by the whole warp. Bound by that chain, at
+// the slowest of 32 lanes' gathers about 1 us each. 2M samples of Chung-Lu 1M /
+// 10M WC (18 members on average, 6 % of the walks above kLtQ): first tier 1.51
+// -> .64 ms, second 1.13 -> .62; 500K of ER 10k / 100k (125 members) 1.2 (three
+// passes) -> .29 and 24.5 -> 3.1. Batches of 4 or 12 lanes: within 2 %, of 1:
+// .74 and .67; kLtQ 64 or 96 in blocks of 128: .96 and 1.10 for the first tier.
 constexpr int kLtBlock = 256;
 constexpr int kLtQ = 48;
+constexpr int kLtRefill = 8;
 
 __device__ __forceinline__ uint64_t lt_weight(uint32_t tau) { return tau == kSentinel ? (1ull << 32) : (uint64_t)tau; }
 
-// one walk step from a vertex with in-row rw: the picked in-neighbour, or -1
-// when the walk ends there
+// step t of sample j from a vertex with in-row rw: the picked in-neighbour, or
+// -1 when the walk ends there
 __device__ __forceinline__ int32_t lt_step(const SampleArgs& a, uint64_t j, uint32_t t, const RowInfo& rw) {
     if (rw.deg == 0) return -1;
-    const uint64_t base = a.lt_cum ? a.lt_cum[rw.off] : 0;
-    const uint64_t S = a.lt_cum ? a.lt_cum[rw.off + rw.deg] - base : (uint64_t)rw.deg * lt_weight(rw.tau);
     const uint4 b = coin_block(a.rk, t, 0, kDomLt, j);
-    uint64_t y;
-    if (t == 0 && !a.ris) {
-        y = __umul64hi((uint64_t)b.x | ((uint64_t)b.y << 32), S);  // Pr[u] = w(u, v) / gamma_v
-    } else {
-        y = b.x;
-        if (y >= S) return -1;  // no in-edge kept
-    }
+    const uint64_t U = (uint64_t)b.x | ((uint64_t)b.y << 32);
+    const bool cond = t == 0 && !a.ris;
     uint32_t i;
-    if (!a.lt_cum) {
-        i = (uint32_t)(y / lt_weight(rw.tau));
+    if (!a.lt_cum) {  // one weight w = tau a row, S = deg w
+        if (cond) {
+            i = (uint32_t)__umul64hi(U, rw.deg);  // floor(floor(U deg w / 2^64) / w)
+        } else if (rw.tau == kSentinel) {  // w = 2^32
+            i = 0;
+        } else {
+            if (b.x >= (uint64_t)rw.deg * rw.tau) return -1;  // no in-edge kept
+            i = b.x / rw.tau;
+        }
     } else {  // the first position whose running sum exceeds y
+        const uint64_t base = a.lt_cum[rw.off];
+        const uint64_t S = a.lt_cum[rw.off + rw.deg] - base;
+        const uint64_t y = cond ? __umul64hi(U, S) : (uint64_t)b.x;  // cond: Pr[u] = w(u, v) / gamma_v
+        if (!cond && y >= S) return -1;  // no in-edge kept
         uint32_t lo = 0, hi = rw.deg - 1;
         while (lo < hi) {
             const uint32_t mid = (lo + hi) >> 1;
@@ -1323,184 +1338,310 @@ __device__ __forceinline__ int32_t lt_step(const SampleArgs& a, uint64_t j, uint
     return a.src[rw.off + i];
 }
 
-__global__ void __launch_bounds__(kLtBlock) k_lt_walk(SampleArgs a) {
-    __shared__ int32_t s_q[kLtBlock / 32][kLtQ][32];
+__device__ __forceinline__ uint32_t warp_incl_sum(uint32_t x) {
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, x, d);
+        if ((threadIdx.x & 31) >= d) x += y;
+    }
+    return x;
+}
+
+// the lane whose run holds place idx of runs laid end to end (incl: this
+// lane's inclusive end); all lanes call it
+__device__ __forceinline__ int warp_owner(uint32_t incl, uint32_t idx) {
+    int owner = 0;
+#pragma unroll
+    for (int step = 16; step > 0; step >>= 1)
+        if (__shfl_sync(kFull, incl, owner + step - 1) <= idx) owner += step;
+    return owner;
+}
+
+__device__ __forceinline__ void lt_header(const SampleArgs& a, uint64_t j, uint64_t at, uint32_t len, uint32_t v,
+                                          uint64_t coins) {
+    a.h_off[j - a.id_base] = at;
+    a.h_len[j - a.id_base] = len;
+    a.h_src[j - a.id_base] = v;
+    a.h_retries[j - a.id_base] = 0;
+    a.h_coins[j - a.id_base] = coins;
+}
+
+// The members of a lane's walk stand four to a 16-byte word, the words of a
+// lane one column further right each, so that a lane compares four members a
+// load and the warp reads one walk's members, both without bank conflicts. A
+// new member whose hashed bit (of 128) is clear needs no search.
+__global__ void __launch_bounds__(kLtBlock, 4) k_lt_walk(SampleArgs a) {
+    __shared__ int4 s_q[kLtBlock / 32][kLtQ / 4][32];
     const int lane = threadIdx.x & 31;
-    int32_t(*const mq)[32] = s_q[threadIdx.x >> 5];  // mq[k][lane]: member k of this lane's sample
+    int4* const words = s_q[threadIdx.x >> 5][0];
+    int32_t* const flat = reinterpret_cast<int32_t*>(words);
+    auto word = [](int l, uint32_t c) { return c * 32 + (((uint32_t)l + c) & 31u); };
     const uint64_t count = input_count(a);
-    bool busy = false, exhausted = false;
-    uint64_t j = 0, coins = 0;
+    bool busy = false, done = false, exhausted = false;
+    uint64_t j = 0, coins = 0, sig0 = 0, sig1 = 0;
     uint32_t v = 0, len = 0, t = 0;
-    int32_t x = 0;
+    RowInfo row = {};
+    // up to 32 sources drawn together, one a lane
+    uint64_t pool_base = 0;
+    uint32_t pool_n = 0, pool_used = 0, p_v = 0;
+    RowInfo p_row = {};
     uint64_t chunk_pos = 0, chunk_end = 0;
     uint32_t chunk = kLaneArenaChunk;
 
+    auto add = [&](int32_t u) {  // member len of this lane's walk
+        const uint32_t h = ((uint32_t)u * 0x9E3779B9u) >> 25;
+        const uint64_t bit = 1ull << (h & 63u);
+        if (h < 64u) sig0 |= bit;
+        else sig1 |= bit;
+        const uint32_t w = word(lane, len >> 2);
+        if ((len & 3u) == 0) words[w] = make_int4(u, -1, -1, -1);
+        else flat[4 * w + (len & 3u)] = u;
+        ++len;
+    };
+
     for (;;) {
-        const unsigned idle = __ballot_sync(kFull, !busy);
-        if (idle && !exhausted) {
-            const int leader = __ffs(idle) - 1;
-            unsigned long long base = 0;
-            if (lane == leader) base = atomicAdd(a.work, (unsigned long long)__popc(idle));
-            base = __shfl_sync(kFull, base, leader);
-            if (base + __popc(idle) >= count) exhausted = true;
-            if (!busy) {
+        const unsigned dn = __ballot_sync(kFull, done);
+        const unsigned free_l = __ballot_sync(kFull, !busy || done);
+        if (__popc(free_l) >= kLtRefill || free_l == kFull) {
+            if (dn) {
+                const uint32_t mylen = done ? len : 0u;
+                const uint32_t incl = warp_incl_sum(mylen);
+                const uint32_t total = __shfl_sync(kFull, incl, 31);
+                bool fits = true;
+                if (chunk_end - chunk_pos < total) {
+                    const uint64_t size = max((uint64_t)chunk, (uint64_t)total);
+                    unsigned long long base = 0;
+                    if (lane == 0) base = atomicAdd(a.arena_cursor, (unsigned long long)size);
+                    base = __shfl_sync(kFull, base, 0);
+                    if (base + size > a.arena_cap) {
+                        fits = false;
+                        chunk = 0;
+                        chunk_pos = chunk_end = 0;
+                    } else {
+                        chunk_pos = base;
+                        chunk_end = base + size;
+                    }
+                }
+                if (done) {
+                    if (fits) lt_header(a, j, chunk_pos + (incl - mylen), len, v, coins);
+                    else arena_overflow(a, j);
+                    busy = done = false;
+                }
+                __syncwarp();
+                if (fits) {
+                    for (uint32_t b0 = 0; b0 < total; b0 += 32) {
+                        const uint32_t idx = b0 + (uint32_t)lane;
+                        const int owner = warp_owner(incl, idx);
+                        const uint32_t i = idx - __shfl_sync(kFull, incl - mylen, owner);
+                        if (idx < total) {
+                            const int32_t u = flat[4 * word(owner, i >> 2) + (i & 3u)];
+                            a.arena[chunk_pos + idx] = u;
+                            count_member(a, u);
+                        }
+                    }
+                    chunk_pos += total;
+                }
+                __syncwarp();
+            }
+            unsigned idle = __ballot_sync(kFull, !busy);
+            while (idle && !exhausted) {
+                if (pool_used == pool_n) {
+                    unsigned long long base = 0;
+                    if (lane == 0) base = atomicAdd(a.work, 32ull);
+                    base = __shfl_sync(kFull, base, 0);
+                    if (base >= count) {
+                        exhausted = true;
+                        break;
+                    }
+                    pool_base = base;
+                    pool_n = (uint32_t)min((unsigned long long)32, count - base);
+                    pool_used = 0;
+                    if ((uint32_t)lane < pool_n) {
+                        p_v = draw_source<true>(a, input_id(a, base + lane));
+                        p_row = a.rows[p_v];
+                    }
+                }
+                const uint32_t take = min((uint32_t)__popc(idle), pool_n - pool_used);
+                const uint32_t rank = __popc(idle & lanemask_lt());
+                const int from = (int)min(pool_used + rank, 31u);
+                const uint32_t n_v = __shfl_sync(kFull, p_v, from);
+                RowInfo n_row;
+                n_row.off = shfl_u64(p_row.off, from);
+                n_row.deg = __shfl_sync(kFull, p_row.deg, from);
+                n_row.tau = __shfl_sync(kFull, p_row.tau, from);
+                if (!busy && rank < take) {
+                    j = input_id(a, pool_base + pool_used + rank);
+                    v = n_v;
+                    row = n_row;
+                    len = t = 0;
+                    coins = sig0 = sig1 = 0;
+                    busy = true;
+                    add((int32_t)v);
+                }
+                pool_used += take;
+                idle = __ballot_sync(kFull, !busy);
+            }
+            if (!__any_sync(kFull, busy)) {
+                if (exhausted) break;
+                continue;
+            }
+        }
+        if (!busy || done) continue;  // the lane waits for the next batch
+        coins += row.deg;
+        const int32_t u = lt_step(a, j, t, row);
+        ++t;
+        if (u < 0) {
+            done = true;
+            continue;
+        }
+        row = a.rows[u];  // in flight during the visited check
+        const uint32_t h = ((uint32_t)u * 0x9E3779B9u) >> 25;
+        bool seen = false;
+        if (((h < 64u ? sig0 : sig1) >> (h & 63u)) & 1ull) {
+            for (uint32_t c = 0; c * 4 < len && !seen; ++c) {
+                const int4 m = words[word(lane, c)];
+                seen = m.x == u || m.y == u || m.z == u || m.w == u;
+            }
+        }
+        if (seen) {
+            done = true;  // the walk closes on R_j
+        } else if (len == (uint32_t)kLtQ) {
+            hand_on(a, j);  // a long walk: the next tier redraws it
+            busy = false;
+        } else {
+            add(u);
+        }
+    }
+}
+
+// Medium LT walks: a lane a walk, its members listed in global memory and in
+// an open-addressing visited table there, at most half full. Which slots are
+// taken stands in a shared bitmap, which alone is cleared between walks, and a
+// second bitmap by another hash tells most new vertices: a slot is read only
+// where both bits are set (the tables of 77,824 lanes are 640 MB, so a read is
+// a DRAM latency for the whole warp: .78 ms without the second bitmap, .62 with
+// it, 1.13 with tables read at each probe and restored slot by slot). A walk
+// longer than kLtMidCap is handed on.
+constexpr int kLtMidBlock = 128;
+constexpr int kLtMidBlocks = 4;  // an SM: 48 KB of bitmaps a block
+constexpr uint32_t kLtMidHash = 2048;
+constexpr uint32_t kLtMidBloom = 1024;
+constexpr uint32_t kLtMidCap = 1024;
+
+__global__ void __launch_bounds__(kLtMidBlock) k_lt_mid(SampleArgs a, uint32_t* __restrict__ hash_all,
+                                                        int32_t* list_all) {
+    __shared__ uint32_t s_occ[kLtMidBlock / 32][(kLtMidHash + kLtMidBloom) / 32][32];
+    const int lane = threadIdx.x & 31;
+    const uint64_t me = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    uint32_t* const hash = hash_all + me * kLtMidHash;
+    int32_t* const list = list_all + me * kLtMidCap;
+    const int32_t* const warp_list = list_all + (me - lane) * kLtMidCap;
+    uint32_t(*const occ)[32] = s_occ[threadIdx.x >> 5];  // word w of this lane's bitmap: occ[w][lane]
+    uint32_t(*const bloom)[32] = occ + kLtMidHash / 32;
+    auto bloom_bit = [](uint32_t u) { return (u * 0x9E3779B9u) >> 22; };
+    static_assert(kLtMidBloom == 1u << 10, "bloom_bit: ten bits");
+    const uint64_t count = input_count(a);
+    bool busy = false, done = false, exhausted = false;
+    uint64_t j = 0, coins = 0;
+    uint32_t v = 0, len = 0, t = 0;
+    RowInfo row = {};
+
+    for (;;) {
+        const unsigned dn = __ballot_sync(kFull, done);
+        const unsigned free_l = __ballot_sync(kFull, !busy || done);
+        if (__popc(free_l) >= kLtRefill || free_l == kFull) {
+            if (dn) {
+                const uint32_t mylen = done ? len : 0u;
+                const uint32_t incl = warp_incl_sum(mylen);
+                const uint32_t total = __shfl_sync(kFull, incl, 31);
+                unsigned long long base = 0;
+                if (lane == 0) base = atomicAdd(a.arena_cursor, (unsigned long long)total);
+                base = __shfl_sync(kFull, base, 0);
+                const bool fits = base + total <= a.arena_cap;
+                if (done) {
+                    if (fits) lt_header(a, j, base + (incl - mylen), len, v, coins);
+                    else arena_overflow(a, j);
+                    busy = done = false;
+                }
+                __syncwarp();
+                for (uint32_t b0 = 0; fits && b0 < total; b0 += 128) {
+                    int32_t u[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {  // four loads in flight
+                        const uint32_t idx = b0 + 32 * k + (uint32_t)lane;
+                        const int owner = warp_owner(incl, idx);
+                        const uint32_t i = idx - __shfl_sync(kFull, incl - mylen, owner);
+                        u[k] = idx < total ? warp_list[owner * kLtMidCap + i] : 0;
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const uint32_t idx = b0 + 32 * k + (uint32_t)lane;
+                        if (idx < total) {
+                            a.arena[base + idx] = u[k];
+                            count_member(a, u[k]);
+                        }
+                    }
+                }
+                __syncwarp();
+            }
+            const unsigned idle = __ballot_sync(kFull, !busy);
+            if (!exhausted) {
+                unsigned long long base = 0;
+                if (lane == 0) base = atomicAdd(a.work, (unsigned long long)__popc(idle));
+                base = __shfl_sync(kFull, base, 0);
+                if (base + __popc(idle) >= count) exhausted = true;
                 const uint64_t ti = base + __popc(idle & lanemask_lt());
-                if (ti < count) {
+                if (!busy && ti < count) {
                     j = input_id(a, ti);
                     v = draw_source(a, j);
-                    x = (int32_t)v;
-                    mq[0][lane] = x;
+                    row = a.rows[v];
+#pragma unroll 8
+                    for (uint32_t w = 0; w < (kLtMidHash + kLtMidBloom) / 32; ++w) occ[w][lane] = 0;
+                    const uint32_t h = (v * 2654435761u) & (kLtMidHash - 1);
+                    occ[h >> 5][lane] = 1u << (h & 31u);
+                    const uint32_t b = bloom_bit(v);
+                    bloom[b >> 5][lane] = 1u << (b & 31u);
+                    hash[h] = v;
+                    list[0] = (int32_t)v;
                     len = 1;
                     t = 0;
                     coins = 0;
                     busy = true;
                 }
             }
+            if (!__any_sync(kFull, busy)) {
+                if (exhausted) break;
+                continue;
+            }
         }
-        if (!__any_sync(kFull, busy)) {
-            if (exhausted) break;
+        if (!busy || done) continue;  // the lane waits for the next batch
+        coins += row.deg;
+        const int32_t u = lt_step(a, j, t, row);
+        ++t;
+        if (u < 0) {
+            done = true;
             continue;
         }
-        bool done = false;
-        if (busy) {
-            const RowInfo rw = a.rows[x];
-            coins += rw.deg;
-            const int32_t u = lt_step(a, j, t, rw);
-            ++t;
-            if (u < 0) {
-                done = true;
-            } else {
-                bool seen = false;
-                for (uint32_t i = 0; i < len; ++i)
-                    if (mq[i][lane] == u) { seen = true; break; }
-                if (seen) {
-                    done = true;  // the walk closes on R_j
-                } else if (len == (uint32_t)kLtQ) {
-                    hand_on(a, j);  // a long walk: the slot tier redraws it
-                    busy = false;
-                } else {
-                    mq[len++][lane] = u;
-                    x = u;
-                }
-            }
+        row = a.rows[u];  // in flight during the visited check
+        uint32_t g = ((uint32_t)u * 2654435761u) & (kLtMidHash - 1);
+        const uint32_t b = bloom_bit((uint32_t)u);
+        const bool maybe = (bloom[b >> 5][lane] >> (b & 31u)) & 1u;
+        bool seen = false;
+        while ((occ[g >> 5][lane] >> (g & 31u)) & 1u) {  // the table is at most half full: the probe ends
+            if (maybe && hash[g] == (uint32_t)u) { seen = true; break; }
+            g = (g + 1) & (kLtMidHash - 1);
         }
-        const unsigned dm = __ballot_sync(kFull, done);
-        if (dm) {
-            const uint32_t mylen = done ? len : 0u;
-            uint32_t incl = mylen;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const uint32_t y = __shfl_up_sync(kFull, incl, d);
-                if (lane >= d) incl += y;
-            }
-            const uint32_t total = __shfl_sync(kFull, incl, 31);
-            bool fits = true;
-            if (chunk_end - chunk_pos < total) {
-                const uint64_t size = max((uint64_t)chunk, (uint64_t)total);
-                unsigned long long base = 0;
-                if (lane == 0) base = atomicAdd(a.arena_cursor, (unsigned long long)size);
-                base = __shfl_sync(kFull, base, 0);
-                if (base + size > a.arena_cap) {
-                    fits = false;
-                    chunk = 0;
-                    chunk_pos = chunk_end = 0;
-                } else {
-                    chunk_pos = base;
-                    chunk_end = base + size;
-                }
-            }
-            if (done) {
-                if (fits) {
-                    const uint64_t at = chunk_pos + (incl - mylen);
-                    for (uint32_t i = 0; i < len; ++i) {
-                        a.arena[at + i] = mq[i][lane];
-                        count_member(a, mq[i][lane]);
-                    }
-                    a.h_off[j - a.id_base] = at;
-                    a.h_len[j - a.id_base] = len;
-                    a.h_src[j - a.id_base] = v;
-                    a.h_retries[j - a.id_base] = 0;
-                    a.h_coins[j - a.id_base] = coins;
-                } else {
-                    arena_overflow(a, j);
-                }
-                busy = false;
-            }
-            if (fits) chunk_pos += total;
-        }
-    }
-}
-
-// Medium LT walks: one lane per walk with its own open-addressing visited
-// table (kLtMidHash slots, at most half full) and member list in global
-// memory; the table is restored to empty slot by slot after each walk. A
-// walk longer than kLtMidCap is handed on to the slot tier.
-constexpr int kLtMidBlock = 256;
-constexpr uint32_t kLtMidHash = 2048;
-constexpr uint32_t kLtMidCap = 1024;
-
-__global__ void __launch_bounds__(kLtMidBlock) k_lt_mid(SampleArgs a, uint32_t* __restrict__ hash_all,
-                                                        int32_t* __restrict__ list_all,
-                                                        uint32_t* __restrict__ slot_all) {
-    const uint64_t me = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    uint32_t* hash = hash_all + me * kLtMidHash;
-    int32_t* list = list_all + me * kLtMidCap;
-    uint32_t* slot = slot_all + me * kLtMidCap;
-    const uint64_t count = input_count(a);
-    for (;;) {
-        const unsigned long long ti = atomicAdd(a.work, 1ull);
-        if (ti >= count) break;
-        const uint64_t j = input_id(a, ti);
-        const uint32_t v = draw_source(a, j);
-        uint32_t len = 0;
-        bool over = false;
-        uint64_t coins = 0;
-        int32_t x = (int32_t)v;
-        for (uint32_t t = 0;; ++t) {  // each step adds a new member or ends the walk
-            // x joins the visited table and the list
-            uint32_t h = ((uint32_t)x * 2654435761u) & (kLtMidHash - 1);
-            while (hash[h] != kEmpty) h = (h + 1) & (kLtMidHash - 1);  // x is new: a free slot exists
-            hash[h] = (uint32_t)x;
-            slot[len] = h;
-            list[len++] = x;
-            const RowInfo rw = a.rows[x];
-            coins += rw.deg;
-            const int32_t u = lt_step(a, j, t, rw);
-            if (u < 0) break;
-            uint32_t g = ((uint32_t)u * 2654435761u) & (kLtMidHash - 1);
-            bool seen = false;
-            for (;;) {  // the table is at most half full: the probe ends
-                const uint32_t key = hash[g];
-                if (key == kEmpty) break;
-                if (key == (uint32_t)u) { seen = true; break; }
-                g = (g + 1) & (kLtMidHash - 1);
-            }
-            if (seen) break;
-            if (len == kLtMidCap) {
-                over = true;
-                break;
-            }
-            x = u;
-        }
-        if (over) {
+        if (seen) {
+            done = true;
+        } else if (len == kLtMidCap) {
             hand_on(a, j);
+            busy = false;
         } else {
-            const unsigned long long base = atomicAdd(a.arena_cursor, (unsigned long long)len);
-            if (base + len <= a.arena_cap) {
-                for (uint32_t i = 0; i < len; ++i) {
-                    a.arena[base + i] = list[i];
-                    count_member(a, list[i]);
-                }
-                a.h_off[j - a.id_base] = base;
-                a.h_len[j - a.id_base] = len;
-                a.h_src[j - a.id_base] = v;
-                a.h_retries[j - a.id_base] = 0;
-                a.h_coins[j - a.id_base] = coins;
-            } else {
-                arena_overflow(a, j);
-            }
+            occ[g >> 5][lane] |= 1u << (g & 31u);
+            bloom[b >> 5][lane] |= 1u << (b & 31u);
+            hash[g] = (uint32_t)u;
+            list[len++] = u;
         }
-        for (uint32_t i = 0; i < len; ++i) hash[slot[i]] = kEmpty;
     }
 }
 
@@ -1525,12 +1666,12 @@ __global__ void __launch_bounds__(32) k_lt_long(SampleArgs a) {
             bitmap[v >> 5] |= 1u << (v & 31);
             queue[0] = (int32_t)v;
             len = 1;
-            int32_t x = (int32_t)v;
+            RowInfo rw = a.rows[v];
             for (uint32_t t = 0;; ++t) {  // at most n steps: each adds a new member
-                const RowInfo rw = a.rows[x];
                 coins += rw.deg;
                 const int32_t u = lt_step(a, j, t, rw);
                 if (u < 0) break;
+                rw = a.rows[u];  // in flight during the visited check
                 const uint32_t bit = 1u << (u & 31);
                 if (bitmap[(uint32_t)u >> 5] & bit) break;
                 if (len == a.queue_cap) {  // the walk outgrew the slot's queue
@@ -1539,7 +1680,6 @@ __global__ void __launch_bounds__(32) k_lt_long(SampleArgs a) {
                 }
                 bitmap[(uint32_t)u >> 5] |= bit;
                 queue[len++] = u;
-                x = u;
             }
         }
         __syncwarp();
@@ -1666,12 +1806,10 @@ static int ensure_sample_buffers(skis_sketch* s, uint64_t count, uint64_t slack,
             else SK_CUDA(e);
         }
     }
-    if (g->lt && !s->lt_hash) {  // medium LT walks: one table, list and slot record per lane
-        s->lt_mid_lanes = (uint64_t)sm_count() * kLtMidBlock * 2;  // two blocks per SM
-        SK_CUDA(dev_alloc_t(&s->lt_hash, (size_t)(s->lt_mid_lanes * kLtMidHash), st));
-        SK_CUDA(cudaMemsetAsync(s->lt_hash, 0xFF, s->lt_mid_lanes * kLtMidHash * sizeof(uint32_t), st));
-        SK_CUDA(dev_alloc_t(&s->lt_list, (size_t)(s->lt_mid_lanes * kLtMidCap), st));
-        SK_CUDA(dev_alloc_t(&s->lt_slot, (size_t)(s->lt_mid_lanes * kLtMidCap), st));
+    if (g->lt) {  // medium LT walks: one table and list per lane
+        s->lt_mid_lanes = (uint64_t)sm_count() * kLtMidBlock * kLtMidBlocks;
+        if (!s->lt_hash) SK_CUDA(dev_alloc_t(&s->lt_hash, (size_t)(s->lt_mid_lanes * kLtMidHash), st));
+        if (!s->lt_list) SK_CUDA(dev_alloc_t(&s->lt_list, (size_t)(s->lt_mid_lanes * kLtMidCap), st));
     }
     if (warps > s->spill_warps) {  // warp tier: a spill slot a warp
         dev_free(s->spill_hash, st);
@@ -1880,7 +2018,7 @@ int sketch_sample(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* 
             k_lt_walk<<<lt_blocks, kLtBlock, 0, st>>>(at); note_launch();
             SK_CUDA(cudaGetLastError());
             SK_CUDA(cudaEventRecord(s->ev[1], st));
-            k_lt_mid<<<s->lt_mid_lanes / kLtMidBlock, kLtMidBlock, 0, st>>>(aw, s->lt_hash, s->lt_list, s->lt_slot);
+            k_lt_mid<<<s->lt_mid_lanes / kLtMidBlock, kLtMidBlock, 0, st>>>(aw, s->lt_hash, s->lt_list);
             note_launch();
             SK_CUDA(cudaGetLastError());
             SK_CUDA(cudaEventRecord(s->ev[2], st));

@@ -322,7 +322,6 @@ struct skis_sketch {
     int big_slots = 0;
     uint32_t* lt_hash = nullptr;         // LT medium walks: visited table per lane
     int32_t* lt_list = nullptr;          // LT medium walks: member list per lane
-    uint32_t* lt_slot = nullptr;         // LT medium walks: table slot of each listed member
     uint64_t lt_mid_lanes = 0;
     int cta_slots_alloc = 0;
     uint64_t bitmap_words = 0;
