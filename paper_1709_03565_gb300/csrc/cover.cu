@@ -12,7 +12,9 @@
 // Delta_v W + T (2^f - w_v) (ties to the lowest id), and the samples of the
 // chosen vertex are marked covered and their members' Delta decremented.
 #include <algorithm>
+#include <cstring>
 #include <string>
+#include <vector>
 
 #include "../../include/skis.h"
 #include "skis_internal.cuh"
@@ -1420,22 +1422,25 @@ int sketch_inverted(skis_sketch* s, cudaStream_t st, std::string* err) {
     s->inv = nullptr;
     s->inv_T = 0;
     if (!s->inv_off) CV_CUDA(dev_alloc_t(&s->inv_off, (size_t)n + 1, st));
-    uint32_t* cnt = nullptr;
     uint64_t E = 0;
     const int cblocks = coverage_blocks(T);
-    CV_CUDA(dev_alloc_t(&cnt, (size_t)n, st));
     if (s->vcount && s->vcount_ok && s->vcount_T == T) {  // counted while sampling
-        CV_CUDA(cudaMemcpyAsync(cnt, s->vcount, (size_t)n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, st));
+        CV_CUDA(scan_u32_to_u64(s->vcount, s->inv_off, n, st));
     } else {
-        CV_CUDA(cudaMemsetAsync(cnt, 0, (size_t)n * sizeof(uint32_t), st));
-        k_count_members<<<cblocks, kCovThreads, 0, st>>>(s->h_off, s->h_len, T, s->arena, cnt); note_launch();
-        CV_CUDA(cudaGetLastError());
+        uint32_t* cnt = nullptr;
+        CV_CUDA(dev_alloc_t(&cnt, (size_t)n, st));
+        cudaError_t e = cudaMemsetAsync(cnt, 0, (size_t)n * sizeof(uint32_t), st);
+        if (e == cudaSuccess) {
+            k_count_members<<<cblocks, kCovThreads, 0, st>>>(s->h_off, s->h_len, T, s->arena, cnt); note_launch();
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = scan_u32_to_u64(cnt, s->inv_off, n, st);
+        dev_free(cnt, st);
+        CV_CUDA(e);
     }
-    CV_CUDA(scan_u32_to_u64(cnt, s->inv_off, n, st));
     CV_CUDA(cudaMemcpyAsync(&E, s->inv_off + n, sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
     CV_CUDA(cudaStreamSynchronize(st));
     CV_CUDA(dev_alloc_t(&s->inv, (size_t)std::max<uint64_t>(E, 1), st));
-    dev_free(cnt, st);
     unsigned long long* cursor = nullptr;
     CV_CUDA(dev_alloc_t(&cursor, (size_t)n, st));
     CV_CUDA(cudaMemcpyAsync(cursor, s->inv_off, (size_t)n * sizeof(uint64_t), cudaMemcpyDeviceToDevice, st));
@@ -1463,14 +1468,7 @@ int sketch_greedy(skis_sketch* s, int32_t k, int32_t* h_seeds, int64_t* h_cov, d
     if (k == 0) return SKIS_OK;
     int rc = sketch_inverted(s, st, err);
     if (rc != SKIS_OK) return rc;
-    uint32_t *delta = nullptr, *covered = nullptr;
-    uint8_t* inS = nullptr;
-    Cand *partial = nullptr, *seg_best = nullptr;
-    uint32_t *pool = nullptr, *hist = nullptr;
-    GreedyCtl *ctl = nullptr, h_ctl{};
-    int32_t* d_seeds = nullptr;
-    int64_t* d_cov = nullptr;
-    double* d_est = nullptr;
+    char* buf = nullptr;
     auto body = [&]() -> int {
         int per_sm = 0;
         CV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_greedy_rounds, kGreedyThreads, 0));
@@ -1479,27 +1477,30 @@ int sketch_greedy(skis_sketch* s, int32_t k, int32_t* h_seeds, int64_t* h_cov, d
             return SKIS_ERR_CUDA;
         }
         const int gblocks = sm_count();  // one block per SM
-        CV_CUDA(dev_alloc_t(&delta, (size_t)n, st));
-        CV_CUDA(dev_alloc_t(&inS, (size_t)n, st));
-        CV_CUDA(dev_alloc_t(&covered, (size_t)((T + 31) / 32), st));
-        CV_CUDA(dev_alloc_t(&partial, (size_t)gblocks, st));
         const int64_t nseg = (n + kGreedySeg - 1) / kGreedySeg;
-        CV_CUDA(dev_alloc_t(&seg_best, (size_t)nseg, st));
-        CV_CUDA(dev_alloc_t(&pool, (size_t)kGreedyThreads, st));
-        // one allocation zeroed at once: the histogram and the control words
-        const size_t words = kBuckets + sizeof(GreedyCtl) / sizeof(uint32_t);
-        CV_CUDA(dev_alloc_t(&hist, words, st));
-        CV_CUDA(cudaMemsetAsync(hist, 0, words * sizeof(uint32_t), st));
-        ctl = reinterpret_cast<GreedyCtl*>(hist + kBuckets);
-        CV_CUDA(dev_alloc_t(&d_seeds, (size_t)k, st));
-        CV_CUDA(dev_alloc_t(&d_cov, (size_t)k, st));
-        CV_CUDA(dev_alloc_t(&d_est, (size_t)k, st));
-        CV_CUDA(cudaMemsetAsync(inS, 0, (size_t)n, st));
-        CV_CUDA(cudaMemsetAsync(covered, 0, (size_t)((T + 31) / 32) * sizeof(uint32_t), st));
+        // one allocation, its first part zeroed at once, the control words and
+        // the results next to one another for one copy back (each allocation or
+        // copy more is some microseconds of a call that takes 150 on a small sketch)
+        size_t bytes = 0;
+        auto take = [&](size_t b) {
+            const size_t at = bytes;
+            bytes += (b + 127) & ~(size_t)127;
+            return at;
+        };
+        const size_t at_hist = take(kBuckets * sizeof(uint32_t)), at_inS = take((size_t)n);
+        const size_t at_covered = take((size_t)((T + 31) / 32) * sizeof(uint32_t));
+        const size_t at_ctl = take(sizeof(GreedyCtl)), zeroed = bytes;
+        const size_t at_est = take((size_t)k * sizeof(double)), at_cov = take((size_t)k * sizeof(int64_t));
+        const size_t at_seeds = take((size_t)k * sizeof(int32_t)), copied = bytes - at_ctl;
+        const size_t at_partial = take((size_t)gblocks * sizeof(Cand)), at_seg = take((size_t)nseg * sizeof(Cand));
+        const size_t at_pool = take(kGreedyThreads * sizeof(uint32_t)), at_delta = take((size_t)n * sizeof(uint32_t));
+        std::vector<char> h_out(copied);
+        CV_CUDA(dev_alloc_t(&buf, bytes, st));
+        CV_CUDA(cudaMemsetAsync(buf, 0, zeroed, st));
         GreedyArgs ga;
         ga.w = g->w;
-        ga.inS = inS;
-        ga.delta = delta;
+        ga.inS = reinterpret_cast<uint8_t*>(buf + at_inS);
+        ga.delta = reinterpret_cast<uint32_t*>(buf + at_delta);
         ga.n = n;
         ga.W = g->W;
         ga.T = T;
@@ -1511,16 +1512,16 @@ int sketch_greedy(skis_sketch* s, int32_t k, int32_t* h_seeds, int64_t* h_cov, d
         ga.h_off = s->h_off;
         ga.h_len = s->h_len;
         ga.arena = s->arena;
-        ga.covered = covered;
-        ga.partial = partial;
-        ga.seg_best = seg_best;
+        ga.covered = reinterpret_cast<uint32_t*>(buf + at_covered);
+        ga.partial = reinterpret_cast<Cand*>(buf + at_partial);
+        ga.seg_best = reinterpret_cast<Cand*>(buf + at_seg);
         ga.nseg = nseg;
-        ga.pool = pool;
-        ga.hist = hist;
-        ga.ctl = ctl;
-        ga.seeds = d_seeds;
-        ga.cov_out = d_cov;
-        ga.est_out = d_est;
+        ga.pool = reinterpret_cast<uint32_t*>(buf + at_pool);
+        ga.hist = reinterpret_cast<uint32_t*>(buf + at_hist);
+        ga.ctl = reinterpret_cast<GreedyCtl*>(buf + at_ctl);
+        ga.seeds = reinterpret_cast<int32_t*>(buf + at_seeds);
+        ga.cov_out = reinterpret_cast<int64_t*>(buf + at_cov);
+        ga.est_out = reinterpret_cast<double*>(buf + at_est);
         ga.ris = s->ris;
         const int b1 = (int)std::max<int64_t>(1, std::min<int64_t>((n + kGreedyThreads - 1) / kGreedyThreads,
                                                                    (int64_t)sm_count() * 2));
@@ -1529,28 +1530,19 @@ int sketch_greedy(skis_sketch* s, int32_t k, int32_t* h_seeds, int64_t* h_cov, d
         void* kargs[] = {&ga};
         CV_CUDA(cudaLaunchCooperativeKernel((const void*)k_greedy_rounds, gblocks, kGreedyThreads, kargs, 0, st));
         note_launch();
-        CV_CUDA(cudaMemcpyAsync(h_seeds, d_seeds, (size_t)k * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-        if (h_cov) CV_CUDA(cudaMemcpyAsync(h_cov, d_cov, (size_t)k * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-        if (h_est) CV_CUDA(cudaMemcpyAsync(h_est, d_est, (size_t)k * sizeof(double), cudaMemcpyDeviceToHost, st));
-        CV_CUDA(cudaMemcpyAsync(&h_ctl, ctl, sizeof(GreedyCtl), cudaMemcpyDeviceToHost, st));
+        CV_CUDA(cudaMemcpyAsync(h_out.data(), buf + at_ctl, copied, cudaMemcpyDeviceToHost, st));
         CV_CUDA(cudaStreamSynchronize(st));
-        if (h_ctl.gave_up) {
+        if (reinterpret_cast<const GreedyCtl*>(h_out.data())->gave_up) {
             *err = "skis_greedy_maxcover: internal error: a grid barrier ran out";
             return SKIS_ERR_INTERNAL;
         }
+        std::memcpy(h_seeds, h_out.data() + (at_seeds - at_ctl), (size_t)k * sizeof(int32_t));
+        if (h_cov) std::memcpy(h_cov, h_out.data() + (at_cov - at_ctl), (size_t)k * sizeof(int64_t));
+        if (h_est) std::memcpy(h_est, h_out.data() + (at_est - at_ctl), (size_t)k * sizeof(double));
         return SKIS_OK;
     };
     rc = body();
-    dev_free(delta, st);
-    dev_free(covered, st);
-    dev_free(inS, st);
-    dev_free(partial, st);
-    dev_free(seg_best, st);
-    dev_free(pool, st);
-    dev_free(hist, st);
-    dev_free(d_seeds, st);
-    dev_free(d_cov, st);
-    dev_free(d_est, st);
+    dev_free(buf, st);
     return rc;
 }
 

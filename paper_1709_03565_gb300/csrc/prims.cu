@@ -248,16 +248,26 @@ __global__ void __launch_bounds__(256) k_os_hist(const int32_t* __restrict__ src
 }
 
 // Exclusive prefix of each pass's digit counts, in place: base[p * kOsMaxDigits + d].
-__global__ void __launch_bounds__(kOsMaxDigits) k_os_bases(unsigned long long* __restrict__ hist, int passes) {
-    __shared__ unsigned long long s_c[kOsMaxDigits];
-    for (int p = 0; p < passes; ++p) {
-        s_c[threadIdx.x] = hist[p * kOsMaxDigits + threadIdx.x];
-        __syncthreads();
-        unsigned long long b = 0;
-        for (int d = 0; d < (int)threadIdx.x; ++d) b += s_c[d];
-        hist[p * kOsMaxDigits + threadIdx.x] = b;
-        __syncthreads();
+// A block a pass, by warp scans (a thread summing its predecessors one by one,
+// pass after pass, took 12-16 us of a small load).
+__global__ void __launch_bounds__(kOsMaxDigits) k_os_bases(unsigned long long* __restrict__ hist) {
+    __shared__ unsigned long long s_w[kOsMaxDigits / 32];
+    unsigned long long* const h = hist + blockIdx.x * kOsMaxDigits;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned long long c = h[threadIdx.x];
+    unsigned long long x = c;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned long long y = __shfl_up_sync(kFull, x, d);
+        if (lane >= d) x += y;
     }
+    if (lane == 31) s_w[wid] = x;
+    __syncthreads();
+    unsigned long long before = lane < wid ? s_w[lane] : 0;  // lane < wid < kOsMaxDigits / 32 <= 32
+    static_assert(kOsMaxDigits / 32 <= 32, "a lane a warp");
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) before += __shfl_xor_sync(kFull, before, d);
+    h[threadIdx.x] = before + x - c;
 }
 
 // One pass on the kBits-bit digit at `shift`. kFirst: the items are the
@@ -506,18 +516,18 @@ cudaError_t sort_edges(const int32_t* src, const int32_t* dst, int64_t m, int sr
     if (attr_err != cudaSuccess) return attr_err;
     unsigned long long *hist = nullptr, *status = nullptr;
     unsigned int* tickets = nullptr;
-    cudaError_t e = dev_alloc_t(&hist, (size_t)passes * kOsMaxDigits, st);
-    if (e == cudaSuccess) e = dev_alloc_t(&status, (size_t)ntiles * kOsMaxDigits, st);
-    if (e == cudaSuccess) e = dev_alloc_t(&tickets, (size_t)passes, st);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(hist, 0, (size_t)passes * kOsMaxDigits * sizeof(unsigned long long), st);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(status, 0, (size_t)ntiles * kOsMaxDigits * sizeof(unsigned long long), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(tickets, 0, (size_t)passes * sizeof(unsigned int), st);
+    // one allocation, zeroed at once: the digit counts, the status words, the tickets
+    const size_t words = (size_t)(passes + ntiles) * kOsMaxDigits + (size_t)passes;
+    cudaError_t e = dev_alloc_t(&hist, words, st);
+    if (e == cudaSuccess) {
+        status = hist + (size_t)passes * kOsMaxDigits;
+        tickets = reinterpret_cast<unsigned int*>(status + (size_t)ntiles * kOsMaxDigits);
+        e = cudaMemsetAsync(hist, 0, words * sizeof(unsigned long long), st);
+    }
     if (e == cudaSuccess) {
         const int grid = (int)std::min<int64_t>((int64_t)sm_count() * 8, std::max<int64_t>(1, (m + 255) / 256));
         k_os_hist<<<grid, 256, 0, st>>>(src, dst, m, src_bits, ps, hist); note_launch();
-        k_os_bases<<<1, kOsMaxDigits, 0, st>>>(hist, passes); note_launch();
+        k_os_bases<<<passes, kOsMaxDigits, 0, st>>>(hist); note_launch();
         e = cudaGetLastError();
     }
     const uint64_t* ksrc = nullptr;
@@ -549,8 +559,6 @@ cudaError_t sort_edges(const int32_t* src, const int32_t* dst, int64_t m, int sr
         vsrc = out.vals;
     }
     dev_free(hist, st);
-    dev_free(status, st);
-    dev_free(tickets, st);
     return e;
 }
 
