@@ -970,12 +970,28 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_iis_warp(SampleArgs a) {
 // and take 4.4 ms. Where hubs hold the coins it is bound by the coin
 // generator: R-MAT 2^22 / 2^27 WC 372G blocks/s, 2^25 / 2^30 431G (the hub
 // loop alone, with no other work in the kernel, 455G).
-constexpr int kCtaBlock = 128;  // threads of the default blocks
+// Where a good part of a pass comes here, hubs hold the coins; then few
+// samples are bound by the longest of them, which a larger block shortens. Tier
+// alone, ms, blocks of 512 / 256 / 128: R-MAT 2^22 / 2^27, every sample here,
+// 1,200 samples 1.90 / 1.89 / 2.78, 5K 2.7 / 2.8 / 3.8, 10K 4.3 / 4.2 / 5.1,
+// 20K 7.3 / 6.8 / 6.9; 2^20 / 2^25 .98 / .99 / 1.30, 1.62 / 1.69 / 1.99, 2.46 /
+// 2.12 / 2.41, 4.2 / 3.5 / 3.4; 2^18 / 2^23 at 5K .91 / .77 / .97; the default
+// split of 10K samples of 2^20 / 2^25 (26 % here) 2.33 / 2.13 / 2.50. Where
+// only the largest come here (Chung-Lu 4M / 140M WC, 1.7 % of 65K: 2.5 / 1.56 /
+// 1.24, of 1M: 30 / 15.3 / 10.1) their levels are narrow and more of them at a
+// time count. So blocks of 128, but for passes of which more than 1 /
+// kCtaHubShare comes here: 512 up to kCtaFew samples an SM in the pass, 256 up
+// to kCtaMany of them here.
+constexpr int kCtaBlock = 128;
+constexpr uint64_t kCtaHubShare = 8, kCtaFew = 24, kCtaMany = 96;
 constexpr int kCtaWin = 512;  // rows of a level in shared memory at a time
 
 template <int kCtaThreads>
-__global__ void __launch_bounds__(kCtaThreads, 1024 / kCtaThreads) k_iis_cta(SampleArgs a) {
+__global__ void __launch_bounds__(kCtaThreads, 1024 / kCtaThreads) k_iis_cta(SampleArgs a, uint64_t above,
+                                                                            uint64_t upto, bool within) {
     constexpr int kWarps = kCtaThreads / 32;
+    const uint64_t count = input_count(a);
+    if ((count > above && count <= upto) != within) return;  // the other launch's
     __shared__ unsigned long long s_j;
     __shared__ unsigned long long s_coins;
     __shared__ unsigned long long s_base;
@@ -995,7 +1011,6 @@ __global__ void __launch_bounds__(kCtaThreads, 1024 / kCtaThreads) k_iis_cta(Sam
     int32_t* queue = a.queues + (uint64_t)blockIdx.x * a.queue_cap;
     const uint4* __restrict__ tau4 = reinterpret_cast<const uint4*>(a.tau);
     const uint4* __restrict__ rows4 = reinterpret_cast<const uint4*>(a.rows);  // offset (low, high), degree, threshold
-    const uint64_t count = input_count(a);
     auto is_hub = [&](uint32_t nq) { return a.cta_hub_quads && nq >= a.cta_hub_quads; };
     bool clean = a.slot_clean[blockIdx.x] != 0;
     unsigned long long claim = 0;  // thread 0: the block's next input
@@ -1741,7 +1756,7 @@ static cudaError_t grow_copy(T** p, uint64_t old_n, uint64_t new_n, cudaStream_t
     return cudaSuccess;
 }
 
-// threads of a CTA-tier block
+// threads of the CTA-tier blocks that the slots are counted for (launch_cta)
 static int cta_block(const skis_sketch* s) { return s->cta_threads == 512 ? 512 : kCtaBlock; }
 
 // slack: arena entries that the tiers' warps may leave unused at the ends of their chunks;
@@ -1866,10 +1881,31 @@ static int ensure_big_slots(skis_sketch* s, cudaStream_t st, std::string* err) {
     return SKIS_OK;
 }
 
-static void launch_cta(const skis_sketch* s, const SampleArgs& a, int slots, cudaStream_t st) {
-    if (cta_block(s) == 512) k_iis_cta<512><<<slots, 512, 0, st>>>(a);
-    else k_iis_cta<kCtaBlock><<<slots, kCtaBlock, 0, st>>>(a);
+// At most `slots` blocks of kCtaThreads, for a count in (above, upto] or for any other.
+template <int kCtaThreads>
+static void launch_cta_blocks(const SampleArgs& a, int slots, uint64_t above, uint64_t upto, bool within,
+                              cudaStream_t st) {
+    k_iis_cta<kCtaThreads><<<std::min(slots, sm_count() * (1024 / kCtaThreads)), kCtaThreads, 0, st>>>(a, above, upto,
+                                                                                                      within);
     note_launch();
+}
+
+// The CTA tier for a pass of `pass` samples; how many of them come here is on
+// the device, so a pass that two block sizes may take is launched with both,
+// one of which ends at once.
+static void launch_cta(const skis_sketch* s, const SampleArgs& a, int slots, uint64_t pass, cudaStream_t st) {
+    const uint64_t share = pass / kCtaHubShare;
+    const uint64_t few = kCtaFew * (uint64_t)sm_count(), many = kCtaMany * (uint64_t)sm_count();
+    if (cta_block(s) == 512) {
+        k_iis_cta<512><<<slots, 512, 0, st>>>(a, 0, ~0ull, true);
+        note_launch();
+    } else if (share >= many) {
+        launch_cta_blocks<kCtaBlock>(a, slots, 0, ~0ull, true, st);
+    } else {
+        if (pass <= few) launch_cta_blocks<512>(a, slots, share, many, true, st);
+        else launch_cta_blocks<256>(a, slots, share, many, true, st);
+        launch_cta_blocks<kCtaBlock>(a, slots, share, many, false, st);
+    }
 }
 
 static int occupancy_grid(const void* kernel, int threads, int override_blocks, uint64_t max_useful,
@@ -2045,7 +2081,7 @@ int sketch_sample(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* 
             k_iis_warp<<<warp_blocks, kWarpThreads, 0, st>>>(aw); note_launch();
             SK_CUDA(cudaGetLastError());
             SK_CUDA(cudaEventRecord(s->ev[2], st));
-            launch_cta(s, ac, s->cta_slots_alloc, st);
+            launch_cta(s, ac, s->cta_slots_alloc, base.count, st);
             SK_CUDA(cudaGetLastError());
             SK_CUDA(cudaEventRecord(s->ev[3], st));
         }
@@ -2071,7 +2107,7 @@ int sketch_sample(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* 
             if (g->lt) {
                 k_lt_long<<<s->big_slots, 32, 0, st>>>(ab); note_launch();
             } else {
-                launch_cta(s, ab, s->big_slots, st);
+                launch_cta(s, ab, s->big_slots, hc.n_big, st);
             }
             SK_CUDA(cudaGetLastError());
             SK_CUDA(cudaEventRecord(s->ev[3], st));

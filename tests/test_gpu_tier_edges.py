@@ -65,3 +65,30 @@ def test_sizes_at_the_tiers_edges(shape, size, n, tier, bucket):
     assert_samples_equal(skis.skis_sketch_export(s, 0, T), ora)
     s.close()
     g.close()
+
+
+# the CTA tier's block size goes by the samples of the pass and of the tier: 24 and 96 an SM are the lines
+@pytest.mark.parametrize("per_sm,more", [(1, -1), (24, 0), (24, 1), (96, 0), (96, 1), (130, 0)])
+@pytest.mark.parametrize("hub_quads", [2, 0])
+def test_cta_block_sizes(per_sm, more, hub_quads):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    n = 700
+    rng = np.random.default_rng(5)
+    src = np.concatenate([rng.integers(1, n, 3000), np.arange(1, n)]).astype(np.int32)
+    dst = np.concatenate([rng.integers(1, n, 3000), np.zeros(n - 1)]).astype(np.int32)
+    keep = src != dst
+    src, dst = src[keep], dst[keep]
+    tau = rng.integers(1 << 28, 1 << 31, len(src)).astype(np.uint32)
+    g = skis.skis_load_graph(n, src, dst, tau, skis.SKIS_W_EXPLICIT_TAU)
+    o = oracle.OracleGraph(n, src, dst, weights=tau, model=oracle.W_TAU)
+    T, seed = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + more, 0xB10C
+    s = skis.skis_sketch_create(g, seed)
+    for k, v in ((skis.SKIS_OPT_THREAD_MAX_DEG, 0), (skis.SKIS_OPT_WARP_MAX_COINS, 1),
+                 (skis.SKIS_OPT_CTA_HUB_QUADS, hub_quads)):
+        skis.skis_sketch_set_option(s, k, v)
+    skis.skis_sample(s, T)
+    assert_samples_equal(skis.skis_sketch_export(s, 0, T), o.sample_ids(seed, np.arange(T, dtype=np.uint64)))
+    s.close()
+    g.close()
