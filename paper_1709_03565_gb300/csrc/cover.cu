@@ -208,14 +208,19 @@ __global__ void __launch_bounds__(kCovThreads) k_coverage(const uint64_t* __rest
 
 // The scan of a sketch whose members are in sample-id order (arena
 // positions [h_off[0], ...) contiguous): the seed filter sits in shared
-// memory; a warp takes 1024 consecutive samples at a time (from an atomic
-// cursor, so that warps meeting large samples or many seeds take fewer), whose
-// members are one run, and streams it as 16-byte vectors testing each member
-// against the filter. Only a member that is a seed (rare) looks up its
-// sample, by a binary search over the task's 1024 offsets, and ORs its query
-// mask into the sample's
-// word of smask; the first setter of a (sample, query) bit counts it, and the
-// first setter of a sample's word lists the sample for the reset.
+// memory; a warp takes a task of 2^tlog consecutive samples at a time (from an
+// atomic cursor, so that warps meeting many seeds take fewer), whose members
+// are one run, and streams it as 16-byte vectors testing each member against
+// the filter. Possible seeds (rare) are held back per warp and join the hit
+// list for k_scan_hits with one atomic for dozens; only when the list is full
+// is a hit resolved here. The first setter of a (sample, query) bit of smask
+// counts it, and the first setter of a sample's word lists the sample for the
+// reset. Bound by the returning list atomics when each hit took one on the same
+// counter, and by too few tasks where samples are large (1024 samples a task):
+// 10M samples of 4 members and 64 queries of 50 seeds 71 -> 53 us, the whole
+// call 177 -> 168; 1M of 70 members 309 -> 175; 6M of 4 members and 64 queries
+// of 250 seeds 778 -> 470. Now by the chain of load, filter read and branch at
+// one block an SM (the filter's 128 KiB); the members' bytes alone take 25 us.
 constexpr int kScanThreads = 1024;
 
 // Asynchronous bulk prefetch of [p, p + bytes) into L2 (p 16-byte aligned,
@@ -223,54 +228,79 @@ constexpr int kScanThreads = 1024;
 __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
-constexpr uint32_t kScanSamples = 1024;
 constexpr int kScanUnroll = 4;
-constexpr uint64_t kScanAhead = 4;  // warp steps prefetched ahead
+constexpr unsigned int kScanHits = 128;  // hits a warp holds back
+constexpr uint64_t kScanMembers = 2048;
+constexpr uint64_t kScanAhead = 8;  // warp steps prefetched ahead
 constexpr unsigned long long kHitCap = 1ull << 22;  // hits listed per query chunk (32 MiB); more are resolved in the scan
 
 __global__ void __launch_bounds__(kScanThreads, 1) k_scan_ordered(
-    const uint64_t* __restrict__ h_off, const uint32_t* __restrict__ h_len, uint64_t T,
+    const uint64_t* __restrict__ h_off, const uint32_t* __restrict__ h_len, uint64_t T, int tlog,
     const int32_t* __restrict__ arena, const uint32_t* __restrict__ qbits, uint32_t fwords, int hashed,
     const uint64_t* __restrict__ qmask, unsigned long long* __restrict__ smask, uint32_t* __restrict__ touched,
     unsigned long long* __restrict__ ntouched, unsigned long long* __restrict__ cursor,
     unsigned long long* __restrict__ hits, unsigned long long* __restrict__ nhits, unsigned long long hit_cap,
     unsigned long long* __restrict__ cov) {
-    extern __shared__ uint32_t s_f[];
+    extern __shared__ __align__(16) uint32_t s_f[];
     __shared__ unsigned int s_cnt[64];
-    for (uint32_t i = threadIdx.x; i < fwords; i += blockDim.x) s_f[i] = qbits[i];
+    __shared__ unsigned long long s_hit[kScanThreads / 32][kScanHits];
+    __shared__ unsigned int s_nhit[kScanThreads / 32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint4* q4 = reinterpret_cast<const uint4*>(qbits);
+#pragma unroll 8
+    for (uint32_t i = threadIdx.x; i < fwords / 4; i += kScanThreads) reinterpret_cast<uint4*>(s_f)[i] = q4[i];
+    if (threadIdx.x < fwords % 4) s_f[(fwords & ~3u) + threadIdx.x] = qbits[(fwords & ~3u) + threadIdx.x];
     if (threadIdx.x < 64) s_cnt[threadIdx.x] = 0;
+    if (lane == 0) s_nhit[wid] = 0;
     __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const uint64_t ntask = (T + kScanSamples - 1) / kScanSamples;
+    unsigned long long* const my_hit = s_hit[wid];
+    // hit h = (task << 40) | position takes place `slot` of the list; where that
+    // is full, it is resolved here: the member's query mask, its sample (the
+    // last whose run starts at or before it) and the counts
+    auto list = [&](unsigned long long h, unsigned long long slot) {
+        if (slot < hit_cap) {
+            hits[slot] = h;
+            return;
+        }
+        const uint64_t pos = h & ((1ull << 40) - 1);
+        const uint64_t msk = qmask[arena[pos]];
+        if (!msk) return;  // a filter collision
+        uint64_t lo = (h >> 40) << tlog, hi = min(T, lo + (1u << tlog)) - 1;
+        while (lo < hi) {
+            const uint64_t mid = (lo + hi + 1) >> 1;
+            if (h_off[mid] <= pos) lo = mid;
+            else hi = mid - 1;
+        }
+        const unsigned long long old = atomicOr(smask + lo, (unsigned long long)msk);
+        if (old == 0) touched[atomicAdd(ntouched, 1ull)] = (uint32_t)lo;
+        for (uint64_t nb = msk & ~old; nb; nb &= nb - 1) atomicAdd(&s_cnt[__ffsll((long long)nb) - 1], 1u);
+    };
+    // the warp's hits join the list, one atomic for all
+    auto flush = [&](unsigned int cnt) {
+        unsigned long long base = 0;
+        if (lane == 0) base = atomicAdd(nhits, (unsigned long long)cnt);
+        base = __shfl_sync(kFull, base, 0);
+        for (unsigned int i = lane; i < cnt; i += 32) list(my_hit[i], base + i);
+        __syncwarp();
+        if (lane == 0) s_nhit[wid] = 0;
+        __syncwarp();
+    };
+    const uint64_t ntask = (T + (1u << tlog) - 1) >> tlog;
     unsigned long long claim = 0;
     if (lane == 0) claim = atomicAdd(cursor, 1ull);
     for (;;) {
         const unsigned long long task = __shfl_sync(kFull, claim, 0);
         if (task >= ntask) break;
         if (lane == 0) claim = atomicAdd(cursor, 1ull);  // the next task, claimed while this one streams
-        const uint64_t j0 = task * kScanSamples, j1 = min(T, j0 + kScanSamples);
+        const uint64_t j0 = task << tlog, j1 = min(T, j0 + (1u << tlog));
         const uint64_t p0 = h_off[j0], p1 = h_off[j1 - 1] + h_len[j1 - 1];
         auto member = [&](uint64_t pos, int32_t u) {
             const uint32_t f = filter_index((uint32_t)u, hashed);
             if (!((s_f[f >> 5] >> (f & 31)) & 1u)) return;
-            // a possible seed: its (task, position) goes to the hit list for
-            // k_scan_hits; only when the list is full is it resolved here
-            const unsigned long long slot = atomicAdd(nhits, 1ull);
-            if (slot < hit_cap) {
-                hits[slot] = ((unsigned long long)task << 40) | pos;
-                return;
-            }
-            const uint64_t msk = qmask[u];
-            if (!msk) return;  // a filter collision
-            uint64_t lo = j0, hi = j1 - 1;  // the last sample whose run starts at or before pos
-            while (lo < hi) {
-                const uint64_t mid = (lo + hi + 1) >> 1;
-                if (h_off[mid] <= pos) lo = mid;
-                else hi = mid - 1;
-            }
-            const unsigned long long old = atomicOr(smask + lo, (unsigned long long)msk);
-            if (old == 0) touched[atomicAdd(ntouched, 1ull)] = (uint32_t)lo;
-            for (uint64_t nb = msk & ~old; nb; nb &= nb - 1) atomicAdd(&s_cnt[__ffsll((long long)nb) - 1], 1u);
+            // a possible seed: its (task, position) goes to the hit list for k_scan_hits
+            const unsigned int slot = atomicAdd(&s_nhit[wid], 1u);
+            if (slot < kScanHits) my_hit[slot] = ((unsigned long long)task << 40) | pos;
+            else list(((unsigned long long)task << 40) | pos, atomicAdd(nhits, 1ull));
         };
         const uint64_t up = (p0 + 3) & ~(uint64_t)3, down = p1 & ~(uint64_t)3;
         const uint64_t ph = p1 < up ? p1 : up, pt = down > ph ? down : ph;
@@ -282,11 +312,10 @@ __global__ void __launch_bounds__(kScanThreads, 1) k_scan_ordered(
         constexpr uint64_t kStep = 32 * kScanUnroll;  // 16-byte vectors a warp step loads
         if (lane == 0 && v0 < v_end)
             prefetch_l2(a4 + v0, (uint32_t)(min(v_end - v0, kStep * kScanAhead) * 16));
-        uint64_t v = v0 + lane;
         // kScanUnroll 16-byte loads in flight a lane before any member is tested
         // (the last step of a task predicated, not a step per load)
-        for (; v < v_end; v += 32 * kScanUnroll) {
-            const uint64_t ahead = (v - lane) + kStep * kScanAhead;
+        for (uint64_t vb = v0; vb < v_end; vb += kStep) {
+            const uint64_t ahead = vb + kStep * kScanAhead, v = vb + lane;
             if (lane == 0 && ahead < v_end) prefetch_l2(a4 + ahead, (uint32_t)(min(v_end - ahead, kStep) * 16));
             int4 m[kScanUnroll];
 #pragma unroll
@@ -301,11 +330,26 @@ __global__ void __launch_bounds__(kScanThreads, 1) k_scan_ordered(
                 member(pos + 2, m[k].z);
                 member(pos + 3, m[k].w);
             }
+            __syncwarp();
+            const unsigned int cnt = s_nhit[wid];
+            if (cnt >= kScanHits / 2) flush(min(cnt, kScanHits));
         }
         if (pt + lane < p1) member(pt + lane, arena[pt + lane]);
     }
+    __syncwarp();
+    if (s_nhit[wid]) flush(min(s_nhit[wid], kScanHits));
     __syncthreads();
     if (threadIdx.x < 64 && s_cnt[threadIdx.x]) atomicAdd(&cov[threadIdx.x], (unsigned long long)s_cnt[threadIdx.x]);
+}
+
+// Samples of a scan task, as a power of two: about kScanMembers members (of
+// 1024, 2048, 4096 members a task the calls above took 183, 168, 178 us, 185,
+// 179, 190 and 470, 469, 520), and the tasks' numbers fit the 24 bits of a hit.
+static int scan_task_log(uint64_t T, uint64_t members) {
+    int tlog = 5;
+    while (tlog < 10 && (members << tlog) < kScanMembers * T) ++tlog;
+    while ((T >> tlog) >= (1ull << 24) - 1) ++tlog;
+    return tlog;
 }
 
 // The hits the scan listed: each (task, position) resolves to its member,
@@ -314,7 +358,7 @@ __global__ void __launch_bounds__(kScanThreads, 1) k_scan_ordered(
 __global__ void __launch_bounds__(256) k_scan_hits(const unsigned long long* __restrict__ hits,
                                                    const unsigned long long* __restrict__ nhits,
                                                    unsigned long long hit_cap, const uint64_t* __restrict__ h_off,
-                                                   uint64_t T, const int32_t* __restrict__ arena,
+                                                   uint64_t T, int tlog, const int32_t* __restrict__ arena,
                                                    const uint64_t* __restrict__ qmask,
                                                    unsigned long long* __restrict__ smask,
                                                    uint32_t* __restrict__ touched,
@@ -329,7 +373,7 @@ __global__ void __launch_bounds__(256) k_scan_hits(const unsigned long long* __r
         const uint64_t pos = h & ((1ull << 40) - 1), task = h >> 40;
         const uint64_t msk = qmask[arena[pos]];
         if (!msk) continue;  // a filter collision
-        uint64_t lo = task * kScanSamples, hi = min(T, lo + kScanSamples) - 1;
+        uint64_t lo = task << tlog, hi = min(T, lo + (1u << tlog)) - 1;
         while (lo < hi) {
             const uint64_t mid = (lo + hi + 1) >> 1;
             if (h_off[mid] <= pos) lo = mid;
@@ -740,6 +784,7 @@ int sketch_estimate(skis_sketch* s, int32_t q, const int64_t* d_off, const int32
                                      (int)(kFilterMaxWords * sizeof(uint32_t))));
     int cblocks = 0, glog = 0;
     coverage_shape(s->T, &cblocks, &glog);
+    const int tlog = scan_task_log(s->T, s->arena_used);
     float query_ms = 0;
     for (int32_t q0 = 0; q0 < q; q0 += 64) {
         const int32_t qn = std::min<int32_t>(64, q - q0);
@@ -753,12 +798,12 @@ int sketch_estimate(skis_sketch* s, int32_t q, const int64_t* d_off, const int32
                                       queue_cap, s->smask, s->qcov, st));
         } else if (ordered_scan) {
             k_scan_ordered<<<sm_count(), kScanThreads, fwords * sizeof(uint32_t), st>>>(
-                s->h_off, s->h_len, s->T, s->arena, s->qbits, fwords, hashed, s->qmask,
+                s->h_off, s->h_len, s->T, tlog, s->arena, s->qbits, fwords, hashed, s->qmask,
                 reinterpret_cast<unsigned long long*>(s->smask), s->touched, s->ntouched, s->ntouched + 1, s->hits,
                 s->ntouched + 2, kHitCap, s->qcov);
             note_launch();
             CV_CUDA(cudaGetLastError());
-            k_scan_hits<<<sm_count() * 8, 256, 0, st>>>(s->hits, s->ntouched + 2, kHitCap, s->h_off, s->T, s->arena,
+            k_scan_hits<<<sm_count() * 8, 256, 0, st>>>(s->hits, s->ntouched + 2, kHitCap, s->h_off, s->T, tlog, s->arena,
                                                         s->qmask, reinterpret_cast<unsigned long long*>(s->smask),
                                                         s->touched, s->ntouched, s->qcov);
             note_launch();
