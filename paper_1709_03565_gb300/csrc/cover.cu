@@ -14,7 +14,6 @@
 #include <algorithm>
 #include <cstring>
 #include <string>
-#include <vector>
 
 #include "../../include/skis.h"
 #include "skis_internal.cuh"
@@ -1496,6 +1495,8 @@ int sketch_inverted(skis_sketch* s, cudaStream_t st, std::string* err) {
     return SKIS_OK;
 }
 
+constexpr int32_t kGreedyPacked = 4096;  // largest k whose results come back in one copy through the stack
+
 int sketch_greedy(skis_sketch* s, int32_t k, int32_t* h_seeds, int64_t* h_cov, double* h_est, cudaStream_t st,
                   std::string* err) {
     const char* where = "skis_greedy_maxcover";
@@ -1539,7 +1540,8 @@ int sketch_greedy(skis_sketch* s, int32_t k, int32_t* h_seeds, int64_t* h_cov, d
         const size_t at_seeds = take((size_t)k * sizeof(int32_t)), copied = bytes - at_ctl;
         const size_t at_partial = take((size_t)gblocks * sizeof(Cand)), at_seg = take((size_t)nseg * sizeof(Cand));
         const size_t at_pool = take(kGreedyThreads * sizeof(uint32_t)), at_delta = take((size_t)n * sizeof(uint32_t));
-        std::vector<char> h_out(copied);
+        const bool packed = k <= kGreedyPacked;  // else straight to the caller's arrays
+        alignas(128) char h_out[sizeof(GreedyCtl) + kGreedyPacked * 20 + 3 * 128];
         CV_CUDA(dev_alloc_t(&buf, bytes, st));
         CV_CUDA(cudaMemsetAsync(buf, 0, zeroed, st));
         GreedyArgs ga;
@@ -1575,15 +1577,22 @@ int sketch_greedy(skis_sketch* s, int32_t k, int32_t* h_seeds, int64_t* h_cov, d
         void* kargs[] = {&ga};
         CV_CUDA(cudaLaunchCooperativeKernel((const void*)k_greedy_rounds, gblocks, kGreedyThreads, kargs, 0, st));
         note_launch();
-        CV_CUDA(cudaMemcpyAsync(h_out.data(), buf + at_ctl, copied, cudaMemcpyDeviceToHost, st));
+        CV_CUDA(cudaMemcpyAsync(h_out, buf + at_ctl, packed ? copied : sizeof(GreedyCtl), cudaMemcpyDeviceToHost, st));
+        if (!packed) {
+            CV_CUDA(cudaMemcpyAsync(h_seeds, ga.seeds, (size_t)k * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+            if (h_cov) CV_CUDA(cudaMemcpyAsync(h_cov, ga.cov_out, (size_t)k * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+            if (h_est) CV_CUDA(cudaMemcpyAsync(h_est, ga.est_out, (size_t)k * sizeof(double), cudaMemcpyDeviceToHost, st));
+        }
         CV_CUDA(cudaStreamSynchronize(st));
-        if (reinterpret_cast<const GreedyCtl*>(h_out.data())->gave_up) {
+        if (reinterpret_cast<const GreedyCtl*>(h_out)->gave_up) {
             *err = "skis_greedy_maxcover: internal error: a grid barrier ran out";
             return SKIS_ERR_INTERNAL;
         }
-        std::memcpy(h_seeds, h_out.data() + (at_seeds - at_ctl), (size_t)k * sizeof(int32_t));
-        if (h_cov) std::memcpy(h_cov, h_out.data() + (at_cov - at_ctl), (size_t)k * sizeof(int64_t));
-        if (h_est) std::memcpy(h_est, h_out.data() + (at_est - at_ctl), (size_t)k * sizeof(double));
+        if (packed) {
+            std::memcpy(h_seeds, h_out + (at_seeds - at_ctl), (size_t)k * sizeof(int32_t));
+            if (h_cov) std::memcpy(h_cov, h_out + (at_cov - at_ctl), (size_t)k * sizeof(int64_t));
+            if (h_est) std::memcpy(h_est, h_out + (at_est - at_ctl), (size_t)k * sizeof(double));
+        }
         return SKIS_OK;
     };
     rc = body();

@@ -19,7 +19,8 @@ REL = 1e-12  # FP64 estimates of exact integers
     (1000, 8000, 500, 1000),    # every vertex fits the pool; Delta runs out long before k
     (1025, 8000, 5000, 1025),   # one vertex outside the pool
     (5000, 40000, 200, 1500),   # few samples: thousands of ties at Delta 0 and 1
-    (6000, 60000, 60000, 2500)  # refills
+    (6000, 60000, 60000, 2500),  # refills
+    (4200, 30000, 3000, 4096), (4200, 30000, 3000, 4097)  # results copied back together or one by one
 ])
 def test_greedy_seeds_over_pool_refills_and_ties(n, m, T, k, ris):
     torch = pytest.importorskip("torch")
