@@ -557,7 +557,7 @@ def chunglu_line(skis, torch, dev, stream, args, peak):
             cov[name].update({"algorithmic_bytes": nbytes, "gb_per_s": nbytes / (kms / 1e3) / 1e9,
                               "frac_of_hbm_peak": nbytes / (kms / 1e3) / 1e9 / peak,
                               "call_gb_per_s": nbytes / (cms / 1e3) / 1e9,
-                              "kernel": "k_scan_ordered + k_unmark (members in sample-id order)"})
+                              "kernel": "k_scan_ordered + k_scan_hits (members in sample-id order)"})
     s.close()
     out["coverage"] = cov
     if not args.no_variants:
