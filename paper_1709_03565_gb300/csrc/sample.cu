@@ -39,9 +39,9 @@ constexpr int kIdBatch = 16;       // most sample ids a warp takes per work-curs
 // Members a sample may have in the warp tier, past kQCap in the warp's global
 // spill slot, and the slot's hash bits (load at most 1/2). The longest samples
 // that are still narrow (a few rows a level) belong here, where 32 of them
-// share an SM, and not on the CTA tier, where four do: on Chung-Lu 1M / 17.5M
-// WC (levels of 13 rows) the two tiers take 10.6 ms with 1536 members and
-// 7.5 ms with 4096. A sample that holds a sixth of the graph has levels wide
+// share an SM, and not on the CTA tier, where at most eight do: on Chung-Lu 1M /
+// 17.5M WC (levels of 13 rows; four blocks an SM then) the two tiers take
+// 10.6 ms with 1536 members and 7.5 ms with 4096. A sample that holds a sixth of the graph has levels wide
 // enough for a block, so a small graph keeps the smaller slot.
 struct SpillSize {
     uint32_t cap, hash_bits;
