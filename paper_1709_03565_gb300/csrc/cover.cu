@@ -185,6 +185,7 @@ __global__ void __launch_bounds__(kCovThreads) k_coverage(const uint64_t* __rest
             }
         });
         if (!__any_sync(kFull, hit)) continue;
+        __syncwarp();  // every lane has the others' ORs (a vote orders no memory)
         const uint64_t acc = acc_row[lane];
         uint64_t present = acc;
 #pragma unroll
