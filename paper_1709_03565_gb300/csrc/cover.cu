@@ -331,13 +331,15 @@ __global__ void __launch_bounds__(kScanThreads, 1) k_scan_ordered(
                 member(pos + 3, m[k].w);
             }
             __syncwarp();
-            const unsigned int cnt = s_nhit[wid];
+            // one lane's read decides for the warp (a lane of its own might already see the next step's hits)
+            const unsigned int cnt = __shfl_sync(kFull, s_nhit[wid], 0);
             if (cnt >= kScanHits / 2) flush(min(cnt, kScanHits));
         }
         if (pt + lane < p1) member(pt + lane, arena[pt + lane]);
     }
     __syncwarp();
-    if (s_nhit[wid]) flush(min(s_nhit[wid], kScanHits));
+    const unsigned int rest = __shfl_sync(kFull, s_nhit[wid], 0);
+    if (rest) flush(min(rest, kScanHits));
     __syncthreads();
     if (threadIdx.x < 64 && s_cnt[threadIdx.x]) atomicAdd(&cov[threadIdx.x], (unsigned long long)s_cnt[threadIdx.x]);
 }
