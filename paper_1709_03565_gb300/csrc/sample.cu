@@ -1853,9 +1853,10 @@ static int ensure_sample_buffers(skis_sketch* s, uint64_t count, uint64_t slack,
         dev_free(s->bitmaps, st);
         dev_free(s->queues, st);
         dev_free(s->slot_clean, st);
+        dev_free(s->big_queues, st);  // the pass for outgrown samples uses the first slots' bitmaps: as many at most
         s->bitmaps = s->slot_clean = nullptr;
-        s->queues = nullptr;
-        s->cta_slots_alloc = 0;
+        s->queues = s->big_queues = nullptr;
+        s->cta_slots_alloc = s->big_slots = 0;
         s->bitmap_words = ((uint64_t)g->n + 31) / 32;
         SK_CUDA(dev_alloc_t(&s->bitmaps, (size_t)(s->bitmap_words * slots), st));
         SK_CUDA(dev_alloc_t(&s->slot_clean, (size_t)slots, st));
