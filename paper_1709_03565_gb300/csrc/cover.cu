@@ -738,35 +738,45 @@ int sketch_estimate(skis_sketch* s, int32_t q, const int64_t* d_off, const int32
     }
     const uint32_t fwords = filter_words(g->n);
     const int hashed = g->n > ((int64_t)1 << kFilterLog2);
+    // each buffer by its own pointer: a call that ran out of memory may have left any of them
     if (!s->qmask) {
         CV_CUDA(dev_alloc_t(&s->qmask, (size_t)g->n, st));
         CV_CUDA(cudaMemsetAsync(s->qmask, 0, (size_t)g->n * sizeof(uint64_t), st));
+    }
+    if (!s->qbits) {
         CV_CUDA(dev_alloc_t(&s->qbits, (size_t)fwords, st));
         CV_CUDA(cudaMemsetAsync(s->qbits, 0, (size_t)fwords * sizeof(uint32_t), st));
-        // coverage counts, the index walk's queue length and the status, zero
-        // (first_bad all ones) between calls
+    }
+    // coverage counts, the index walk's queue length and the status, zero
+    // (first_bad all ones) between calls
+    if (!s->qcov) {
         CV_CUDA(dev_alloc_t(&s->qcov, 65, st));
-        CV_CUDA(dev_alloc_t(&s->qstatus, 1, st));
         CV_CUDA(cudaMemsetAsync(s->qcov, 0, 65 * sizeof(unsigned long long), st));
+    }
+    if (!s->qstatus) {
+        CV_CUDA(dev_alloc_t(&s->qstatus, 1, st));
         CV_CUDA(cudaMemsetAsync(s->qstatus, 0, sizeof(DevStatus), st));
         CV_CUDA(cudaMemsetAsync(&s->qstatus->first_bad, 0xFF, sizeof(unsigned long long), st));
-        CV_CUDA(cudaEventCreate(&s->qev[0]));
-        CV_CUDA(cudaEventCreate(&s->qev[1]));
     }
+    for (int i = 0; i < 2; ++i)
+        if (!s->qev[i]) CV_CUDA(cudaEventCreate(&s->qev[i]));
     uint64_t* queue = nullptr;
     uint64_t queue_cap = 0;
-    if (ordered_scan && s->touched_cap < s->T) {
-        dev_free(s->touched, st);
-        s->touched = nullptr;
-        CV_CUDA(dev_alloc_t(&s->touched, (size_t)s->T, st));
-        if (!s->ntouched) {  // list count, task cursor and hit count (k_qmask_set resets them)
-            CV_CUDA(dev_alloc_t(&s->ntouched, 3, st));
-            CV_CUDA(dev_alloc_t(&s->hits, (size_t)kHitCap, st));
+    if (ordered_scan) {
+        if (s->touched_cap < s->T) {
+            s->touched_cap = 0;
+            dev_free(s->touched, st);
+            s->touched = nullptr;
+            CV_CUDA(dev_alloc_t(&s->touched, (size_t)s->T, st));
+            s->touched_cap = s->T;
         }
-        s->touched_cap = s->T;
+        // list count, task cursor and hit count (k_qmask_set resets them)
+        if (!s->ntouched) CV_CUDA(dev_alloc_t(&s->ntouched, 3, st));
+        if (!s->hits) CV_CUDA(dev_alloc_t(&s->hits, (size_t)kHitCap, st));
     }
     if (by_index || ordered_scan) {
         if (s->smask_cap < s->T) {
+            s->smask_cap = 0;
             dev_free(s->smask, st);
             s->smask = nullptr;
             CV_CUDA(dev_alloc_t(&s->smask, (size_t)s->T, st));

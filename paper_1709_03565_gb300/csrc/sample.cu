@@ -1764,12 +1764,16 @@ static int cta_block(const skis_sketch* s) { return s->cta_threads == 512 ? 512 
 static int ensure_sample_buffers(skis_sketch* s, uint64_t count, uint64_t slack, uint64_t warps, cudaStream_t st,
                                  std::string* err) {
     const skis_graph* g = s->g;
+    // each buffer is asked for by its own pointer (or a size that is reset before
+    // its group is freed), so that after an allocation failed the next call finds
+    // out which are missing
     if (!s->ctr) {
         SK_CUDA(dev_alloc_t(&s->ctr, 1, st));
         SK_CUDA(cudaMemsetAsync(s->ctr, 0, sizeof(SampleCounters), st));
-        SK_CUDA(dev_alloc_t(&s->status, 1, st));
-        for (int i = 0; i < 4; ++i) SK_CUDA(cudaEventCreate(&s->ev[i]));
     }
+    if (!s->status) SK_CUDA(dev_alloc_t(&s->status, 1, st));
+    for (int i = 0; i < 4; ++i)
+        if (!s->ev[i]) SK_CUDA(cudaEventCreate(&s->ev[i]));
     const uint64_t need = s->T + count;
     if (need > s->hcap) {
         const uint64_t nc = std::max<uint64_t>(need, s->hcap * 2);
@@ -1781,6 +1785,7 @@ static int ensure_sample_buffers(skis_sketch* s, uint64_t count, uint64_t slack,
         s->hcap = nc;
     }
     if (count > s->list_cap) {
+        s->list_cap = 0;
         dev_free(s->to_warp_ids, st);
         dev_free(s->to_cta_ids, st);
         dev_free(s->big_ids, st);

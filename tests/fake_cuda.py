@@ -49,7 +49,7 @@ def lib():
                                 ("fk_allocs", U64, []), ("fk_used", U64, []),
                                 ("fk_script", None, [P, P, ctypes.c_int]), ("fk_set_W", None, [P, U64]),
                                 ("fk_value", U64, [P, S]), ("fk_bytes", U64, [P, S]), ("fk_cursor", U64, [P]),
-                                ("fk_events", ctypes.c_int, [P]),
+                                ("fk_first_bad", U64, [P]), ("fk_events", ctypes.c_int, [P]),
                                 ("fk_launch", ctypes.c_int, [U64, P, U64, P, P])):
             f = getattr(h, name)
             f.restype, f.argtypes = res, args

@@ -63,6 +63,7 @@ uint64_t fk_bytes(const skis_sketch* s, const char* f) {
     return fk_live(p);
 }
 uint64_t fk_cursor(const skis_sketch* s) { return s->ctr ? s->ctr->arena : 0; }
+uint64_t fk_first_bad(const skis_sketch* s) { return s->qstatus->first_bad; }
 int fk_events(const skis_sketch* s) { return s->ev[0] && s->ev[1] && s->ev[2] && s->ev[3]; }
 
 }  // extern "C"
