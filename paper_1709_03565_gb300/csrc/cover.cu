@@ -1165,11 +1165,13 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) k_greedy_rounds(GreedyArgs 
         par ^= 1;
         return r;
     };
-    // the grid's best, known to every thread (one grid barrier)
-    auto grid_cand = [&](const Cand& c) -> Cand {
+    // the grid's best, known to every thread (one grid barrier). false, here and
+    // from its callers: a barrier's wait ran out, so that other blocks' writes may
+    // be missing; nothing is read by them, the block ends
+    auto grid_cand = [&](const Cand& c, Cand* best) -> bool {
         const Cand b = block_cand(c);
         if (threadIdx.x == 0) a.partial[blockIdx.x] = b;
-        bar.sync();
+        if (!bar.sync()) return false;
         Cand r = no_cand();
         for (unsigned i = lane; i < gridDim.x; i += 32) {
             const Cand x = ldcg_cand(a.partial + i);
@@ -1181,7 +1183,8 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) k_greedy_rounds(GreedyArgs 
         r.k0 = __shfl_sync(kFull, r.k0, src);
         r.id = __shfl_sync(kFull, r.id, src);
         r.d = __shfl_sync(kFull, r.d, src);
-        return r;
+        *best = r;
+        return true;
     };
     auto bucket = [&](uint32_t d, uint64_t w) { return greedy_bucket(d, one_f - w, a.ratio, a.ris); };
 
@@ -1197,9 +1200,9 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) k_greedy_rounds(GreedyArgs 
         }
         return block_cand(c);
     };
-    // Fills the pool from the vertices outside S; returns the best of the others.
+    // Fills the pool from the vertices outside S; *rest: the best of the others.
     bool hist_ready = true;  // k_greedy_init's
-    auto refill = [&]() -> Cand {
+    auto refill = [&](Cand* rest) -> bool {
         const int64_t stride = (int64_t)gridDim.x * kGreedyThreads;
         const int64_t first = (int64_t)blockIdx.x * kGreedyThreads + threadIdx.x;
         if (threadIdx.x == 0) s_cut = kBuckets;
@@ -1217,7 +1220,7 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) k_greedy_rounds(GreedyArgs 
             __syncthreads();
             for (int i = threadIdx.x; i < kBuckets; i += kGreedyThreads)
                 if (s_hist[i]) atomicAdd(&a.hist[i], s_hist[i]);
-            bar.sync();
+            if (!bar.sync()) return false;
         }
         hist_ready = false;
         // the lowest bucket down to which the pool has room: thread t counts
@@ -1275,7 +1278,7 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) k_greedy_rounds(GreedyArgs 
                 }
             }
         }
-        out = grid_cand(out);
+        if (!grid_cand(out, rest)) return false;
         const uint32_t np = min(__ldcg(&a.ctl->pool_n), (uint32_t)kGreedyThreads);
         p_id = kNone;
         if (threadIdx.x < np) {
@@ -1284,14 +1287,14 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) k_greedy_rounds(GreedyArgs 
             p_lo = a.inv_off[p_id];
             p_cnt = (uint32_t)(a.inv_off[p_id + 1] - p_lo);
         }
-        return out;
+        return true;
     };
     // The best vertex outside S by segments. Warp gw of W takes segments
     // gw + W i, 32 of them at a time (lane l: gw + W (32 i + l)); the block
     // index varies fastest over gw, so a few segments already spread over
     // every SM.
     bool seg_init = false;
-    auto seg_scan = [&]() -> Cand {
+    auto seg_scan = [&](Cand* best) -> bool {
         Cand wbest = no_cand();
         const int64_t W = (int64_t)gridDim.x * nw, gw = (int64_t)wib * gridDim.x + blockIdx.x;
         for (int64_t g0 = gw; g0 < a.nseg; g0 += 32 * W) {
@@ -1330,19 +1333,19 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) k_greedy_rounds(GreedyArgs 
                         if (cand_better(c, r)) r = c;
                     }
                 }
-                const int best = warp_best_lane(r);
-                r.k2 = __shfl_sync(kFull, r.k2, best);
-                r.k1 = __shfl_sync(kFull, r.k1, best);
-                r.k0 = __shfl_sync(kFull, r.k0, best);
-                r.id = __shfl_sync(kFull, r.id, best);
-                r.d = __shfl_sync(kFull, r.d, best);
+                const int top = warp_best_lane(r);
+                r.k2 = __shfl_sync(kFull, r.k2, top);
+                r.k1 = __shfl_sync(kFull, r.k1, top);
+                r.k0 = __shfl_sync(kFull, r.k0, top);
+                r.id = __shfl_sync(kFull, r.id, top);
+                r.d = __shfl_sync(kFull, r.d, top);
                 if (lane == src) b = r;
                 if (lane == 0) a.seg_best[g0 + src * W] = r;
             }
             if (cand_better(b, wbest)) wbest = b;
         }
         seg_init = true;
-        return grid_cand(wbest);
+        return grid_cand(wbest, best);
     };
 
     uint64_t cov = 0, sum_c = 0;  // running totals, kept by one thread
@@ -1359,9 +1362,9 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) k_greedy_rounds(GreedyArgs 
         }
         if (!found && seg_left) {
             --seg_left;
-            win = seg_scan();
+            if (!seg_scan(&win)) return;  // the host reports it
         } else if (!found) {
-            bound = refill();
+            if (!refill(&bound)) return;
             refilled = true;
             win = pool_best();
             if (!cand_better(win, bound)) win = bound;
