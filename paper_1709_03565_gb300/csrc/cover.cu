@@ -1269,10 +1269,15 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) k_greedy_rounds(GreedyArgs 
             for (int q = 0; q < 4; ++q) {
                 if (in4[q]) continue;
                 const uint32_t v = (uint32_t)(v0 + q * stride);
+                bool pooled = false;
                 if (bucket(d4[q], w4[q]) >= cut) {
                     const uint32_t slot = atomicAdd(&a.ctl->pool_n, 1u);
-                    if (slot < (uint32_t)kGreedyThreads) a.pool[slot] = v;
-                } else {
+                    pooled = slot < (uint32_t)kGreedyThreads;
+                    if (pooled) a.pool[slot] = v;
+                }
+                // the others bound the pool, one that found it full (it cannot
+                // while a key rounds alike here and in the histogram) included
+                if (!pooled) {
                     const Cand x = make(v, d4[q], w4[q]);
                     if (cand_better(x, out)) out = x;
                 }
