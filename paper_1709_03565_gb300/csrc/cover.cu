@@ -499,6 +499,9 @@ void coverage_shape(uint64_t T, int* blocks, int* glog) {
 // its prefix sums and a search of it per chunk of 2048, in seven launches; 154,
 // 66 and 50 us like this with chunks of 2048, 512 and 256.
 constexpr uint32_t kInvChunk = 256;
+// queue item: the seed's place in the batch (below 64 n <= 2^37) and the chunk
+// of its list (below 2^32 / kInvChunk = 2^24: a list holds a sample once)
+constexpr int kInvChunkBits = 24;
 
 struct InvWalk {
     const int64_t* off;     // the batch's seed offsets and seeds
@@ -509,7 +512,7 @@ struct InvWalk {
     const uint32_t* inv;
     unsigned long long* smask;
     unsigned long long* cov;      // qn counts
-    uint64_t* queue;              // seed << 32 | chunk
+    uint64_t* queue;              // seed << kInvChunkBits | chunk
     uint64_t queue_cap;
     unsigned long long* nqueue;   // chunks queued or past the capacity
 };
@@ -581,7 +584,7 @@ __global__ void __launch_bounds__(kCovThreads) k_cover_inv(InvWalk a, int mode) 
                     if (lane == 0) at = atomicAdd(a.nqueue, (unsigned long long)more);
                     at = __shfl_sync(kFull, at, 0);
                     const uint64_t fit = at < a.queue_cap ? min(more, (uint64_t)(a.queue_cap - at)) : 0;
-                    for (uint64_t c = lane; c < fit; c += 32) a.queue[at + c] = ((uint64_t)i << 32) | (c + 1);
+                    for (uint64_t c = lane; c < fit; c += 32) a.queue[at + c] = ((uint64_t)i << kInvChunkBits) | (c + 1);
                     rest = min(len, (fit + 1) * kInvChunk);
                 }
             }
@@ -592,9 +595,9 @@ __global__ void __launch_bounds__(kCovThreads) k_cover_inv(InvWalk a, int mode) 
     }
     for (uint64_t k = w0; k < queued; k += nwarps) {
         const uint64_t item = a.queue[k];
-        const int64_t i = (int64_t)(item >> 32);
+        const int64_t i = (int64_t)(item >> kInvChunkBits);
         const int32_t v = a.seeds[a.seed_base + i];
-        const uint64_t x = a.inv_off[v] + (item & 0xFFFFFFFFu) * kInvChunk;
+        const uint64_t x = a.inv_off[v] + (item & ((1u << kInvChunkBits) - 1u)) * kInvChunk;
         const int b = query_of(i);
         const uint32_t fresh = walk_list(a, x, min(x + kInvChunk, a.inv_off[v + 1]), 1ull << b, mode == 2);
         if (mode == 1) add(b, fresh);
