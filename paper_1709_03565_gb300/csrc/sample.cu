@@ -1926,7 +1926,7 @@ static int occupancy_grid(const void* kernel, int threads, int override_blocks, 
     return SKIS_OK;
 }
 
-int sketch_sample(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* err) {
+static int sample_passes(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* err) {
     const skis_graph* g = s->g;
     if (g->W == 0 && !s->ris) {
         *err = "skis_sample: Gamma = 0, the graph has no non-singular sample";
@@ -2172,6 +2172,16 @@ int sketch_sample(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* 
         return SKIS_ERR_RETRY_LIMIT;
     }
     return SKIS_OK;
+}
+
+int sketch_sample(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* err) {
+    const uint64_t T0 = s->T;
+    const int rc = sample_passes(s, count, st, err);
+    // a call that appended nothing: what its passes reserved is free again (and is
+    // not taken for demand when a later call's overflow sizes the arena)
+    if (rc != SKIS_OK && s->T == T0 && s->ctr)
+        cudaMemcpyAsync(&s->ctr->arena, &s->arena_used, sizeof(s->arena_used), cudaMemcpyHostToDevice, st);
+    return rc;
 }
 
 // The one batch sample whose inclusive prefix of sizes first reaches need:

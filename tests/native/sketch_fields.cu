@@ -33,6 +33,7 @@ void fk_on_launch(const char* kernel) {
     const Pass& p = g_passes[g_next++];
     g_sketch->ctr->novf = p.novf;
     g_sketch->ctr->arena += p.arena;
+    if (g_sketch->ctr->arena > g_sketch->arena_cap && !p.novf) g_sketch->ctr->novf = 1;  // the last one does not fit
     g_sketch->ctr->n_big = p.n_big;
 }
 
