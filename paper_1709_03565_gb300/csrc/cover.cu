@@ -704,6 +704,8 @@ int sketch_order_arena(skis_sketch* s, cudaStream_t st, std::string* err) {
             CV_CUDA(cudaMemcpyAsync(&s->ctr->arena, &cur, sizeof(cur), cudaMemcpyHostToDevice, st));
         }
         s->arena_used = E0 + E1;
+        s->arena_drawn = s->T;
+        s->arena_ends = 0;
         CV_CUDA(cudaStreamSynchronize(st));
         return SKIS_OK;
     };

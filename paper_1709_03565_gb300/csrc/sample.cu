@@ -1759,6 +1759,26 @@ static cudaError_t grow_copy(T** p, uint64_t old_n, uint64_t new_n, cudaStream_t
 // threads of the CTA-tier blocks that the slots are counted for (launch_cta)
 static int cta_block(const skis_sketch* s) { return s->cta_threads == 512 ? 512 : kCtaBlock; }
 
+// Arena entries a sketch's first `count` samples get: room for samples of 128
+// members within 2 GiB, at least 8 a sample. Sizes run from 4 members a sample
+// (trivalency) to 60-75 (weighted cascade, LT 18), and a pass that overflows
+// draws what did not fit again.
+static uint64_t first_arena(uint64_t count) {
+    return std::max<uint64_t>({count * 8, std::min<uint64_t>(count * 128, 1u << 29), 1u << 20});
+}
+
+// Entries that `count` more samples are given: what the samples so far had, as
+// far as it is known. The entries they reserved are no fewer than their members,
+// and more by the unused ends of the warps' chunks, at most arena_ends; a first
+// allotment's size is taken within these two. (By the reserved entries alone, a
+// call for one sample, which opens a chunk for it, made the next call of 10M
+// samples ask for 115 GB.)
+static uint64_t more_arena(const skis_sketch* s, uint64_t count, uint64_t used) {
+    const double c = 1.125 * (double)count / (double)std::max<uint64_t>(s->arena_drawn, 1);
+    const double least = c * (double)(used - std::min(used, s->arena_ends)), most = c * (double)used;
+    return (uint64_t)std::min(std::max(least, std::min(most, (double)first_arena(count))), (double)(1ull << 50));
+}
+
 // slack: arena entries that the tiers' warps may leave unused at the ends of their chunks;
 // warps: the warp tier's warps (0: no such tier)
 static int ensure_sample_buffers(skis_sketch* s, uint64_t count, uint64_t slack, uint64_t warps, cudaStream_t st,
@@ -1806,19 +1826,15 @@ static int ensure_sample_buffers(skis_sketch* s, uint64_t count, uint64_t slack,
         s->list_cap = count;
     }
     if (!s->arena) {
-        // the default: room for samples of 128 members within 2 GiB, at least 8 a sample, and the
-        // ends of the warps' chunks. Sizes run from 4 members a sample (trivalency) to 60-75
-        // (weighted cascade, LT 18), and a pass that overflows draws what did not fit again
         uint64_t cap = s->arena_hint;
-        if (!cap) cap = std::max<uint64_t>({count * 8, std::min<uint64_t>(count * 128, 1u << 29), 1u << 20}) + slack;
+        if (!cap) cap = first_arena(count) + slack;
         SK_CUDA(dev_alloc_t(&s->arena, (size_t)cap, st));
         s->arena_cap = cap;
     } else if (s->T > 0) {
         // more samples like the ones so far: the arena grows before the pass
         // when they would not fit (or, without the memory now, as it overflows)
         const uint64_t used = std::min(s->arena_used, s->arena_cap);
-        const double mean = (double)used / (double)s->T;
-        const uint64_t want = used + (uint64_t)((double)count * mean * 1.125) + slack;
+        const uint64_t want = used + more_arena(s, count, used) + slack;
         if (want > s->arena_cap) {
             const cudaError_t e = grow_copy(&s->arena, used, std::max(want, s->arena_cap * 2), st);
             if (e == cudaSuccess) s->arena_cap = std::max(want, s->arena_cap * 2);
@@ -2158,6 +2174,8 @@ static int sample_passes(skis_sketch* s, uint64_t count, cudaStream_t st, std::s
     }
     s->T += count;
     s->arena_used = hc.arena;
+    s->arena_drawn += count;
+    s->arena_ends += slack * s->last_passes;
     if (counting) {
         s->vcount_ok = true;
         s->vcount_T = s->T;

@@ -300,6 +300,8 @@ struct skis_sketch {
     uint64_t arena_cap = 0;
     uint64_t arena_hint = 0;
     uint64_t arena_used = 0;             // the arena cursor after the last call
+    uint64_t arena_drawn = 0;            // samples drawn into those entries, dropped ones included,
+    uint64_t arena_ends = 0;             // and how many of the entries their warps may have left unused
     skis::SampleCounters* ctr = nullptr;
     skis::DevStatus* status = nullptr;
     uint64_t* to_warp_ids = nullptr;     // thread tier -> warp tier
