@@ -20,9 +20,17 @@ static std::once_flag g_pool_once;
 static std::atomic<uint64_t> g_allocs{0};
 uint64_t allocations() { return g_allocs.load(std::memory_order_relaxed); }
 
+// An allocation that failed is reported by its status alone: the runtime also
+// keeps it as the thread's last error, where the next launch's check, on this
+// call or a later one, would find it and refuse a call that has its memory.
+static cudaError_t taken(cudaError_t e) {
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+    return e;
+}
+
 cudaError_t dev_malloc(void** p, size_t bytes) {
     g_allocs.fetch_add(1, std::memory_order_relaxed);
-    return cudaMalloc(p, bytes);
+    return taken(cudaMalloc(p, bytes));
 }
 
 cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t st) {
@@ -40,7 +48,7 @@ cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t st) {
     *p = nullptr;
     if (bytes == 0) bytes = 16;
     g_allocs.fetch_add(1, std::memory_order_relaxed);
-    return cudaMallocAsync(p, bytes, st);
+    return taken(cudaMallocAsync(p, bytes, st));
 }
 
 void dev_free(void* p, cudaStream_t st) {

@@ -1838,8 +1838,7 @@ static int ensure_sample_buffers(skis_sketch* s, uint64_t count, uint64_t slack,
         if (want > s->arena_cap) {
             const cudaError_t e = grow_copy(&s->arena, used, std::max(want, s->arena_cap * 2), st);
             if (e == cudaSuccess) s->arena_cap = std::max(want, s->arena_cap * 2);
-            else if (e == cudaErrorMemoryAllocation) cudaGetLastError();
-            else SK_CUDA(e);
+            else if (e != cudaErrorMemoryAllocation) SK_CUDA(e);
         }
     }
     if (g->lt) {  // medium LT walks: one table and list per lane

@@ -45,7 +45,7 @@ def lib():
             f = getattr(h, name)
             f.restype, f.argtypes = res, args
         P, U64, S = ctypes.c_void_p, ctypes.c_uint64, ctypes.c_char_p
-        for name, res, args in (("fk_start", None, [U64]), ("fk_fail_at", None, [ctypes.c_int64]),
+        for name, res, args in (("fk_start", None, [U64]), ("fk_fail_at", None, [ctypes.c_int64, ctypes.c_int]),
                                 ("fk_allocs", U64, []), ("fk_used", U64, []),
                                 ("fk_script", None, [P, P, ctypes.c_int]), ("fk_set_W", None, [P, U64]),
                                 ("fk_value", U64, [P, S]), ("fk_bytes", U64, [P, S]), ("fk_cursor", U64, [P]),

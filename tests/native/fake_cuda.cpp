@@ -29,6 +29,8 @@ struct State {
     std::map<char*, size_t> live;  // device allocations
     uint64_t limit = ~0ull, used = 0, allocs = 0;
     int64_t fail_at = 0;
+    bool fail_on = false;                  // and every one after it
+    cudaError_t last = cudaSuccess;        // until cudaGetLastError takes it
     std::map<const void*, std::string> names;
     std::vector<Launch> launches;
 };
@@ -42,11 +44,13 @@ cudaError_t alloc(void** p, size_t bytes) {
     std::lock_guard<std::recursive_mutex> lk(S.mu);
     *p = nullptr;
     ++S.allocs;
-    if (S.fail_at > 0 && --S.fail_at == 0) return cudaErrorMemoryAllocation;
-    if (bytes > S.limit || S.used > S.limit - bytes) return cudaErrorMemoryAllocation;
-    void* q = mmap(nullptr, (bytes + kPage - 1) / kPage * kPage, PROT_READ | PROT_WRITE,
-                   MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
-    if (q == MAP_FAILED) return cudaErrorMemoryAllocation;
+    bool fail = S.fail_at > 0 && --S.fail_at == 0;
+    if (fail && S.fail_on) S.fail_at = 1;
+    fail = fail || bytes > S.limit || S.used > S.limit - bytes;
+    void* q = fail ? MAP_FAILED
+                   : mmap(nullptr, (bytes + kPage - 1) / kPage * kPage, PROT_READ | PROT_WRITE,
+                          MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
+    if (q == MAP_FAILED) return S.last = cudaErrorMemoryAllocation;
     S.live[(char*)q] = bytes;
     S.used += bytes;
     *p = q;
@@ -146,7 +150,11 @@ cudaError_t cudaGetDevice(int* d) {
     *d = 0;
     return cudaSuccess;
 }
-cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaGetLastError() {
+    const cudaError_t e = state().last;
+    state().last = cudaSuccess;
+    return e;
+}
 const char* cudaGetErrorString(cudaError_t e) { return e == cudaErrorMemoryAllocation ? "out of memory" : "error"; }
 cudaError_t cudaGetSymbolAddress(void** p, const void*) {
     *p = nullptr;
@@ -191,9 +199,14 @@ void fk_start(uint64_t limit) {
     S.limit = limit;
     S.allocs = 0;
     S.fail_at = 0;
+    S.last = cudaSuccess;
     S.launches.clear();
 }
-void fk_fail_at(int64_t k) { state().fail_at = k; }  // the k-th allocation from here fails (0: none)
+// the k-th allocation from here fails, and every one after it if `on` (0: none)
+void fk_fail_at(int64_t k, int on) {
+    state().fail_at = k;
+    state().fail_on = on != 0;
+}
 uint64_t fk_allocs() { return state().allocs; }
 uint64_t fk_live(const void* p) {  // bytes of the live allocation that starts at p, 0 if there is none
     State& S = state();

@@ -33,8 +33,9 @@ def test_after_the_pass_for_outgrown_samples_failed():
     s.option(skis.SKIS_OPT_CTA_SLOTS, 4)
     assert s.sample(10) == skis.SKIS_OK
     s.script((0, 3000, 5))
-    s.fk.fk_fail_at(1)  # the n-entry queues
+    s.fk.fk_fail_at(1, 1)  # the n-entry queues
     assert s.sample(10) == skis.SKIS_ENOMEM
+    s.fk.fk_fail_at(0, 0)
     assert s.fk.fk_cursor(s.s) == 0 and s.value("T") == 10
     s.script((0, 3000, 5))
     assert s.sample(10) == skis.SKIS_OK

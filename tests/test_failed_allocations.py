@@ -36,9 +36,9 @@ def test_sampling_after_any_allocation_failed(before, lt):
         s = fake_cuda.Sketch(N, lt=lt)
         if before:
             assert s.sample(before) == skis.SKIS_OK
-        s.fk.fk_fail_at(k)
+        s.fk.fk_fail_at(k, 1)
         rc = s.sample(9000)
-        s.fk.fk_fail_at(0)
+        s.fk.fk_fail_at(0, 0)
         assert rc in (skis.SKIS_OK, skis.SKIS_ENOMEM)
         done = before + (9000 if rc == skis.SKIS_OK else 0)
         for count in (60, 7000):
@@ -65,9 +65,9 @@ def test_queries_after_any_allocation_failed(mode, T):
         s = fake_cuda.Sketch(N)
         s.option(skis.SKIS_OPT_QUERY_INDEX, mode)
         assert s.sample(T) == skis.SKIS_OK
-        s.fk.fk_fail_at(k)
+        s.fk.fk_fail_at(k, 1)
         rc = _estimate(s, off, seeds)
-        s.fk.fk_fail_at(0)
+        s.fk.fk_fail_at(0, 0)
         if rc == skis.SKIS_OK:
             s.close()
             assert k > 5
