@@ -1827,7 +1827,7 @@ static int ensure_sample_buffers(skis_sketch* s, uint64_t count, uint64_t slack,
     }
     if (!s->arena) {
         uint64_t cap = s->arena_hint;
-        if (!cap) cap = first_arena(count) + slack;
+        if (!cap) cap = s->lean ? std::max<uint64_t>(count * 8, 1u << 20) : first_arena(count) + slack;
         SK_CUDA(dev_alloc_t(&s->arena, (size_t)cap, st));
         s->arena_cap = cap;
     } else if (s->T > 0) {
@@ -1842,7 +1842,7 @@ static int ensure_sample_buffers(skis_sketch* s, uint64_t count, uint64_t slack,
         }
     }
     if (g->lt) {  // medium LT walks: one table and list per lane
-        s->lt_mid_lanes = (uint64_t)sm_count() * kLtMidBlock * kLtMidBlocks;
+        s->lt_mid_lanes = (uint64_t)std::max(1, (sm_count() * kLtMidBlocks) >> s->lean) * kLtMidBlock;
         if (!s->lt_hash) SK_CUDA(dev_alloc_t(&s->lt_hash, (size_t)(s->lt_mid_lanes * kLtMidHash), st));
         if (!s->lt_list) SK_CUDA(dev_alloc_t(&s->lt_list, (size_t)(s->lt_mid_lanes * kLtMidCap), st));
     }
@@ -1868,6 +1868,7 @@ static int ensure_sample_buffers(skis_sketch* s, uint64_t count, uint64_t slack,
         const uint64_t budget = 12ull << 30;
         const uint64_t per_sm = g->lt ? 2 : 1024 / cta_block(s);
         slots = (int)std::min<uint64_t>((uint64_t)sm_count() * per_sm, std::max<uint64_t>(1, budget / per_slot));
+        slots = std::max(1, slots >> s->lean);
     }
     if (slots != s->cta_slots_alloc || qcap != s->queue_cap) {
         dev_free(s->bitmaps, st);
@@ -1896,7 +1897,8 @@ static int ensure_big_slots(skis_sketch* s, cudaStream_t st, std::string* err) {
     if (s->big_queues) return SKIS_OK;
     const uint64_t n = (uint64_t)s->g->n;
     const uint64_t budget = 8ull << 30;
-    const int slots = (int)std::min<uint64_t>((uint64_t)s->cta_slots_alloc, std::max<uint64_t>(1, budget / (n * 4)));
+    int slots = (int)std::min<uint64_t>((uint64_t)s->cta_slots_alloc, std::max<uint64_t>(1, budget / (n * 4)));
+    slots = std::max(1, slots >> s->lean);
     SK_CUDA(dev_alloc_t(&s->big_queues, (size_t)(n * slots), st));
     s->big_slots = slots;
     return SKIS_OK;
@@ -1959,6 +1961,7 @@ static int sample_passes(skis_sketch* s, uint64_t count, cudaStream_t st, std::s
                         (count + kWarpThreads / 32 - 1) / (kWarpThreads / 32), err, &warp_blocks);
     if (rc != SKIS_OK) return rc;
     if (s->warp_blocks > 0) warp_blocks = std::min(warp_blocks, s->warp_blocks);
+    warp_blocks = std::max(1, warp_blocks >> s->lean);
     if (g->lt) {
         rc = occupancy_grid((const void*)k_lt_walk, kLtBlock, s->thread_blocks, (count + kLtBlock - 1) / kLtBlock,
                             err, &lt_blocks);
@@ -2021,7 +2024,6 @@ static int sample_passes(skis_sketch* s, uint64_t count, cudaStream_t st, std::s
     // per-vertex member counts, kept while they describe exactly samples
     // [0, T): invalid until this call succeeds
     const bool counting = s->vcount_ok && s->vcount_T == s->T;
-    s->vcount_ok = false;
     base.vcount = nullptr;
     if (counting) {
         if (!s->vcount) {
@@ -2030,6 +2032,7 @@ static int sample_passes(skis_sketch* s, uint64_t count, cudaStream_t st, std::s
         }
         base.vcount = s->vcount;
     }
+    s->vcount_ok = false;
     base.chain = nullptr;
     if (s->bucket && !s->ris && !g->lt) {
         rc = graph_ensure_chain(g, st, err);
@@ -2152,12 +2155,11 @@ static int sample_passes(skis_sketch* s, uint64_t count, cudaStream_t st, std::s
         // reservation, placed or not, so what the rerun needs is known up to
         // the ends of chunks that a next sample does not fit in
         const uint64_t old_cap = s->arena_cap;
-        const uint64_t new_cap = std::max<uint64_t>(old_cap * 2, hc.arena + hc.arena / 8) + slack;
-        rc = [&]() -> int {
-            SK_CUDA(grow_copy(&s->arena, old_cap, new_cap, st));
-            return SKIS_OK;
-        }();
-        if (rc != SKIS_OK) {
+        uint64_t new_cap = std::max<uint64_t>(old_cap * 2, hc.arena + hc.arena / 8) + slack;
+        cudaError_t e = grow_copy(&s->arena, old_cap, new_cap, st);
+        if (e == cudaErrorMemoryAllocation)  // no room for all of it: what fits at twice the size, then further
+            e = grow_copy(&s->arena, old_cap, new_cap = old_cap * 2, st);
+        if (e != cudaSuccess) {
             *err = "skis_sample: the member arena could not grow to " + std::to_string(new_cap) + " entries";
             return SKIS_ERR_ARENA_FULL;
         }
@@ -2191,14 +2193,53 @@ static int sample_passes(skis_sketch* s, uint64_t count, cudaStream_t st, std::s
     return SKIS_OK;
 }
 
+// Gives the tiers' scratch back, and an arena of the library's own choice that
+// holds no sample yet.
+static void release_scratch(skis_sketch* s, cudaStream_t st) {
+    dev_free(s->spill_hash, st);
+    dev_free(s->spill_queue, st);
+    dev_free(s->bitmaps, st);
+    dev_free(s->slot_clean, st);
+    dev_free(s->queues, st);
+    dev_free(s->big_queues, st);
+    dev_free(s->lt_hash, st);
+    dev_free(s->lt_list, st);
+    s->spill_hash = s->bitmaps = s->slot_clean = s->lt_hash = nullptr;
+    s->spill_queue = s->queues = s->big_queues = s->lt_list = nullptr;
+    s->spill_warps = 0;
+    s->cta_slots_alloc = s->big_slots = 0;
+    if (s->T == 0 && !s->arena_hint) {
+        dev_free(s->arena, st);
+        s->arena = nullptr;
+        s->arena_cap = s->arena_used = 0;
+    }
+    cudaStreamSynchronize(st);  // the pool may merge and unmap what was freed
+}
+
+// The passes of one call; where the device has no room for their scratch, again
+// with half of the slots, spill slots and LT lanes each time, and room for 8
+// members a sample at first (the sketch keeps to what was found). At half, all
+// of it takes less than 608 CTA-tier slots within 8 GB did with blocks of 256.
 int sketch_sample(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* err) {
+    constexpr int kLeanMost = 11;  // one slot, one block of warps
     const uint64_t T0 = s->T;
-    const int rc = sample_passes(s, count, st, err);
-    // a call that appended nothing: what its passes reserved is free again (and is
-    // not taken for demand when a later call's overflow sizes the arena)
-    if (rc != SKIS_OK && s->T == T0 && s->ctr)
-        cudaMemcpyAsync(&s->ctr->arena, &s->arena_used, sizeof(s->arena_used), cudaMemcpyHostToDevice, st);
-    return rc;
+    const int lean0 = s->lean;
+    for (;;) {
+        const int rc = sample_passes(s, count, st, err);
+        if (rc == SKIS_OK || s->T != T0) return rc;
+        // a call that appended nothing: what its passes reserved is free again (and is
+        // not taken for demand when a later call's overflow sizes the arena)
+        if (s->ctr)
+            cudaMemcpyAsync(&s->ctr->arena, &s->arena_used, sizeof(s->arena_used), cudaMemcpyHostToDevice, st);
+        const bool again = (rc == SKIS_ENOMEM && s->lean < kLeanMost) || (rc == SKIS_ERR_ARENA_FULL && s->lean == lean0);
+        if (again || s->lean != lean0) release_scratch(s, st);  // its sizes go by lean
+        if (!again) {
+            s->lean = lean0;
+            return rc;
+        }
+        ++s->lean;
+        err->clear();
+    }
 }
 
 // The one batch sample whose inclusive prefix of sizes first reaches need:

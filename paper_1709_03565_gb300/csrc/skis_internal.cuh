@@ -327,6 +327,7 @@ struct skis_sketch {
     uint64_t lt_mid_lanes = 0;
     int cta_slots_alloc = 0;
     uint64_t bitmap_words = 0;
+    int lean = 0;                        // the device had no room for more than 2^-lean of the tiers' scratch
     // options
     uint32_t retry_cap = 1u << 24;
     int cta_slots = 0;                   // 0 = automatic

@@ -94,6 +94,7 @@ class Sketch:
         return out
 
     def close(self):
-        self.fk.skis_sketch_free(self.s)
+        if self.s:
+            self.fk.skis_sketch_free(self.s)
         self.fk.skis_graph_free(self.g)
         assert self.fk.fk_used() == self.before

@@ -45,7 +45,7 @@ uint64_t fk_value(const skis_sketch* s, const char* f) {
 #define FIELD(x) \
     if (n == #x) return (uint64_t)s->x;
     FIELD(T) FIELD(hcap) FIELD(list_cap) FIELD(arena_cap) FIELD(spill_warps) FIELD(cta_slots_alloc) FIELD(queue_cap)
-    FIELD(bitmap_words) FIELD(big_slots) FIELD(lt_mid_lanes) FIELD(smask_cap) FIELD(touched_cap)
+    FIELD(bitmap_words) FIELD(big_slots) FIELD(lean) FIELD(lt_mid_lanes) FIELD(smask_cap) FIELD(touched_cap)
 #undef FIELD
     return ~0ull;
 }

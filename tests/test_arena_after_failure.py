@@ -17,7 +17,7 @@ def test_the_cursor_returns_to_the_samples_end(before, lt):
         assert s.sample(before) == skis.SKIS_OK
         used = 7777
     for _ in range(3):
-        s.script((900, 1 << 36, 0))  # the samples of this pass would take 256 GiB
+        s.script(*[(900, 1 << 36, 0)] * 200)  # the samples of a pass would take 256 GiB, whatever the arena holds
         assert s.sample(1000) == skis.SKIS_ERR_ARENA_FULL
         assert s.value("T") == before
         assert s.fk.fk_cursor(s.s) == used

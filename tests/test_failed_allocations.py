@@ -9,8 +9,9 @@ import paper_1709_03565_gb300 as skis
 N = 3000
 
 
-def _sampler_buffers(s, count, lt):
-    """The bytes the sampling kernels of a call for `count` more samples may touch, buffer by buffer."""
+def sampler_buffers(s, count, lt, n=N, first=0):
+    """The bytes the sampling kernels of a call for `count` more samples (launches from record `first` on) may touch,
+    buffer by buffer."""
     T, slots = s.value("T"), s.value("cta_slots_alloc")
     want = {"ctr": 72, "status": 16, "arena": s.value("arena_cap") * 4, "h_off": 8 * T, "h_len": 4 * T, "h_src": 4 * T,
             "h_retries": 4 * T, "h_coins": 8 * T, "to_warp_ids": 8 * count, "to_cta_ids": 8 * count, "big_ids": 8 * count,
@@ -18,13 +19,15 @@ def _sampler_buffers(s, count, lt):
             "bitmaps": 4 * slots * s.value("bitmap_words"), "queues": 4 * slots * s.value("queue_cap"),
             "slot_clean": 4 * slots}
     if lt:
-        want.update({"lt_hash": s.value("lt_mid_lanes") * 2048 * 4, "lt_list": s.value("lt_mid_lanes") * 1024 * 4})
+        lanes = 128 * [g for name, g, _ in s.launches()[first:] if "k_lt_mid" in name][-1]
+        want.update({"lt_hash": lanes * 2048 * 4, "lt_list": lanes * 1024 * 4})
     else:
-        grid = [g for name, g, _ in s.launches() if "k_iis_warp" in name][-1]
-        assert s.value("spill_warps") >= 8 * grid
-        want.update({"spill_hash": 8 * grid * 4096 * 4, "spill_queue": 8 * grid * 1536 * 4})
+        grid = [g for name, g, _ in s.launches()[first:] if "k_iis_warp" in name][-1]
+        slot_hash, slot_members = (8192, 4096) if n >= 24_576 else (4096, 1536)
+        want.update({"spill_hash": 8 * grid * slot_hash * 4, "spill_queue": 8 * grid * slot_members * 4})
     for name, size in want.items():
         assert size > 0 and s.bytes(name) >= size, name
+    assert all(g <= slots for name, g, _ in s.launches()[first:] if "k_iis_cta" in name or "k_lt_long" in name)
 
 
 @pytest.mark.parametrize("lt", [False, True])
@@ -45,7 +48,7 @@ def test_sampling_after_any_allocation_failed(before, lt):
             assert s.sample(count) == skis.SKIS_OK
             done += count
             assert s.value("T") == done and s.fk.fk_events(s.s)
-            _sampler_buffers(s, count, lt)
+            sampler_buffers(s, count, lt)
         allocs = s.fk.fk_allocs()
         s.close()
         if k > allocs:  # every allocation has failed once
