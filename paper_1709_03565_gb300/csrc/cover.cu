@@ -719,9 +719,9 @@ int sketch_order_arena(skis_sketch* s, cudaStream_t st, std::string* err) {
     return rc;
 }
 
-int sketch_estimate(skis_sketch* s, int32_t q, const int64_t* d_off, const int32_t* d_seeds, const int64_t* h_off,
-                    int64_t* d_cov, double* d_est, cudaStream_t st, std::string* err, void* d_pack, void* h_pack,
-                    size_t pack_bytes) {
+static int estimate_queries(skis_sketch* s, int32_t q, const int64_t* d_off, const int32_t* d_seeds,
+                            const int64_t* h_off, int64_t* d_cov, double* d_est, cudaStream_t st, std::string* err,
+                            void* d_pack, void* h_pack, size_t pack_bytes) {
     const char* where = "skis_estimate";
     const skis_graph* g = s->g;
     if (s->T == 0) {
@@ -857,6 +857,14 @@ int sketch_estimate(skis_sketch* s, int32_t q, const int64_t* d_off, const int32
         return SKIS_EINVAL;
     }
     return SKIS_OK;
+}
+
+int sketch_estimate(skis_sketch* s, int32_t q, const int64_t* d_off, const int32_t* d_seeds, const int64_t* h_off,
+                    int64_t* d_cov, double* d_est, cudaStream_t st, std::string* err, void* d_pack, void* h_pack,
+                    size_t pack_bytes) {
+    return with_room(s, st, err, [&] {  // every buffer is there before the first launch
+        return estimate_queries(s, q, d_off, d_seeds, h_off, d_cov, d_est, st, err, d_pack, h_pack, pack_bytes);
+    });
 }
 
 // --------------------------------------------------------------- greedy
@@ -1479,7 +1487,7 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) k_greedy_rounds(GreedyArgs 
     }
 }
 
-int sketch_inverted(skis_sketch* s, cudaStream_t st, std::string* err) {
+static int build_inverted(skis_sketch* s, cudaStream_t st, std::string* err) {
     const char* where = "inverted index";
     if (s->inv && s->inv_T == s->T) return SKIS_OK;
     const int64_t n = s->g->n;
@@ -1519,6 +1527,10 @@ int sketch_inverted(skis_sketch* s, cudaStream_t st, std::string* err) {
     dev_free(cursor, st);
     s->inv_T = T;
     return SKIS_OK;
+}
+
+int sketch_inverted(skis_sketch* s, cudaStream_t st, std::string* err) {
+    return with_room(s, st, err, [&] { return build_inverted(s, st, err); });
 }
 
 constexpr int32_t kGreedyPacked = 4096;  // largest k whose results come back in one copy through the stack
@@ -1568,7 +1580,11 @@ int sketch_greedy(skis_sketch* s, int32_t k, int32_t* h_seeds, int64_t* h_cov, d
         const size_t at_pool = take(kGreedyThreads * sizeof(uint32_t)), at_delta = take((size_t)n * sizeof(uint32_t));
         const bool packed = k <= kGreedyPacked;  // else straight to the caller's arrays
         alignas(128) char h_out[sizeof(GreedyCtl) + kGreedyPacked * 20 + 3 * 128];
-        CV_CUDA(dev_alloc_t(&buf, bytes, st));
+        const int room = with_room(s, st, err, [&]() -> int {
+            CV_CUDA(dev_alloc_t(&buf, bytes, st));
+            return SKIS_OK;
+        });
+        if (room != SKIS_OK) return room;
         CV_CUDA(cudaMemsetAsync(buf, 0, zeroed, st));
         GreedyArgs ga;
         ga.w = g->w;
@@ -1813,15 +1829,19 @@ int sketch_greedy_sharded(skis_sketch* s, int32_t k, int32_t* h_seeds, int64_t* 
     const int nb = sm_count() * 4;
     const uint64_t cwords = std::max<uint64_t>(1, (s->T + 31) / 32);
     auto body = [&]() -> int {
-        CV_CUDA(dev_alloc_t(&delta, (size_t)n, st));
-        CV_CUDA(dev_alloc_t(&inS, (size_t)n, st));
-        CV_CUDA(dev_alloc_t(&covered, (size_t)cwords, st));
-        CV_CUDA(dev_alloc_t(&win, 1, st));
-        CV_CUDA(dev_alloc_t(&partial, (size_t)nb, st));
-        CV_CUDA(dev_alloc_t(&d_seeds, (size_t)k, st));
-        CV_CUDA(dev_alloc_t(&d_cov, (size_t)k, st));
-        CV_CUDA(dev_alloc_t(&d_est, (size_t)k, st));
-        CV_CUDA(dev_alloc_t(&acc, 2, st));
+        int e = with_room(s, st, err, [&]() -> int {
+            if (!delta) CV_CUDA(dev_alloc_t(&delta, (size_t)n, st));
+            if (!inS) CV_CUDA(dev_alloc_t(&inS, (size_t)n, st));
+            if (!covered) CV_CUDA(dev_alloc_t(&covered, (size_t)cwords, st));
+            if (!win) CV_CUDA(dev_alloc_t(&win, 1, st));
+            if (!partial) CV_CUDA(dev_alloc_t(&partial, (size_t)nb, st));
+            if (!d_seeds) CV_CUDA(dev_alloc_t(&d_seeds, (size_t)k, st));
+            if (!d_cov) CV_CUDA(dev_alloc_t(&d_cov, (size_t)k, st));
+            if (!d_est) CV_CUDA(dev_alloc_t(&d_est, (size_t)k, st));
+            if (!acc) CV_CUDA(dev_alloc_t(&acc, 2, st));
+            return SKIS_OK;
+        });
+        if (e != SKIS_OK) return e;
         CV_CUDA(cudaMemsetAsync(inS, 0, (size_t)n, st));
         CV_CUDA(cudaMemsetAsync(covered, 0, cwords * sizeof(uint32_t), st));
         CV_CUDA(cudaMemsetAsync(acc, 0, 2 * sizeof(uint64_t), st));
@@ -1829,7 +1849,7 @@ int sketch_greedy_sharded(skis_sketch* s, int32_t k, int32_t* h_seeds, int64_t* 
         const int b1 = (int)std::max<int64_t>(1, std::min<int64_t>((n + 256) / 256, (int64_t)sm_count() * 8));
         k_shard_delta0<<<b1, 256, 0, st>>>(s->inv_off, n, exch); note_launch();
         CV_CUDA(cudaGetLastError());
-        int e = exchange(fn, ctx, exch, n + 1, st, where, err);
+        e = exchange(fn, ctx, exch, n + 1, st, where, err);
         if (e != SKIS_OK) return e;
         CV_CUDA(cudaMemcpyAsync(delta, exch, (size_t)n * sizeof(int64_t), cudaMemcpyDeviceToDevice, st));
         const int cb = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)sm_count() * 8, (s->T + 255) / 256));

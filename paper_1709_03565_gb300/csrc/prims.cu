@@ -55,6 +55,14 @@ void dev_free(void* p, cudaStream_t st) {
     if (p) cudaFreeAsync(p, st);
 }
 
+void dev_trim(cudaStream_t st) {
+    int dev = 0;
+    cudaMemPool_t pool;
+    if (cudaStreamSynchronize(st) == cudaSuccess && cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess)
+        cudaMemPoolTrimTo(pool, 0);
+}
+
 int sm_count() {
     static int cached = 0;
     if (cached == 0) {

@@ -2193,9 +2193,10 @@ static int sample_passes(skis_sketch* s, uint64_t count, cudaStream_t st, std::s
     return SKIS_OK;
 }
 
-// Gives the tiers' scratch back, and an arena of the library's own choice that
-// holds no sample yet.
-static void release_scratch(skis_sketch* s, cudaStream_t st) {
+// The tiers' scratch, and an arena of the library's own choice that holds no
+// sample yet.
+bool sketch_release_scratch(skis_sketch* s, cudaStream_t st) {
+    const bool any = s->spill_hash || s->bitmaps || s->queues || s->lt_hash || s->lt_list;
     dev_free(s->spill_hash, st);
     dev_free(s->spill_queue, st);
     dev_free(s->bitmaps, st);
@@ -2213,7 +2214,8 @@ static void release_scratch(skis_sketch* s, cudaStream_t st) {
         s->arena = nullptr;
         s->arena_cap = s->arena_used = 0;
     }
-    cudaStreamSynchronize(st);  // the pool may merge and unmap what was freed
+    dev_trim(st);
+    return any;
 }
 
 // The passes of one call; where the device has no room for their scratch, again
@@ -2232,7 +2234,7 @@ int sketch_sample(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* 
         if (s->ctr)
             cudaMemcpyAsync(&s->ctr->arena, &s->arena_used, sizeof(s->arena_used), cudaMemcpyHostToDevice, st);
         const bool again = (rc == SKIS_ENOMEM && s->lean < kLeanMost) || (rc == SKIS_ERR_ARENA_FULL && s->lean == lean0);
-        if (again || s->lean != lean0) release_scratch(s, st);  // its sizes go by lean
+        if (again || s->lean != lean0) sketch_release_scratch(s, st);  // its sizes go by lean
         if (!again) {
             s->lean = lean0;
             return rc;

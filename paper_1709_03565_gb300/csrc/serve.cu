@@ -121,7 +121,7 @@ extern "C" int skis_server_create(skis_server** out, skis_sketch* s, int32_t slo
             // members are laid out in id order now, so that no later scan of
             // the (unchanged) sketch moves them while the server reads them
             std::string err;
-            int rc = sketch_order_arena(s, s->stream, &err);
+            int rc = with_room(s, s->stream, &err, [&] { return sketch_order_arena(s, s->stream, &err); });
             if (rc == SKIS_OK) rc = sketch_inverted(s, s->stream, &err);
             if (rc != SKIS_OK) return serve_fail(rc, err);
             const cudaError_t e = cudaStreamSynchronize(s->stream);
@@ -133,7 +133,7 @@ extern "C" int skis_server_create(skis_server** out, skis_sketch* s, int32_t slo
         srv->seed_cap = seed_capacity;
         srv->slots.resize((size_t)slots);
         srv->mark.assign((size_t)s->g->n, 0);
-        for (Slot& sl : srv->slots) {
+        auto make = [&](Slot& sl) -> cudaError_t {
             cudaError_t e = cudaSuccess;
             auto chk = [&](cudaError_t x) { if (e == cudaSuccess) e = x; };
             chk(cudaStreamCreateWithFlags(&sl.stream, cudaStreamNonBlocking));
@@ -153,6 +153,14 @@ extern "C" int skis_server_create(skis_server** out, skis_sketch* s, int32_t slo
             chk(dev_malloc((void**)&sl.d_status, sizeof(DevStatus)));
             if (e == cudaSuccess) e = cudaMemsetAsync(sl.d_smask, 0, (size_t)s->T * sizeof(uint64_t), sl.stream);
             if (e == cudaSuccess) e = cudaStreamSynchronize(sl.stream);
+            return e;
+        };
+        for (Slot& sl : srv->slots) {
+            cudaError_t e = make(sl);
+            if (e == cudaErrorMemoryAllocation && sketch_release_scratch(s, s->stream)) {  // once more, in its room
+                release_slot(sl);
+                e = make(sl);
+            }
             if (e != cudaSuccess) {
                 skis_server_free(srv);
                 return serve_fail(e == cudaErrorMemoryAllocation ? SKIS_ENOMEM : SKIS_ERR_CUDA,

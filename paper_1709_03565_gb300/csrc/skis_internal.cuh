@@ -207,6 +207,8 @@ inline int div_up(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 // Stream-ordered allocation helpers (cudaMallocAsync / cudaFreeAsync).
 cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t st);
 void dev_free(void* p, cudaStream_t st);
+// What the pool keeps of freed memory goes back to the device, where any allocation finds it.
+void dev_trim(cudaStream_t st);
 // Synchronous allocation (cudaMalloc), for long-lived buffers.
 cudaError_t dev_malloc(void** p, size_t bytes);
 // Process-wide count of device allocations made through dev_alloc / dev_malloc.
@@ -406,6 +408,19 @@ cudaError_t coverage_by_index(const skis_sketch* s, const int64_t* off, const in
                               int32_t qn, int64_t seed_base, int64_t nseeds, uint64_t* queue, uint64_t queue_cap,
                               uint64_t* smask, unsigned long long* cov, cudaStream_t st);
 void sketch_release(skis_sketch* s);
+// Gives the sampler's scratch back (the next sampling call takes it again);
+// false when there was none.
+bool sketch_release_scratch(skis_sketch* s, cudaStream_t st);
+// f once more, without the sampler's scratch, where the device had no room for f's buffers.
+template <class F>
+int with_room(skis_sketch* s, cudaStream_t st, std::string* err, F&& f) {
+    int rc = f();
+    if (rc == SKIS_ENOMEM && sketch_release_scratch(s, st)) {
+        err->clear();
+        rc = f();
+    }
+    return rc;
+}
 int sketch_autotune(skis_sketch* s, uint64_t pilot, cudaStream_t st, double* cand_ms, int cand_cap, int* ncand,
                     std::string* err);
 // The coin generator's throughput on this GPU (the ALU ceiling probe).

@@ -146,6 +146,7 @@ cudaError_t cudaDeviceGetDefaultMemPool(cudaMemPool_t* p, int) {
     return cudaSuccess;
 }
 cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void*) { return cudaSuccess; }
+cudaError_t cudaMemPoolTrimTo(cudaMemPool_t, size_t) { return cudaSuccess; }
 cudaError_t cudaGetDevice(int* d) {
     *d = 0;
     return cudaSuccess;
