@@ -163,9 +163,9 @@ typedef enum skis_option {
     SKIS_OPT_CTA_QUEUE_CAP = 13,   /* member queue entries of a CTA-tier slot (default 2^20, at most n;
                                       in [32, 2^31]): a sample with more members moves to a second
                                       pass over fewer slots with n-entry queues */
-    SKIS_OPT_CTA_THREADS = 14      /* size of the CTA tier's blocks, a sample a block: 256 (default: 128 threads,
-                                      eight blocks per SM; 256 or 512 for a small pass of which a good part
-                                      reaches the tier) or 512 (always 512 threads, two per SM) */
+    SKIS_OPT_CTA_THREADS = 14      /* threads of the CTA tier's blocks, a sample a block: 256 (four per SM) or
+                                      512 (two per SM). Without this option 128, eight per SM, or 256 or 512 for
+                                      a small pass of which a good part reaches the tier */
 } skis_option;
 
 /* Load G = (V, E, w) (Sec. II-A) and build the device structures every later

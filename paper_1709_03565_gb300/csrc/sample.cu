@@ -949,7 +949,8 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_iis_warp(SampleArgs a) {
 
 // -------------------------------------------------------------- CTA tier
 // One block of kCtaThreads threads per sample, 1024 threads of such blocks per
-// SM: eight blocks of 128 by default, or two of 512 (SKIS_OPT_CTA_THREADS).
+// SM: eight blocks of 128 by default, or four of 256 or two of 512 where
+// SKIS_OPT_CTA_THREADS asks for them.
 // Four warps a sample pay a level's fixed cost half as often as eight, and
 // twice as many samples hide one another's latencies. R-MAT 2^22 / 2^27 WC,
 // 200K samples: 47.2 ms with blocks of 256, 44.7 with 128, 48.0 with 64;
@@ -1757,7 +1758,7 @@ static cudaError_t grow_copy(T** p, uint64_t old_n, uint64_t new_n, cudaStream_t
 }
 
 // threads of the CTA-tier blocks that the slots are counted for (launch_cta)
-static int cta_block(const skis_sketch* s) { return s->cta_threads == 512 ? 512 : kCtaBlock; }
+static int cta_block(const skis_sketch* s) { return s->cta_threads ? s->cta_threads : kCtaBlock; }
 
 // Arena entries a sketch's first `count` samples get: room for samples of 128
 // members within 2 GiB, at least 8 a sample. Sizes run from 4 members a sample
@@ -1919,8 +1920,11 @@ static void launch_cta_blocks(const SampleArgs& a, int slots, uint64_t above, ui
 static void launch_cta(const skis_sketch* s, const SampleArgs& a, int slots, uint64_t pass, cudaStream_t st) {
     const uint64_t share = pass / kCtaHubShare;
     const uint64_t few = kCtaFew * (uint64_t)sm_count(), many = kCtaMany * (uint64_t)sm_count();
-    if (cta_block(s) == 512) {
+    if (s->cta_threads == 512) {
         k_iis_cta<512><<<slots, 512, 0, st>>>(a, 0, ~0ull, true);
+        note_launch();
+    } else if (s->cta_threads == 256) {
+        k_iis_cta<256><<<slots, 256, 0, st>>>(a, 0, ~0ull, true);
         note_launch();
     } else if (share >= many) {
         launch_cta_blocks<kCtaBlock>(a, slots, 0, ~0ull, true, st);
