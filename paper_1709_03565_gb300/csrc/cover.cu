@@ -12,7 +12,10 @@
 // Delta_v W + T (2^f - w_v) (ties to the lowest id), and the samples of the
 // chosen vertex are marked covered and their members' Delta decremented.
 #include <algorithm>
+#include <cstddef>
 #include <cstring>
+#include <memory>
+#include <new>
 #include <string>
 
 #include "../../include/skis.h"
@@ -1533,7 +1536,7 @@ int sketch_inverted(skis_sketch* s, cudaStream_t st, std::string* err) {
     return with_room(s, st, err, [&] { return build_inverted(s, st, err); });
 }
 
-constexpr int32_t kGreedyPacked = 4096;  // largest k whose results come back in one copy through the stack
+constexpr int32_t kGreedyPacked = 4096;  // largest k whose results come back in one copy
 
 int sketch_greedy(skis_sketch* s, int32_t k, int32_t* h_seeds, int64_t* h_cov, double* h_est, cudaStream_t st,
                   std::string* err) {
@@ -1579,7 +1582,13 @@ int sketch_greedy(skis_sketch* s, int32_t k, int32_t* h_seeds, int64_t* h_cov, d
         const size_t at_partial = take((size_t)gblocks * sizeof(Cand)), at_seg = take((size_t)nseg * sizeof(Cand));
         const size_t at_pool = take(kGreedyThreads * sizeof(uint32_t)), at_delta = take((size_t)n * sizeof(uint32_t));
         const bool packed = k <= kGreedyPacked;  // else straight to the caller's arrays
-        alignas(128) char h_out[sizeof(GreedyCtl) + kGreedyPacked * 20 + 3 * 128];
+        const size_t out_bytes = packed ? copied : sizeof(GreedyCtl);
+        // on the heap: the caller's thread may have little stack
+        const std::unique_ptr<char[]> h_out(new (std::nothrow) char[out_bytes]);
+        if (!h_out) {
+            *err = "skis_greedy_maxcover: host allocation failed";
+            return SKIS_ENOMEM;
+        }
         const int room = with_room(s, st, err, [&]() -> int {
             CV_CUDA(dev_alloc_t(&buf, bytes, st));
             return SKIS_OK;
@@ -1619,21 +1628,23 @@ int sketch_greedy(skis_sketch* s, int32_t k, int32_t* h_seeds, int64_t* h_cov, d
         void* kargs[] = {&ga};
         CV_CUDA(cudaLaunchCooperativeKernel((const void*)k_greedy_rounds, gblocks, kGreedyThreads, kargs, 0, st));
         note_launch();
-        CV_CUDA(cudaMemcpyAsync(h_out, buf + at_ctl, packed ? copied : sizeof(GreedyCtl), cudaMemcpyDeviceToHost, st));
+        CV_CUDA(cudaMemcpyAsync(h_out.get(), buf + at_ctl, out_bytes, cudaMemcpyDeviceToHost, st));
         if (!packed) {
             CV_CUDA(cudaMemcpyAsync(h_seeds, ga.seeds, (size_t)k * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
             if (h_cov) CV_CUDA(cudaMemcpyAsync(h_cov, ga.cov_out, (size_t)k * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
             if (h_est) CV_CUDA(cudaMemcpyAsync(h_est, ga.est_out, (size_t)k * sizeof(double), cudaMemcpyDeviceToHost, st));
         }
         CV_CUDA(cudaStreamSynchronize(st));
-        if (reinterpret_cast<const GreedyCtl*>(h_out)->gave_up) {
+        unsigned int gave_up = 0;
+        std::memcpy(&gave_up, h_out.get() + offsetof(GreedyCtl, gave_up), sizeof(gave_up));
+        if (gave_up) {
             *err = "skis_greedy_maxcover: internal error: a grid barrier ran out";
             return SKIS_ERR_INTERNAL;
         }
         if (packed) {
-            std::memcpy(h_seeds, h_out + (at_seeds - at_ctl), (size_t)k * sizeof(int32_t));
-            if (h_cov) std::memcpy(h_cov, h_out + (at_cov - at_ctl), (size_t)k * sizeof(int64_t));
-            if (h_est) std::memcpy(h_est, h_out + (at_est - at_ctl), (size_t)k * sizeof(double));
+            std::memcpy(h_seeds, h_out.get() + (at_seeds - at_ctl), (size_t)k * sizeof(int32_t));
+            if (h_cov) std::memcpy(h_cov, h_out.get() + (at_cov - at_ctl), (size_t)k * sizeof(int64_t));
+            if (h_est) std::memcpy(h_est, h_out.get() + (at_est - at_ctl), (size_t)k * sizeof(double));
         }
         return SKIS_OK;
     };
