@@ -345,6 +345,7 @@ struct RowBatch {
         total = __shfl_sync(kFull, incl, 31);
         excl = incl - nq;
         const unsigned m = __ballot_sync(kFull, nq > 0);
+        __syncwarp();  // the last batch's rows are read (shuffles and votes order no memory)
         if (nq) row[__popc(m & lanemask_lt())] = make_uint4(excl, lo, hi, tau);
         __syncwarp();
     }

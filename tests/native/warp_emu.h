@@ -54,6 +54,7 @@ struct Thread {
     Kind at = kNone;  // waiting there
     Word in = 0, out = 0;
     int arg = 0;
+    unsigned syncs = 0;  // __syncwarp and __syncthreads passed
     std::vector<std::pair<unsigned long long*, unsigned long long>> held;  // deferred ORs
 };
 
@@ -77,6 +78,7 @@ inline Word wait(Kind k, Word in, int arg = 0) {
     t->in = in;
     t->arg = arg;
     swapcontext(&t->ctx, &sched);
+    if (k == kSyncwarp || k == kBlock) ++t->syncs;
     return t->out;
 }
 
