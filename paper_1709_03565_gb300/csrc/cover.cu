@@ -77,14 +77,10 @@ __device__ __forceinline__ void warp_members(uint64_t off, uint32_t len, const i
 // Lanes adding to the same counter in one step (hub vertices recur across
 // samples) are merged: one atomic per distinct address among the calling
 // lanes, carrying the number of lanes.
-__device__ __forceinline__ void add_aggregated(uint32_t* counter, int32_t u, int sign) {
+__device__ __forceinline__ void add_aggregated(uint32_t* counter, int32_t u) {
     const unsigned active = __activemask();
     const unsigned peers = __match_any_sync(active, u);
-    if ((threadIdx.x & 31) == __ffs(peers) - 1) {
-        const uint32_t c = (uint32_t)__popc(peers);
-        if (sign > 0) atomicAdd(&counter[u], c);
-        else atomicSub(&counter[u], c);
-    }
+    if ((threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&counter[u], (uint32_t)__popc(peers));
 }
 
 // Greedy's cover walk: a block-local table merges the decrements of vertices
@@ -882,7 +878,7 @@ __global__ void __launch_bounds__(kCovThreads) k_count_members(const uint64_t* _
         const uint64_t j = gidx * 32 + lane;
         const bool valid = j < T;
         warp_members(valid ? h_off[j] : 0, valid ? h_len[j] : 0u, arena,
-                     [&](int, int32_t u) { add_aggregated(cnt, u, +1); });
+                     [&](int, int32_t u) { add_aggregated(cnt, u); });
     }
 }
 
@@ -914,8 +910,6 @@ struct KeyId {
     u128 key;
     uint32_t id;
     uint32_t valid;
-    uint32_t d;    // Delta of the vertex (carried with the key)
-    uint32_t pad;
 };
 
 __device__ __forceinline__ bool better(const KeyId& a, const KeyId& b) {
@@ -929,8 +923,6 @@ __device__ __forceinline__ KeyId shfl_down_keyid(const KeyId& x, int d) {
     y.key = shfl_down_u128(x.key, d);
     y.id = __shfl_down_sync(kFull, x.id, d);
     y.valid = __shfl_down_sync(kFull, x.valid, d);
-    y.d = __shfl_down_sync(kFull, x.d, d);
-    y.pad = 0;
     return y;
 }
 
@@ -1679,7 +1671,7 @@ __global__ void __launch_bounds__(256) k_shard_argmax(const int64_t* __restrict_
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
         if (inS[v]) continue;
         const u128 dv = (u128)(uint64_t)delta[v];
-        const KeyId c{ris ? dv : dv * W + (u128)T * (one_f - w[v]), (uint32_t)v, 1u, 0u, 0u};
+        const KeyId c{ris ? dv : dv * W + (u128)T * (one_f - w[v]), (uint32_t)v, 1u};
         if (better(c, best)) best = c;
     }
     best = block_best(best, s_part);

@@ -175,22 +175,16 @@ __device__ __forceinline__ uint64_t bucket_pick(const SampleArgs& a, uint64_t j,
 }
 
 // The source record (source, in-row) of sample j, from the prepass when it
-// holds j, else drawn; *pe / *pu receive the prepass's bucket pick (or -1).
-__device__ __forceinline__ uint32_t source_of(const SampleArgs& a, uint64_t j, RowInfo* rv, int64_t* pe,
-                                              int32_t* pu) {
+// holds j, else drawn; *pe receives the prepass's bucket pick (or -1).
+__device__ __forceinline__ uint32_t source_of(const SampleArgs& a, uint64_t j, RowInfo* rv, int64_t* pe) {
     *pe = -1;
-    *pu = -1;
     if (a.up_rec && j - a.up_first < a.up_count) {
         const uint64_t t = j - a.up_first;
         const uint4 r = __ldg(a.up_rec + t);
         rv->deg = r.y;
         rv->off = r.z;
         rv->tau = r.w;
-        if (a.up_pick && a.chain && r.y > 0) {
-            const uint2 p = __ldg(a.up_pick + t);
-            *pe = p.x;
-            *pu = (int32_t)p.y;
-        }
+        if (a.up_pick && a.chain && r.y > 0) *pe = __ldg(&a.up_pick[t].x);
         return r.x;
     }
     const uint32_t v = draw_source(a, j);
@@ -802,8 +796,7 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_iis_warp(SampleArgs a) {
             // Alg. 1: the source, alone in the sample
             RowInfo rv;
             int64_t pe;
-            int32_t pu;
-            const uint32_t v = source_of(a, j, &rv, &pe, &pu);
+            const uint32_t v = source_of(a, j, &rv, &pe);
             WarpInserter ins{hash, s_queue[wib], s_ring[wib], a.spill_hash + (wid << a.spill.hash_bits),
                              a.spill_queue + wid * a.spill.cap, a.rows, a.spill, 1u, 1u, false, false};
             if (lane == 0) {
@@ -1037,8 +1030,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1024 / kCtaThreads) k_iis_cta(Sam
 
         RowInfo rv;
         int64_t pe;
-        int32_t pu;
-        const uint32_t v = source_of(a, j, &rv, &pe, &pu);
+        const uint32_t v = source_of(a, j, &rv, &pe);
         if (threadIdx.x == 0) {
             bitmap[v >> 5] |= 1u << (v & 31);
             queue[0] = (int32_t)v;
