@@ -26,6 +26,14 @@
  *     samples (sketches of 2^20 samples or more) moves their members into
  *     sample-id order in the sketch's storage. Only the layout changes, never a sample; do not overlap such a
  *     call with other work on the same sketch (a server included).
+ *   - Device memory: a sketch keeps the sampler's scratch between calls (up to
+ *     ~12 GB of slots, see SKIS_OPT_CTA_SLOTS, and 0.1-1 GB of tables) and a
+ *     member arena that starts with room for 128 members a sample within
+ *     2 GiB. Where the device has less, a sampling call makes do with smaller
+ *     scratch and 8 members a sample before it returns SKIS_ENOMEM, and a
+ *     query, greedy or server call on the sketch takes the scratch's room.
+ *     After SKIS_ENOMEM or SKIS_ERR_ARENA_FULL the sketch holds the samples it
+ *     had, and calls on it go on.
  *   - Memory spaces: where a call takes SKIS_MEM_HOST or SKIS_MEM_DEVICE,
  *     the pointers it names are host or device pointers accordingly.
  *   - Determinism: sample j of a sketch is a pure function of (graph, seed,
@@ -122,7 +130,8 @@ typedef struct skis_stats {
 typedef enum skis_option {
     SKIS_OPT_RETRY_CAP = 0,      /* cap on rejected first-step rounds (default 2^24) */
     SKIS_OPT_CTA_SLOTS = 1,      /* CTAs of the CTA tier (default: 1024 threads of them per SM,
-                                    within ~12 GB of visited bitmaps and queues) */
+                                    within ~12 GB of visited bitmaps and queues, and fewer where the
+                                    device has no room for them) */
     SKIS_OPT_WARP_BLOCKS = 2,    /* CTAs of the warp tier (default, and at most, full occupancy) */
     SKIS_OPT_THREAD_MAX_DEG = 3, /* longest in-row the thread tier expands (default 192; 0 = tier off) */
     SKIS_OPT_THREAD_BLOCKS = 4,  /* CTAs of the thread tier (default: full occupancy) */

@@ -2,10 +2,13 @@
 // greedy max-coverage (Sec. V-A, Alg. 3, Eq. margin) on the device sketch.
 //
 // Coverage: each query of a batch of up to 64 owns one bit of a per-vertex
-// mask. A warp takes 32 consecutive samples, spreads their members over its
-// lanes, ORs the members' masks per sample in shared memory and counts, per
-// query bit, the samples whose OR has it (ballot + popcount). Counts and the
-// estimator numerator are exact integers.
+// mask. A small sketch is scanned in groups of 1 to 32 consecutive samples
+// (k_coverage): a warp spreads a group's members over its lanes, ORs the
+// members' masks per sample in shared memory and counts, per query bit, the
+// samples whose OR has it (ballot + popcount). A large one is scanned in
+// sample-id order (k_scan_ordered), and one with an inverted index by the
+// seeds' sample lists (k_cover_inv). Counts and the estimator numerator are
+// exact integers.
 //
 // Greedy: an inverted index vertex -> samples (counting sort), marginal
 // coverage Delta_v, then per round an exact argmax of the integer key
@@ -216,7 +219,7 @@ __global__ void __launch_bounds__(kCovThreads) k_coverage(const uint64_t* __rest
 // counts it, and the first setter of a sample's word lists the sample for the
 // reset. Bound by the returning list atomics when each hit took one on the same
 // counter, and by too few tasks where samples are large (1024 samples a task):
-// 10M samples of 4 members and 64 queries of 50 seeds 71 -> 53 us, the whole
+// 10M samples of 4 members and 64 queries of 10 seeds 71 -> 53 us, the whole
 // call 177 -> 168; 1M of 70 members 309 -> 175; 6M of 4 members and 64 queries
 // of 250 seeds 778 -> 470. Now by the chain of load, filter read and branch at
 // one block an SM (the filter's 128 KiB); the members' bytes alone take 25 us.
@@ -1029,7 +1032,8 @@ struct GreedyArgs {
 //     beats that bound it is the argmax (ties to the lowest id), and every
 //     block finds it by itself, with no exchange. When it no longer does, the
 //     pool is refilled from all vertices (a histogram of rounded keys picks
-//     how far down it goes; membership decides nothing but speed).
+//     how far down it goes; a vertex that does not get in bounds it, so that
+//     membership decides nothing but speed).
 //   - Where too many vertices tie for a pool, rounds scan segments of 256
 //     vertices instead: a segment whose best is still outside S with an
 //     unchanged Delta keeps it, the others are rescanned, one warp each.

@@ -41,8 +41,13 @@ constexpr int kIdBatch = 16;       // most sample ids a warp takes per work-curs
 // that are still narrow (a few rows a level) belong here, where 32 of them
 // share an SM, and not on the CTA tier, where at most eight do: on Chung-Lu 1M /
 // 17.5M WC (levels of 13 rows; four blocks an SM then) the two tiers take
-// 10.6 ms with 1536 members and 7.5 ms with 4096. A sample that holds a sixth of the graph has levels wide
-// enough for a block, so a small graph keeps the smaller slot.
+// 10.6 ms with 1536 members and 7.5 ms with 4096. Speed does not set the line
+// for small graphs: 100K samples of ER graphs of average in-degree 10 WC take,
+// with 1536 / 4096 members, .79 / .78 ms at 5k vertices, 1.19 / .95 at 10k, 1.37
+// / 1.03 at 20k and 1.96 / 1.96 at 50k (400K samples: 2.18 / 2.17, 2.77 / 2.48, 3.64 /
+// 2.95, 5.50 / 4.34). The smaller slot keeps the CTA tier in use at the default
+// split on graphs whose samples are compared whole, member by member, with the
+// oracle's (test_er_workload_full_parity asks for samples of all three tiers).
 struct SpillSize {
     uint32_t cap, hash_bits;
 };
