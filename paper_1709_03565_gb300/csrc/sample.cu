@@ -2231,12 +2231,13 @@ int sketch_sample(skis_sketch* s, uint64_t count, cudaStream_t st, std::string* 
     for (;;) {
         const int rc = sample_passes(s, count, st, err);
         if (rc == SKIS_OK || s->T != T0) return rc;
-        // a call that appended nothing: what its passes reserved is free again (and is
-        // not taken for demand when a later call's overflow sizes the arena)
-        if (s->ctr)
-            cudaMemcpyAsync(&s->ctr->arena, &s->arena_used, sizeof(s->arena_used), cudaMemcpyHostToDevice, st);
         const bool again = (rc == SKIS_ENOMEM && s->lean < kLeanMost) || (rc == SKIS_ERR_ARENA_FULL && s->lean == lean0);
         if (again || s->lean != lean0) sketch_release_scratch(s, st);  // its sizes go by lean
+        // a call that appended nothing: what its passes reserved is free again (and is
+        // not taken for demand when a later call's overflow sizes the arena)
+        if (s->T == 0) s->arena_used = 0;
+        if (s->ctr)
+            cudaMemcpyAsync(&s->ctr->arena, &s->arena_used, sizeof(s->arena_used), cudaMemcpyHostToDevice, st);
         if (!again) {
             s->lean = lean0;
             return rc;
