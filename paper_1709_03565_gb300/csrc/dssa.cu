@@ -13,6 +13,7 @@
 // exact integers (coverage, W, T, sum of 2^f - w_v) with correctly rounded
 // conversions, in the order written here, so the decisions are reproducible.
 #include <cmath>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -38,9 +39,9 @@ double exact_estimate(uint64_t cov, uint64_t W, uint64_t T, u128 sum_c, int f) {
 
 }  // namespace
 
-extern "C" int skis_dssa_maxinf(const skis_graph* g, uint64_t seed_r, uint64_t seed_rc, int32_t k, double eps,
-                                double delta, uint64_t lambda2, uint64_t n0, uint64_t n_max, int32_t* seeds_out,
-                                skis_dssa_result* res, void* cuda_stream) {
+static int dssa(const skis_graph* g, uint64_t seed_r, uint64_t seed_rc, int32_t k, double eps, double delta,
+                uint64_t lambda2, uint64_t n0, uint64_t n_max, int32_t* seeds_out, skis_dssa_result* res,
+                void* cuda_stream) {
     if (!g || !seeds_out || !res) return set_last_error(SKIS_EINVAL, "skis_dssa_maxinf: NULL argument");
     if (k < 1 || k > g->n) return set_last_error(SKIS_EINVAL, "skis_dssa_maxinf: k must be in [1, n]");
     if (!(eps > 0.0 && eps < 1.0 - kInvE)) return set_last_error(SKIS_EINVAL, "skis_dssa_maxinf: eps must be in (0, 1 - 1/e)");
@@ -59,6 +60,9 @@ extern "C" int skis_dssa_maxinf(const skis_graph* g, uint64_t seed_r, uint64_t s
         const double l = (2.0 * gamma_n + 2.0 * eps / 3.0) * std::log(2.0 * (double)t_max / delta) / (eps * eps);
         lambda2 = (uint64_t)std::ceil(l);
     }
+    std::vector<int64_t> cov(k);  // these may throw: before anything that would have to be released
+    std::vector<double> est(k);
+    std::vector<uint64_t> wsel(k);
     skis_sketch R, Rc;
     R.g = g;
     R.seed = seed_r;
@@ -68,9 +72,6 @@ extern "C" int skis_dssa_maxinf(const skis_graph* g, uint64_t seed_r, uint64_t s
     Rc.stream = st;
     std::string err;
     int rc = SKIS_OK;
-    std::vector<int64_t> cov(k);
-    std::vector<double> est(k);
-    std::vector<uint64_t> wsel(k);
     int32_t* d_sel = nullptr;
     uint64_t* d_w = nullptr;
     int64_t* d_q = nullptr;
@@ -155,4 +156,14 @@ extern "C" int skis_dssa_maxinf(const skis_graph* g, uint64_t seed_r, uint64_t s
     if (rc != SKIS_OK) return set_last_error(rc, "skis_dssa_maxinf: " + err);
     *res = out;
     return SKIS_OK;
+}
+
+extern "C" int skis_dssa_maxinf(const skis_graph* g, uint64_t seed_r, uint64_t seed_rc, int32_t k, double eps,
+                                double delta, uint64_t lambda2, uint64_t n0, uint64_t n_max, int32_t* seeds_out,
+                                skis_dssa_result* res, void* cuda_stream) {
+    try {
+        return dssa(g, seed_r, seed_rc, k, eps, delta, lambda2, n0, n_max, seeds_out, res, cuda_stream);
+    } catch (const std::bad_alloc&) {
+        return set_last_error(SKIS_ENOMEM, "skis_dssa_maxinf: host allocation failed");
+    }
 }
