@@ -27,6 +27,7 @@
 namespace skis {
 
 constexpr int kCovThreads = 256;
+constexpr int kCovBlocks = 8;  // an SM: every warp slot
 constexpr int kFillRuns = 4;  // k_fill_inverted
 
 // Calls f(owner_lane, member) for every member of the samples held by the
@@ -151,8 +152,10 @@ __global__ void k_qmask_set(const int64_t* __restrict__ off, const int32_t* __re
 // a small sketch left most warp slots empty (ER 10k / 100k, 100K samples, 60
 // members on average and up to 1,700: 3,125 groups for 9,728 slots, 76 us), so
 // a group is only as large as keeps every slot supplied (coverage_shape), and
-// four runs of 32 members are in flight.
-__global__ void __launch_bounds__(kCovThreads) k_coverage(const uint64_t* __restrict__ h_off,
+// four runs of 32 members are in flight. Without the bound on its registers the
+// compiler takes 40, a quarter of the warp slots (64 queries of 679K samples of
+// 70 members 182 us, 155 with 32).
+__global__ void __launch_bounds__(kCovThreads, kCovBlocks) k_coverage(const uint64_t* __restrict__ h_off,
                                                           const uint32_t* __restrict__ h_len, uint64_t T,
                                                           const int32_t* __restrict__ arena,
                                                           const uint64_t* __restrict__ qmask,
@@ -166,14 +169,14 @@ __global__ void __launch_bounds__(kCovThreads) k_coverage(const uint64_t* __rest
     unsigned long long c_lo = 0, c_hi = 0;  // counts of queries `lane` and `lane + 32`
     const uint64_t nwarps = (uint64_t)gridDim.x * (kCovThreads / 32);
     const uint64_t groups = (T + (1u << glog) - 1) >> glog;
-    unsigned long long* acc_row = s_acc[wib];
+    unsigned long long* acc_row = s_acc[wib];  // zero between groups
+    acc_row[lane] = 0;
+    __syncwarp();
     for (uint64_t gidx = (uint64_t)blockIdx.x * (kCovThreads / 32) + wib; gidx < groups; gidx += nwarps) {
         const uint64_t j = (gidx << glog) + lane;
         const bool valid = lane < (1 << glog) && j < T;
         const uint64_t off = valid ? h_off[j] : 0;
         const uint32_t len = valid ? h_len[j] : 0;
-        acc_row[lane] = 0;
-        __syncwarp();
         bool hit = false;
         warp_members<4>(off, len, arena, [&](int owner, int32_t u) {
             if (qbits) {  // not a seed
@@ -189,9 +192,10 @@ __global__ void __launch_bounds__(kCovThreads) k_coverage(const uint64_t* __rest
         if (!__any_sync(kFull, hit)) continue;
         __syncwarp();  // every lane has the others' ORs (a vote orders no memory)
         const uint64_t acc = acc_row[lane];
-        uint64_t present = acc;
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) present |= __shfl_xor_sync(kFull, present, d);
+        acc_row[lane] = 0;
+        __syncwarp();
+        uint64_t present = (uint64_t)__reduce_or_sync(kFull, (uint32_t)(acc >> 32)) << 32 |
+                           __reduce_or_sync(kFull, (uint32_t)acc);
         while (present) {
             const int b = __ffsll((long long)present) - 1;
             present &= present - 1;
@@ -480,12 +484,12 @@ static int coverage_blocks(uint64_t T) {
 // k_coverage's grid and group size: the largest groups (at most 32 samples)
 // that still give two to each of the GPU's warps.
 void coverage_shape(uint64_t T, int* blocks, int* glog) {
-    const uint64_t warps = (uint64_t)sm_count() * 8 * (kCovThreads / 32);
+    const uint64_t warps = (uint64_t)sm_count() * kCovBlocks * (kCovThreads / 32);
     *glog = 5;
     while (*glog > 0 && (T >> *glog) < 2 * warps) --*glog;
     const uint64_t groups = (T + (1u << *glog) - 1) >> *glog;
     const uint64_t want = (groups + kCovThreads / 32 - 1) / (kCovThreads / 32);
-    *blocks = (int)std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)sm_count() * 8));
+    *blocks = (int)std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)sm_count() * kCovBlocks));
 }
 
 // ------------------------------------------- coverage by inverted index

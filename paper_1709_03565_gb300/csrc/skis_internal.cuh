@@ -434,7 +434,7 @@ int set_last_error(int code, const std::string& msg);
 __global__ void k_qmask_set(const int64_t* __restrict__ off, const int32_t* __restrict__ seeds, int32_t q0,
                             int32_t qn, int64_t n, uint64_t* __restrict__ qmask, uint32_t* __restrict__ qbits,
                             DevStatus* st, unsigned long long* __restrict__ reset3);
-__global__ void __launch_bounds__(256) k_coverage(const uint64_t* __restrict__ h_off, const uint32_t* __restrict__ h_len, uint64_t T,
+__global__ void __launch_bounds__(256, 8) k_coverage(const uint64_t* __restrict__ h_off, const uint32_t* __restrict__ h_len, uint64_t T,
                            const int32_t* __restrict__ arena, const uint64_t* __restrict__ qmask,
                            const uint32_t* __restrict__ qbits, int hashed, int glog,
                            unsigned long long* __restrict__ cov);

@@ -39,7 +39,7 @@ int main(int argc, char** argv) {
 
 @pytest.mark.parametrize("glog", [0, 3, 5])
 def test_coverage_reads_a_sample_s_queries_after_every_lane_has_added_its_own(tmp_path, glog):
-    exe = warp_emu.build(tmp_path, "cover.cu", ["kCovThreads", "warp_members", "kFilterLog2", "filter_index",
+    exe = warp_emu.build(tmp_path, "cover.cu", ["kCovThreads", "kCovBlocks", "warp_members", "kFilterLog2", "filter_index",
                                                 "k_coverage"], COVER)
     for seed in range(8):
         assert subprocess.run([exe, str(seed), str(glog)], timeout=120).returncode == 0
